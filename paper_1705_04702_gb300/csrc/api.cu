@@ -511,6 +511,9 @@ extern "C" int skirt_trace(skirt_grid_t g, const skirt_source* src, const skirt_
         A.src_df[a] = make_float2(hi, (float)(src->pos[a] - (double)hi));
         A.src_dir_f[a] = (float)src->dir[a];
         A.hi_f[a] = (float)g->bbox[2 * a + 1];
+        A.lo_f[a] = (float)A.lo[a];
+        A.d_f[a] = (float)A.d[a];
+        A.id_f[a] = 1.f / A.d_f[a];
     }
     A.offsets = (const unsigned long long*)(dp + L.offsets);
     A.pk_first = (const unsigned long long*)(dp + L.first);
@@ -543,6 +546,7 @@ extern "C" int skirt_trace(skirt_grid_t g, const skirt_source* src, const skirt_
     A.absorbed = d_acc;
     A.abs_cs = lmajor ? 1 : NL;
     A.abs_ls = lmajor ? g->ncell : 1;
+    A.abs_cs8 = (unsigned)(A.abs_cs * sizeof(double));
     A.images = d_img;
     A.oof = (double*)(dp + L.oof);
     A.ledger = (double*)(dp + L.ledger);

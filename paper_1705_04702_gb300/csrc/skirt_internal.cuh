@@ -33,7 +33,11 @@ __device__ __forceinline__ uint4 philox10(uint4 c, uint32_t k0, uint32_t k1)
 
 // Uniform deviate in (0, 1): (top 23 bits + 1/2) * 2^-23.  Exactly
 // representable in FP32, so both precisions see identical values.
-__device__ __forceinline__ float u01f(uint32_t x) { return ((float)(x >> 9) + 0.5f) * 1.1920928955078125e-7f; }
+// The 23 bits become a float through the 2^23 offset (exact), not by a conversion.
+__device__ __forceinline__ float u01f(uint32_t x)
+{
+    return ((__uint_as_float(0x4B000000u | (x >> 9)) - 8388608.f) + 0.5f) * 1.1920928955078125e-7f;
+}
 
 // Per-instrument constants (host-computed in FP64, FP32 copies for the mixed form).
 struct InstrDev {
@@ -81,7 +85,7 @@ struct TraceArgs {
     const float2* faces;                   // face planes as (hi, lo) FP32 pairs: x [nx+1], y [ny+1], z [nz+1]
     float2 src_df[3];                      // source position as (hi, lo) FP32 pairs
     float src_dir_f[3];
-    float hi_f[3];
+    float lo_f[3], d_f[3], id_f[3], hi_f[3];  // lower corner, cell size, its reciprocal, upper corner in FP32
     float w_min_f;
     const unsigned long long* offsets;     // [nlambda + 1] prefix sums of packet counts
     const unsigned long long* pk_first;    // [nlambda] stream index of each wavelength's first packet
@@ -93,6 +97,7 @@ struct TraceArgs {
     const InstrDev* ins;
     double* absorbed;                      // element (cell, lambda) at cell * abs_cs + lambda * abs_ls
     long long abs_cs, abs_ls;              // [cell][lambda]: (nlambda, 1); [lambda][cell]: (1, ncell)
+    unsigned abs_cs8;                      // abs_cs in bytes
     double* images;                        // per instrument [npx*npx][nlambda]
     double* oof;                           // [ninstr][nlambda] peel-offs outside the frame
     double* ledger;                        // [nlambda][4]

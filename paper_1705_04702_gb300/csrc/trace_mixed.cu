@@ -33,8 +33,22 @@
 //  * Per event, escaped / absorbed / scattered come from one
 //    om = 1 - e^{-tau_path}, so they add up to the packet luminosity.
 //  * Per-thread state used only at events lives in shared memory.
+//
+// What bounds it is instruction issue (72% of the cycles on the 256^3 disk),
+// so the crossing is written for few warp instructions: the exit axis's next
+// face is advanced under predicates from FP32 face indices, leaving the grid
+// is tested by one distance comparison, and the cell index moves by a signed
+// stride.  The lanes handle events in one pass over the stages with a single
+// copy of the traversal set-up and one random block per scattering, which
+// also keeps the loop inside the instruction cache.  Against selecting every
+// operand by axis and setting traversals up inside each stage: 1e7 packets on
+// the 256^3 disk 185.8 ms (250.4), 8e6 packets of 200 wavelengths on the 128^3
+// torus 135.9 ms (192.7), 3e6 packets on an octree of 8.3e5 leaves 63.6 ms
+// (94.6), the same histories bit for bit.
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <type_traits>
 
 #include "skirt_internal.cuh"
 #include "trace_device.cuh"
@@ -120,6 +134,20 @@ __device__ __forceinline__ float df_diff(float2 f, float xh, float xl)
     return __fadd_rn(__fsub_rn(f.x, xh), __fsub_rn(f.y, xl));
 }
 
+// Integer <-> FP32 for 0 <= i < 2^23 by the 2^23 offset: one logical and one
+// FP32 instruction, where a conversion instruction would occupy a slow pipe
+// (measured on the octree kernel, whose crossings held three float-to-int
+// conversions: FP64/conversion pipe 64% active).
+__device__ __forceinline__ float i2f_small(int i) { return __int_as_float(0x4B000000 | i) - 8388608.f; }
+// floor(f) for 0 <= f < 2^23
+__device__ __forceinline__ int floor_small(float f) { return __float_as_int(__fadd_rd(f, 8388608.f)) & 0x7FFFFF; }
+
+// Distance along the ray to face plane k (FP32 index) of one axis.
+__device__ __forceinline__ float face_t(float k, float d, float lo, float x, float iv)
+{
+    return __fmul_rn(__fsub_rn(__fmaf_rn(k, d, lo), x), iv);
+}
+
 // Per-thread state used only at events, struct of arrays in shared memory.
 struct Cold {
     double l_emit[MAXB], l_abs[MAXB], l_esc[MAXB], l_res[MAXB];
@@ -127,18 +155,25 @@ struct Cold {
     unsigned long long c_dep[MAXB], c_loc[MAXB], c_peel[MAXB], c_scat[MAXB];
     float L0[MAXB], p_esc[MAXB], p_abs[MAXB], p_res[MAXB], p_peel[MAXB], om[MAXB], peel_w[MAXB], alb[MAXB];
     float xl0[MAXB], xl1[MAXB], xl2[MAXB];  // low words of the double-float position
-    int lam[MAXB], led_lam[MAXB], nscat[MAXB], peel_i[MAXB], after_peel[MAXB], peel_kind[MAXB];
+    int lam[MAXB], led_lam[MAXB], nscat[MAXB], peel_i[MAXB], peel_kind[MAXB];
     unsigned pk[MAXB], ev[MAXB], started[MAXB];
+    unsigned ry[MAXB], rz[MAXB];            // the event's second and third random words
 };
 
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-// OCT: octree grid (Sect. 7.9).  The traversal state then names a leaf
-// (node, level, lattice corner) instead of a cell; a crossing reads the face
-// neighbour and descends from it by the lattice cell of the entry point.
-template <bool OCT>
+// Grid kinds.  G_CART: Cartesian, face indices held as FP32 integers (every
+// dimension below 2^23, so that they stay exact); G_CART_BIG: Cartesian with a
+// longer axis, face indices as integers; G_OCT: octree (Sect. 7.9), where the
+// traversal state names a leaf (node, level, lattice corner) instead of a cell
+// and a crossing reads the face neighbour and descends from it by the lattice
+// cell of the entry point.
+enum { G_CART = 0, G_CART_BIG = 1, G_OCT = 2 };
+
+template <int G>
 __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
 {
+    constexpr bool OCT = G == G_OCT, BIG = G == G_CART_BIG;
     extern __shared__ __align__(16) unsigned char smem[];
     InstrDev* sins = reinterpret_cast<InstrDev*>(smem);
     Cold& C = *reinterpret_cast<Cold*>(smem + align16(sizeof(InstrDev) * A.ninstr));
@@ -152,38 +187,34 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     C.started[t] = 0;
     __syncthreads();
 
-    const int NL = A.nlambda;
-    const int nx = A.nx, ny = A.ny, nz = A.nz;
-    const float lo0 = (float)A.lo[0], lo1 = (float)A.lo[1], lo2 = (float)A.lo[2];
-    const float d0 = (float)A.d[0], d1 = (float)A.d[1], d2 = (float)A.d[2];
     const float INF = __int_as_float(0x7f800000);
     const float* __restrict__ kr = A.kr32;
-    const float2* __restrict__ fx = A.faces;
-    const float2* __restrict__ fy = A.faces + (nx + 1);
-    const float2* __restrict__ fz = A.faces + (nx + 1) + (ny + 1);
-    double* __restrict__ absorbed = A.absorbed;
-    const int step_min = A.step_min > 0 ? A.step_min : 20;
-    const float tau_cut = A.tau_cut;  // optical depth after which a deposit / peel-off traversal stops
+    const int step_min = A.step_min;
 
     // ---- stepping state (registers)
     int mode = M_NONE;
+    // Cartesian: per axis the index of the next face (kf), its step (sf: +1, -1
+    // or 0) and the cell-index stride of a crossing (st); octree: the leaf's
+    // lattice corner (c) and the step
+    using KF = typename std::conditional<BIG, int, float>::type;
+    KF kf0 = 0, kf1 = 0, kf2 = 0, sf0 = 0, sf1 = 0, sf2 = 0;
+    int st0 = 0, st1 = 0, st2 = 0;
     int c0 = 0, c1 = 0, c2 = 0, s0 = 0, s1 = 0, s2 = 0;
     float iv0 = 0.f, iv1 = 0.f, iv2 = 0.f, tn0 = 0.f, tn1 = 0.f, tn2 = 0.f, tcur = 0.f;
+    float t_end = 0.f;               // Cartesian: no crossing before this distance leaves the grid
     float tau_h = 0.f, tau_l = 0.f;  // running optical depth of the traversal (double-float)
-    float rem_f = 0.f;               // interaction optical depth (search)
+    float par = 0.f;                 // deposit: L (1 - albedo); search: interaction optical depth
     unsigned nsteps = 0;
-    float labs_f = 0.f;
     float s_found = 0.f, last_dusty_end = 0.f;
     bool found = false;
-    int last_axis = -1;  // axis of the face through which the current cell was entered
+    int last_axis = -1;  // search: axis of the face through which the current cell was entered
     int cur_m = 0;       // index of the current cell
     float kr_cur = 0.f;  // its extinction coefficient (loaded one crossing ahead)
-    const int nxy = nx * ny;
-    // octree: the current leaf's node and level (c0..c2: its lattice corner),
-    // the traversal direction, the node of the interaction leaf
+    double* dep_base = nullptr;  // the absorbed table at (cell 0, the packet's wavelength)
+    // octree: the current leaf's node and level, the traversal direction, the
+    // node of the interaction leaf
     const int OL = A.oct_levels;
     const OctNode* __restrict__ nodes = A.oct_nodes;
-    const float id0 = 1.f / d0, id1 = 1.f / d1, id2 = 1.f / d2;
     int onode = 0, olev = 0, pc_node = 0;
     float v0 = 0.f, v1 = 0.f, v2 = 0.f;
     // ---- packet state (registers)
@@ -223,40 +254,67 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         c2 = j2 & mask;
     };
 
+    // starts a traversal of kind m along (vx, vy, vz) from the packet's position
     auto begin = [&](int m, float vx, float vy, float vz) {
         mode = m;
+        const float2* __restrict__ fx = A.faces;
+        const float2* __restrict__ fy = fx + (A.nx + 1);
+        const float2* __restrict__ fz = fy + (A.ny + 1);
         const float l0 = C.xl0[t], l1 = C.xl1[t], l2 = C.xl2[t];
-        if (have_pc) {
-            c0 = pc0; c1 = pc1; c2 = pc2;
-        } else {
-            c0 = axis_cell(x0, l0, lo0, d0, nx, fx);
-            c1 = axis_cell(x1, l1, lo1, d1, ny, fy);
-            c2 = axis_cell(x2, l2, lo2, d2, nz, fz);
+        int b0 = pc0, b1 = pc1, b2 = pc2;
+        if (!have_pc) {
+            b0 = axis_cell(x0, l0, A.lo_f[0], A.d_f[0], A.nx, fx);
+            b1 = axis_cell(x1, l1, A.lo_f[1], A.d_f[1], A.ny, fy);
+            b2 = axis_cell(x2, l2, A.lo_f[2], A.d_f[2], A.nz, fz);
         }
         if constexpr (OCT) {
-            if (have_pc) oct_enter(pc_node, 0, c0, c1, c2);
-            else oct_enter(0, 0, c0, c1, c2);
+            oct_enter(have_pc ? pc_node : 0, 0, b0, b1, b2);
+            b0 = c0; b1 = c1; b2 = c2;
             v0 = vx; v1 = vy; v2 = vz;
         }
-        s0 = vx > 0.f ? 1 : (vx < 0.f ? -1 : 0);
-        s1 = vy > 0.f ? 1 : (vy < 0.f ? -1 : 0);
-        s2 = vz > 0.f ? 1 : (vz < 0.f ? -1 : 0);
-        iv0 = s0 ? 1.f / vx : 0.f;
-        iv1 = s1 ? 1.f / vy : 0.f;
-        iv2 = s2 ? 1.f / vz : 0.f;
+        const int g0 = vx > 0.f ? 1 : (vx < 0.f ? -1 : 0);
+        const int g1 = vy > 0.f ? 1 : (vy < 0.f ? -1 : 0);
+        const int g2 = vz > 0.f ? 1 : (vz < 0.f ? -1 : 0);
+        iv0 = g0 ? 1.f / vx : 0.f;
+        iv1 = g1 ? 1.f / vy : 0.f;
+        iv2 = g2 ? 1.f / vz : 0.f;
         // first faces from the exact face planes and the double-float position
         const int e = OCT ? 1 << (OL - olev) : 1;  // the cell's extent in lattice cells
-        tn0 = s0 ? df_diff(__ldg(fx + c0 + (s0 > 0 ? e : 0)), x0, l0) * iv0 : INF;
-        tn1 = s1 ? df_diff(__ldg(fy + c1 + (s1 > 0 ? e : 0)), x1, l1) * iv1 : INF;
-        tn2 = s2 ? df_diff(__ldg(fz + c2 + (s2 > 0 ? e : 0)), x2, l2) * iv2 : INF;
+        const int n0 = b0 + (g0 > 0 ? e : 0), n1 = b1 + (g1 > 0 ? e : 0), n2 = b2 + (g2 > 0 ? e : 0);
+        tn0 = g0 ? df_diff(__ldg(fx + n0), x0, l0) * iv0 : INF;
+        tn1 = g1 ? df_diff(__ldg(fy + n1), x1, l1) * iv1 : INF;
+        tn2 = g2 ? df_diff(__ldg(fz + n2), x2, l2) * iv2 : INF;
         tcur = 0.f;
         tau_h = tau_l = 0.f;
         nsteps = 0;
         last_axis = -1;
-        if constexpr (!OCT) {
-            cur_m = (c2 * ny + c1) * nx + c0;
+        if constexpr (OCT) {
+            s0 = g0; s1 = g1; s2 = g2;
+        } else {
+            kf0 = (KF)n0; kf1 = (KF)n1; kf2 = (KF)n2;
+            sf0 = (KF)g0; sf1 = (KF)g1; sf2 = (KF)g2;
+            st0 = g0;
+            st1 = g1 * A.nx;
+            st2 = g2 * (A.nx * A.ny);
+            // the distance to each axis's last face by the crossing's own
+            // formula: the crossing that leaves the grid lies at one of them
+            const int m0 = g0 > 0 ? A.nx : 0, m1 = g1 > 0 ? A.ny : 0, m2 = g2 > 0 ? A.nz : 0;
+            const float u0 = n0 == m0 ? tn0 : face_t((float)m0, A.d_f[0], A.lo_f[0], x0, iv0);
+            const float u1 = n1 == m1 ? tn1 : face_t((float)m1, A.d_f[1], A.lo_f[1], x1, iv1);
+            const float u2 = n2 == m2 ? tn2 : face_t((float)m2, A.d_f[2], A.lo_f[2], x2, iv2);
+            t_end = fminf(g0 ? u0 : INF, fminf(g1 ? u1 : INF, g2 ? u2 : INF));
+            cur_m = (b2 * A.ny + b1) * A.nx + b0;
             kr_cur = __ldg(kr + cur_m);
         }
+    };
+
+    // deposit of one crossing
+    auto deposit = [&](int m, float tau_prev, float dtau) {
+        const float dep = par * exp_neg(tau_prev) * one_minus_exp_neg(dtau);
+        if (dep >= 1.17549435e-38f)
+            atomicAdd(reinterpret_cast<double*>(reinterpret_cast<char*>(dep_base) +
+                                                (size_t)(unsigned)m * A.abs_cs8),
+                      f2d_pos(dep));
     };
 
     // one leaf crossing of an octree traversal: the face neighbour and its
@@ -281,8 +339,8 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         const float tau_prev = tau_h + tau_l;
         if (mode == M_LOCATE) {
             if (krl > 0.f) {
-                if (tau_h + (tau_l + dtau) >= rem_f) {
-                    s_found = (rem_f - tau_prev) / krl;
+                if (tau_h + (tau_l + dtau) >= par) {
+                    s_found = (par - tau_prev) / krl;
                     found = true;
                     done = true;
                 } else {
@@ -290,9 +348,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                 }
             }
         } else if (mode == M_DEPOSIT && dtau > 0.f) {
-            const float dep = labs_f * exp_neg(tau_prev) * one_minus_exp_neg(dtau);
-            if (dep >= 1.17549435e-38f)
-                atomicAdd(absorbed + ((size_t)m * A.abs_cs + (size_t)lam * A.abs_ls), f2d_pos(dep));
+            deposit(m, tau_prev, dtau);
         }
         df_accumulate(tau_h, tau_l, dtau);
         if (!done) {
@@ -307,12 +363,14 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                 // `axis`, elsewhere the crossing point's cell kept within the
                 // current leaf's cross-section
                 const int e = 1 << (OL - olev);
-                const float p0 = floorf((x0 + tmin * v0 - lo0) * id0);
-                const float p1 = floorf((x1 + tmin * v1 - lo1) * id1);
-                const float p2 = floorf((x2 + tmin * v2 - lo2) * id2);
-                int j0 = (int)fminf(fmaxf(p0, (float)c0), (float)(c0 + e - 1));
-                int j1 = (int)fminf(fmaxf(p1, (float)c1), (float)(c1 + e - 1));
-                int j2 = (int)fminf(fmaxf(p2, (float)c2), (float)(c2 + e - 1));
+                const float em = __int_as_float((127 + OL - olev) << 23) - 1.f;  // e - 1
+                const float f0 = i2f_small(c0), f1 = i2f_small(c1), f2 = i2f_small(c2);
+                const float p0 = (x0 + tmin * v0 - A.lo_f[0]) * A.id_f[0];
+                const float p1 = (x1 + tmin * v1 - A.lo_f[1]) * A.id_f[1];
+                const float p2 = (x2 + tmin * v2 - A.lo_f[2]) * A.id_f[2];
+                int j0 = floor_small(fminf(fmaxf(p0, f0), f0 + em));
+                int j1 = floor_small(fminf(fmaxf(p1, f1), f1 + em));
+                int j2 = floor_small(fminf(fmaxf(p2, f2), f2 + em));
                 const int ja = ss > 0 ? (axis == 0 ? c0 : (axis == 1 ? c1 : c2)) + e
                                       : (axis == 0 ? c0 : (axis == 1 ? c1 : c2)) - 1;
                 j0 = axis == 0 ? ja : j0;
@@ -332,80 +390,91 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                     oct_enter(nb, olev, j0, j1, j2);
                 }
                 const int en = 1 << (OL - olev);
-                tn0 = s0 ? (lo0 + (float)(c0 + (s0 > 0 ? en : 0)) * d0 - x0) * iv0 : INF;
-                tn1 = s1 ? (lo1 + (float)(c1 + (s1 > 0 ? en : 0)) * d1 - x1) * iv1 : INF;
-                tn2 = s2 ? (lo2 + (float)(c2 + (s2 > 0 ? en : 0)) * d2 - x2) * iv2 : INF;
+                tn0 = s0 ? face_t(i2f_small(c0 + (s0 > 0 ? en : 0)), A.d_f[0], A.lo_f[0], x0, iv0) : INF;
+                tn1 = s1 ? face_t(i2f_small(c1 + (s1 > 0 ? en : 0)), A.d_f[1], A.lo_f[1], x1, iv1) : INF;
+                tn2 = s2 ? face_t(i2f_small(c2 + (s2 > 0 ? en : 0)), A.d_f[2], A.lo_f[2], x2, iv2) : INF;
                 last_axis = axis;
             }
         }
-        if (tau_h > tau_cut && mode != M_LOCATE) done = true;
+        if (tau_h > A.tau_cut && mode != M_LOCATE) done = true;
         if (done) mode = M_NONE;
     };
 
-    // one cell crossing of the current traversal
+    // one cell crossing of the current traversal (Cartesian)
     auto step = [&]() {
-        const float tmin = fminf(fminf(tn0, tn1), tn2);
-        const int axis = (tn0 == tmin) ? 0 : ((tn1 == tmin) ? 1 : 2);
+        const float tmin = fminf(tn0, fminf(tn1, tn2));
+        const bool e0 = tn0 == tmin, e1 = tn1 == tmin;  // the exit axis: the first at tmin
         // the next cell is known before the current one is processed: issue
         // its density load now so that it overlaps with this crossing's work
-        const int cs = axis == 0 ? c0 : (axis == 1 ? c1 : c2);
-        const int ss = axis == 0 ? s0 : (axis == 1 ? s1 : s2);
-        const int na = axis == 0 ? nx : (axis == 1 ? ny : nz);
-        const int cn = cs + ss;
-        const bool out = (unsigned)cn >= (unsigned)na;
-        const int mn = cur_m + ss * (axis == 0 ? 1 : (axis == 1 ? nx : nxy));
+        const int mn = cur_m + (e0 ? st0 : (e1 ? st1 : st2));
+        bool out = false;
+        if (!(tmin < t_end)) {  // the last face of an axis, a tie with it, or a NaN
+            out = e0 ? kf0 == (KF)(sf0 > 0 ? A.nx : 0)
+                     : (e1 ? kf1 == (KF)(sf1 > 0 ? A.ny : 0) : kf2 == (KF)(sf2 > 0 ? A.nz : 0));
+        }
         const float kr_next = out ? 0.f : __ldg(kr + mn);
         const float ds = fmaxf(tmin - tcur, 0.f);
-        const int m = cur_m;
         const float krl = kr_cur * krs;
         const float dtau = krl * ds;
         ++nsteps;
-        bool done = false;
-        const float tau_prev = tau_h + tau_l;
-        if (mode == M_LOCATE) {
-            if (krl > 0.f) {
-                if (tau_h + (tau_l + dtau) >= rem_f) {
-                    s_found = (rem_f - tau_prev) / krl;  // distance inside the current cell
-                    found = true;
-                    done = true;
-                } else {
+        if (mode != M_PEEL) {
+            const float tau_prev = tau_h + tau_l;
+            if (mode == M_DEPOSIT) {
+                if (dtau > 0.f) deposit(cur_m, tau_prev, dtau);
+            } else {
+                if (krl > 0.f) {
+                    if (tau_h + (tau_l + dtau) >= par) {
+                        s_found = (par - tau_prev) / krl;  // distance inside the current cell
+                        found = true;
+                        mode = M_NONE;
+                        return;  // the current cell stays
+                    }
                     last_dusty_end = tmin;
                 }
+                last_axis = e0 ? 0 : (e1 ? 1 : 2);
             }
-        } else if (mode == M_DEPOSIT && dtau > 0.f) {
-            const float dep = labs_f * exp_neg(tau_prev) * one_minus_exp_neg(dtau);
-            if (dep >= 1.17549435e-38f)
-                atomicAdd(absorbed + ((size_t)m * A.abs_cs + (size_t)lam * A.abs_ls), f2d_pos(dep));
         }
         df_accumulate(tau_h, tau_l, dtau);
-        if (!done) {
-            tcur = tmin;
-            if (out) {
-                done = true;
-            } else {
-                cur_m = mn;
-                kr_cur = kr_next;
-                const float loa = axis == 0 ? lo0 : (axis == 1 ? lo1 : lo2);
-                const float da = axis == 0 ? d0 : (axis == 1 ? d1 : d2);
-                const float xa = axis == 0 ? x0 : (axis == 1 ? x1 : x2);
-                const float iva = axis == 0 ? iv0 : (axis == 1 ? iv1 : iv2);
-                const float tnew = (loa + (float)(cn + (ss > 0)) * da - xa) * iva;
-                c0 = axis == 0 ? cn : c0;
-                c1 = axis == 1 ? cn : c1;
-                c2 = axis == 2 ? cn : c2;
-                tn0 = axis == 0 ? tnew : tn0;
-                tn1 = axis == 1 ? tnew : tn1;
-                tn2 = axis == 2 ? tnew : tn2;
-                last_axis = axis;
-            }
+        tcur = tmin;
+        cur_m = mn;
+        kr_cur = kr_next;
+        if constexpr (BIG) {
+            if (e0) { kf0 += sf0; tn0 = face_t((float)kf0, A.d_f[0], A.lo_f[0], x0, iv0); }
+            else if (e1) { kf1 += sf1; tn1 = face_t((float)kf1, A.d_f[1], A.lo_f[1], x1, iv1); }
+            else { kf2 += sf2; tn2 = face_t((float)kf2, A.d_f[2], A.lo_f[2], x2, iv2); }
+        } else {
+            // the exit axis's next face: four instructions per axis under its
+            // predicate, in place of selecting nine operands by axis
+            asm("{\n\t"
+                ".reg .pred p0, p1, p2;\n\t"
+                ".reg .f32 u;\n\t"
+                "setp.eq.f32 p0, %0, %6;\n\t"
+                "setp.eq.and.f32 p1, %1, %6, !p0;\n\t"
+                "or.pred p2, p0, p1;\n\t"
+                "@p0 add.rn.f32 %3, %3, %7;\n\t"
+                "@p1 add.rn.f32 %4, %4, %8;\n\t"
+                "@!p2 add.rn.f32 %5, %5, %9;\n\t"
+                "@p0 fma.rn.f32 %0, %3, %10, %13;\n\t"
+                "@p1 fma.rn.f32 %1, %4, %11, %14;\n\t"
+                "@!p2 fma.rn.f32 %2, %5, %12, %15;\n\t"
+                "@p0 sub.rn.f32 %0, %0, %16;\n\t"
+                "@p1 sub.rn.f32 %1, %1, %17;\n\t"
+                "@!p2 sub.rn.f32 %2, %2, %18;\n\t"
+                "@p0 mul.rn.f32 %0, %0, %19;\n\t"
+                "@p1 mul.rn.f32 %1, %1, %20;\n\t"
+                "@!p2 mul.rn.f32 %2, %2, %21;\n\t"
+                "}"
+                : "+f"(tn0), "+f"(tn1), "+f"(tn2), "+f"(kf0), "+f"(kf1), "+f"(kf2)
+                : "f"(tmin), "f"(sf0), "f"(sf1), "f"(sf2), "f"(A.d_f[0]), "f"(A.d_f[1]), "f"(A.d_f[2]),
+                  "f"(A.lo_f[0]), "f"(A.lo_f[1]), "f"(A.lo_f[2]), "f"(x0), "f"(x1), "f"(x2), "f"(iv0), "f"(iv1),
+                  "f"(iv2));
         }
         // Beyond tau = tau_cut (30) a line of sight transmits < e^-30 (1e-13) and a
         // deposit path has handed < e^-30 of the luminosity to its remaining
         // cells; 1 - e^-tau is 1 in FP32 from tau = 17 on, so the forced
         // scattering draw does not change: the traversal ends there (the search
         // never gets that far, since tau_int < 17 in FP32).
-        if (tau_h > tau_cut && mode != M_LOCATE) done = true;
-        if (done) mode = M_NONE;
+        if (out || tau_h > A.tau_cut) mode = M_NONE;
     };
 
     auto draw = [&](uint32_t event, uint32_t block) -> uint4 {
@@ -424,24 +493,160 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         C.l_emit[t] = C.l_abs[t] = C.l_esc[t] = C.l_res[t] = 0.0;
     };
 
-    auto start_peel = [&](int i) {
-        const InstrDev& I = sins[i];
-        float w;
-        if (C.peel_kind[t] == 0) {
-            w = L;  // isotropic emission: phase factor 1
-        } else {
-            const float mu = k0 * I.kobs_f[0] + k1 * I.kobs_f[1] + k2 * I.kobs_f[2];
-            w = L * hg_phase<float>(gg, mu);
-        }
-        C.peel_w[t] = w;
-        if (w > 0.f) begin(M_PEEL, I.kobs_f[0], I.kobs_f[1], I.kobs_f[2]);
-        else nsteps = 0;
-    };
-
-    // event handling: runs the lane's stages until it enters a traversal or
-    // runs out of packets
+    // Event handling, from the end of a traversal to the start of the next, as
+    // one pass over the stages in the order a packet meets them: the lanes of a
+    // warp, whatever traversal they ended, share the code of the later stages
+    // and one copy of the traversal set-up (the previous form set each
+    // traversal up inside its own stage, five copies run by a few lanes each).
+    // A lane goes round again only where no traversal came of a pass (a
+    // peel-off of zero weight).
     auto events = [&]() {
-        while (mode == M_NONE && alive) {
+        int need;
+        do {
+            need = M_NONE;
+            float w0 = k0, w1 = k1, w2 = k2;  // direction of the traversal to start
+            if (stage == ST_PEEL_DONE) {
+                C.c_peel[t] += nsteps;
+                const int pi = C.peel_i[t];
+                const InstrDev& I = sins[pi];
+                const float w = C.peel_w[t];
+                if (w > 0.f) {
+                    const float tobs = tau_h + tau_l;
+                    const float flux = w * expf(-tobs) * I.flux_norm_f;
+                    C.p_peel[t] += flux;
+                    const float a = x0 * I.e1_f[0] + x1 * I.e1_f[1] + x2 * I.e1_f[2] +
+                                    (C.xl0[t] * I.e1_f[0] + C.xl1[t] * I.e1_f[1] + C.xl2[t] * I.e1_f[2]);
+                    const float b = x0 * I.e2_f[0] + x1 * I.e2_f[1] + x2 * I.e2_f[2] +
+                                    (C.xl0[t] * I.e2_f[0] + C.xl1[t] * I.e2_f[1] + C.xl2[t] * I.e2_f[2]);
+                    const float fa = (a + I.half_fov_f) * I.inv_dpx_f;
+                    const float fb = (b + I.half_fov_f) * I.inv_dpx_f;
+                    if (flux >= 1.17549435e-38f) {
+                        // one FP64 reduction per peel-off (lanes of a warp rarely share a
+                        // pixel; aggregating them measured no faster)
+                        const float np = (float)I.npx;
+                        if (fa >= 0.f && fa < np && fb >= 0.f && fb < np) {
+                            const int pix = floor_small(fb) * I.npx + floor_small(fa);
+                            atomicAdd(A.images + I.img_off + (long long)pix * A.nlambda + lam, f2d(flux));
+                        } else {
+                            atomicAdd(A.oof + (size_t)pi * A.nlambda + lam, f2d(flux));
+                        }
+                    }
+                }
+                C.peel_i[t] = pi + 1;
+                stage = pi + 1 < A.ninstr ? ST_PEEL : (C.peel_kind[t] ? ST_AFTER_SCATTER : ST_START_DEP);
+            } else if (stage == ST_DEPOSIT_DONE) {
+                C.c_dep[t] += nsteps;
+                // om = 1 - e^{-tau_path}: from expm1 for small tau, from 1 - exp for
+                // large tau, so that both om and 1 - om keep FP32 relative precision
+                const float tf = tau_h + tau_l;
+                float om, E;
+                if (tf < 0.6931472f) { om = -expm1f(-tf); E = 1.f - om; }
+                else { E = expf(-tf); om = 1.f - E; }
+                C.p_esc[t] += L * E;
+                C.p_abs[t] += L * (1.f - C.alb[t]) * om;
+                // the path's optical depth is positive when its high word is a positive
+                // normal number (the crossings' rounding errors in the low word are far
+                // smaller); a sign bit means a NaN
+                const int th = __float_as_int(tau_h);
+                if (th < 0x00800000) {
+                    if (th < 0) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
+                    L = 0.f;
+                    C.nscat[t] = (int)C.ev[t] - 1;
+                    stage = ST_END_PACKET;
+                } else {
+                    C.om[t] = om;
+                    // forced scattering: tau_int from the exponential truncated at tau_path
+                    const uint4 r = draw(C.ev[t], 0u);
+                    C.ry[t] = r.y;
+                    C.rz[t] = r.z;
+                    par = -log1pf(-u01f(r.x) * om);
+                    need = M_LOCATE;
+                    found = false;
+                    last_dusty_end = 0.f;
+                    stage = ST_LOCATE_DONE;
+                }
+            } else if (stage == ST_LOCATE_DONE) {
+                C.c_loc[t] += nsteps;
+                float l0 = C.xl0[t], l1 = C.xl1[t], l2 = C.xl2[t];
+                have_pc = found;
+                if (found) {
+                    if constexpr (OCT) {
+                        pc0 = c0; pc1 = c1; pc2 = c2;
+                        pc_node = onode;
+                    } else {
+                        pc0 = (int)kf0 - (sf0 > 0); pc1 = (int)kf1 - (sf1 > 0); pc2 = (int)kf2 - (sf2 > 0);
+                    }
+                }
+                float s = found ? s_found : last_dusty_end;
+                if (found && last_axis >= 0) {
+                    // entry point of the interaction cell, snapped onto the exact face plane
+                    df_add_prod(x0, l0, tcur, k0);
+                    df_add_prod(x1, l1, tcur, k1);
+                    df_add_prod(x2, l2, tcur, k2);
+                    const int e = OCT ? 1 << (OL - olev) : 1;
+                    const float ka = last_axis == 0 ? k0 : (last_axis == 1 ? k1 : k2);
+                    const int ca = last_axis == 0 ? pc0 : (last_axis == 1 ? pc1 : pc2);
+                    const int off = last_axis == 0 ? 0 : (last_axis == 1 ? A.nx + 1 : A.nx + 1 + A.ny + 1);
+                    const float2 f = __ldg(A.faces + off + ca + (ka < 0.f ? e : 0));
+                    if (last_axis == 0) { x0 = f.x; l0 = f.y; }
+                    else if (last_axis == 1) { x1 = f.x; l1 = f.y; }
+                    else { x2 = f.x; l2 = f.y; }
+                }
+                df_add_prod(x0, l0, s, k0);
+                df_add_prod(x1, l1, s, k1);
+                df_add_prod(x2, l2, s, k2);
+                C.xl0[t] = l0; C.xl1[t] = l1; C.xl2[t] = l2;
+                L = L * C.alb[t] * C.om[t];
+                C.nscat[t] = (int)C.ev[t];
+                if (L > 0.f && A.peel && A.ninstr > 0) {
+                    C.peel_kind[t] = 1;
+                    C.peel_i[t] = 0;
+                    stage = ST_PEEL;
+                } else {
+                    stage = ST_AFTER_SCATTER;
+                }
+            }
+
+            if (stage == ST_AFTER_SCATTER) {
+                if (L <= A.w_min_f * C.L0[t]) {
+                    C.p_res[t] += L;
+                    stage = ST_END_PACKET;
+                } else if ((int)C.ev[t] >= A.max_events) {
+                    atomicOr(A.err, (unsigned)ERRBIT_EVENT_CAP);
+                    C.p_res[t] += L;
+                    stage = ST_END_PACKET;
+                } else {
+                    // Henyey-Greenstein scattering: mu by inverse CDF, azimuth uniform
+                    const float mu = hg_mu<float>(gg, u01f(C.ry[t]));
+                    float sp, cp;
+                    sincospif(2.f * u01f(C.rz[t]), &sp, &cp);
+                    hg_rotate<float>(k0, k1, k2, mu, sp, cp);
+                    stage = ST_START_DEP;
+                }
+            }
+
+            if (stage == ST_END_PACKET) {
+                C.c_scat[t] += (unsigned long long)C.nscat[t];
+                const float pe = C.p_esc[t], pa = C.p_abs[t], pr = C.p_res[t], pp = C.p_peel[t];
+                C.l_abs[t] += f2d(pa);
+                C.l_esc[t] += f2d(pe);
+                C.l_res[t] += f2d(pr);
+                if (!isfinite(pe + pa + pr + pp)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
+                const unsigned pk = C.pk[t] - (unsigned)__ldg(A.pk_first + lam);  // index within this call
+                if (pk < (unsigned)A.nrec) {
+                    double* rec = A.records + ((size_t)lam * A.nrec + pk) * SKIRT_REC_FIELDS;
+                    rec[0] = (double)C.nscat[t];
+                    rec[1] = f2d(pe);
+                    rec[2] = f2d(pa);
+                    rec[3] = f2d(pr);
+                    rec[4] = f2d(pp);
+                    rec[5] = f2d(x0) + f2d(C.xl0[t]);
+                    rec[6] = f2d(x1) + f2d(C.xl1[t]);
+                    rec[7] = f2d(x2) + f2d(C.xl2[t]);
+                }
+                stage = ST_NEW;
+            }
+
             if (stage == ST_NEW) {
                 if (C.q[t] >= C.q_end[t]) {
                     if (!A.persistent) {
@@ -469,7 +674,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                 const unsigned long long qq = C.q[t]++;
                 int ll = C.lam[t];
                 if (ll < 0 || qq < __ldg(A.offsets + ll) || qq >= __ldg(A.offsets + ll + 1)) {
-                    int a = 0, b = NL - 1;  // last wavelength whose offset <= qq
+                    int a = 0, b = A.nlambda - 1;  // last wavelength whose offset <= qq
                     while (a < b) {
                         const int mid = (a + b + 1) >> 1;
                         if (__ldg(A.offsets + mid) <= qq) a = mid; else b = mid - 1;
@@ -484,6 +689,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                     }
                 }
                 lam = ll;
+                dep_base = A.absorbed + (size_t)lam * A.abs_ls;
                 krs = __ldg(A.kscale_f + lam);
                 gg = __ldg(A.g_f + lam);
                 C.pk[t] = (unsigned)(qq - __ldg(A.offsets + lam) + __ldg(A.pk_first + lam));
@@ -516,7 +722,8 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                         x0 = A.src_df[0].x + Rr * cp;
                         x1 = A.src_df[1].x + Rr * sp;
                         x2 = A.src_df[2].x + z;
-                        if (x0 >= lo0 && x0 <= A.hi_f[0] && x1 >= lo1 && x1 <= A.hi_f[1] && x2 >= lo2 && x2 <= A.hi_f[2])
+                        if (x0 >= A.lo_f[0] && x0 <= A.hi_f[0] && x1 >= A.lo_f[1] && x1 <= A.hi_f[1] &&
+                            x2 >= A.lo_f[2] && x2 <= A.hi_f[2])
                             break;
                         if (tries + 1 >= 64) {
                             atomicOr(A.err, (unsigned)ERRBIT_SOURCE);
@@ -542,20 +749,24 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                         pc0 = lf.x; pc1 = lf.y; pc2 = lf.z;
                         side = (float)(1 << (OL - lf.w));
                     } else {
-                        pc0 = (int)(a % nx);
-                        pc1 = (int)((a / nx) % ny);
-                        pc2 = (int)(a / ((long long)nx * ny));
+                        pc0 = (int)(a % A.nx);
+                        pc1 = (int)((a / A.nx) % A.ny);
+                        pc2 = (int)(a / ((long long)A.nx * A.ny));
                     }
+                    const float2* fx = A.faces;
+                    const float2* fy = fx + (A.nx + 1);
+                    const float2* fz = fy + (A.ny + 1);
                     const float2 f0 = __ldg(fx + pc0), f1 = __ldg(fy + pc1), f2 = __ldg(fz + pc2);
                     x0 = f0.x; l0 = f0.y;
                     x1 = f1.x; l1 = f1.y;
                     x2 = f2.x; l2 = f2.y;
-                    df_add_prod(x0, l0, u01f(r.y), side * d0);
-                    df_add_prod(x1, l1, u01f(r.z), side * d1);
-                    df_add_prod(x2, l2, u01f(r.w), side * d2);
+                    df_add_prod(x0, l0, u01f(r.y), side * A.d_f[0]);
+                    df_add_prod(x1, l1, u01f(r.z), side * A.d_f[1]);
+                    df_add_prod(x2, l2, u01f(r.w), side * A.d_f[2]);
                     have_pc = !OCT;
                 }
                 C.xl0[t] = l0; C.xl1[t] = l1; C.xl2[t] = l2;
+                stage = ST_START_DEP;
                 if (isotropic) {
                     const uint4 r = draw(0u, 1u);
                     const float mu = 2.f * u01f(r.x) - 1.f;
@@ -563,168 +774,37 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                     float sp, cp;
                     sincospif(2.f * u01f(r.y), &sp, &cp);
                     k0 = st * cp; k1 = st * sp; k2 = mu;
-                }
-                if (isotropic && A.peel && A.ninstr > 0) {
-                    C.peel_kind[t] = 0;
-                    C.peel_i[t] = 0;
-                    C.after_peel[t] = ST_START_DEP;
-                    stage = ST_PEEL_DONE;
-                    start_peel(0);
-                } else {
-                    stage = ST_START_DEP;
-                }
-                continue;
-            }
-
-            if (stage == ST_START_DEP) {
-                C.ev[t] += 1;
-                labs_f = L * (1.f - C.alb[t]);
-                begin(M_DEPOSIT, k0, k1, k2);
-                stage = ST_DEPOSIT_DONE;
-                continue;
-            }
-
-            if (stage == ST_DEPOSIT_DONE) {
-                C.c_dep[t] += nsteps;
-                const double tau_path = f2d(tau_h) + f2d(tau_l);  // the path's optical depth, FP64
-                // om = 1 - e^{-tau_path}: from expm1 for small tau, from 1 - exp for
-                // large tau, so that both om and 1 - om keep FP32 relative precision
-                const float tf = tau_h + tau_l;
-                float om, E;
-                if (tf < 0.6931472f) { om = -expm1f(-tf); E = 1.f - om; }
-                else { E = expf(-tf); om = 1.f - E; }
-                C.p_esc[t] += L * E;
-                C.p_abs[t] += L * (1.f - C.alb[t]) * om;
-                if (!(tau_path > 0.0)) {
-                    if (!(tau_path == 0.0)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
-                    L = 0.f;
-                    C.nscat[t] = (int)C.ev[t] - 1;
-                    stage = ST_END_PACKET;
-                    continue;
-                }
-                C.om[t] = om;
-                // forced scattering: tau_int from the exponential truncated at tau_path
-                const uint4 r = draw(C.ev[t], 0u);
-                const float tau_int = -log1pf(-u01f(r.x) * om);
-                begin(M_LOCATE, k0, k1, k2);
-                rem_f = tau_int;
-                found = false;
-                last_dusty_end = 0.f;
-                stage = ST_LOCATE_DONE;
-                continue;
-            }
-
-            if (stage == ST_LOCATE_DONE) {
-                C.c_loc[t] += nsteps;
-                float l0 = C.xl0[t], l1 = C.xl1[t], l2 = C.xl2[t];
-                if (found && last_axis >= 0) {
-                    // entry point of the interaction cell, snapped onto the exact face plane
-                    df_add_prod(x0, l0, tcur, k0);
-                    df_add_prod(x1, l1, tcur, k1);
-                    df_add_prod(x2, l2, tcur, k2);
-                    const int e = OCT ? 1 << (OL - olev) : 1;
-                    if (last_axis == 0) { const float2 f = __ldg(fx + c0 + (s0 < 0 ? e : 0)); x0 = f.x; l0 = f.y; }
-                    else if (last_axis == 1) { const float2 f = __ldg(fy + c1 + (s1 < 0 ? e : 0)); x1 = f.x; l1 = f.y; }
-                    else { const float2 f = __ldg(fz + c2 + (s2 < 0 ? e : 0)); x2 = f.x; l2 = f.y; }
-                    df_add_prod(x0, l0, s_found, k0);
-                    df_add_prod(x1, l1, s_found, k1);
-                    df_add_prod(x2, l2, s_found, k2);
-                } else {
-                    const float s = found ? s_found : last_dusty_end;
-                    df_add_prod(x0, l0, s, k0);
-                    df_add_prod(x1, l1, s, k1);
-                    df_add_prod(x2, l2, s, k2);
-                }
-                C.xl0[t] = l0; C.xl1[t] = l1; C.xl2[t] = l2;
-                have_pc = found;
-                if (found) { pc0 = c0; pc1 = c1; pc2 = c2; pc_node = onode; }
-                L = L * C.alb[t] * C.om[t];
-                C.nscat[t] = (int)C.ev[t];
-                if (L > 0.f && A.peel && A.ninstr > 0) {
-                    C.peel_kind[t] = 1;
-                    C.peel_i[t] = 0;
-                    C.after_peel[t] = ST_AFTER_SCATTER;
-                    stage = ST_PEEL_DONE;
-                    start_peel(0);
-                } else {
-                    stage = ST_AFTER_SCATTER;
-                }
-                continue;
-            }
-
-            if (stage == ST_PEEL_DONE) {
-                C.c_peel[t] += nsteps;
-                const int pi = C.peel_i[t];
-                const InstrDev& I = sins[pi];
-                const float w = C.peel_w[t];
-                if (w > 0.f) {
-                    const float tobs = tau_h + tau_l;
-                    const float flux = w * expf(-tobs) * I.flux_norm_f;
-                    C.p_peel[t] += flux;
-                    const float a = x0 * I.e1_f[0] + x1 * I.e1_f[1] + x2 * I.e1_f[2] +
-                                    (C.xl0[t] * I.e1_f[0] + C.xl1[t] * I.e1_f[1] + C.xl2[t] * I.e1_f[2]);
-                    const float b = x0 * I.e2_f[0] + x1 * I.e2_f[1] + x2 * I.e2_f[2] +
-                                    (C.xl0[t] * I.e2_f[0] + C.xl1[t] * I.e2_f[1] + C.xl2[t] * I.e2_f[2]);
-                    const float fa = floorf((a + I.half_fov_f) * I.inv_dpx_f);
-                    const float fb = floorf((b + I.half_fov_f) * I.inv_dpx_f);
-                    if (flux >= 1.17549435e-38f) {
-                        // one FP64 reduction per peel-off (lanes of a warp rarely share a
-                        // pixel; aggregating them measured no faster)
-                        if (fa >= 0.f && fa < (float)I.npx && fb >= 0.f && fb < (float)I.npx) {
-                            const long long pix = (long long)fb * I.npx + (long long)fa;
-                            atomicAdd(A.images + I.img_off + pix * NL + lam, f2d(flux));
-                        } else {
-                            atomicAdd(A.oof + (size_t)pi * NL + lam, f2d(flux));
-                        }
+                    if (A.peel && A.ninstr > 0) {
+                        C.peel_kind[t] = 0;
+                        C.peel_i[t] = 0;
+                        stage = ST_PEEL;
                     }
                 }
-                C.peel_i[t] = pi + 1;
-                if (pi + 1 < A.ninstr) start_peel(pi + 1);
-                else stage = C.after_peel[t];
-                continue;
             }
 
-            if (stage == ST_AFTER_SCATTER) {
-                if (L <= A.w_min_f * C.L0[t]) {
-                    C.p_res[t] += L;
-                    stage = ST_END_PACKET;
-                } else if ((int)C.ev[t] >= A.max_events) {
-                    atomicOr(A.err, (unsigned)ERRBIT_EVENT_CAP);
-                    C.p_res[t] += L;
-                    stage = ST_END_PACKET;
-                } else {
-                    // Henyey-Greenstein scattering: mu by inverse CDF, azimuth uniform
-                    const uint4 r = draw(C.ev[t], 0u);
-                    const float mu = hg_mu<float>(gg, u01f(r.y));
-                    float sp, cp;
-                    sincospif(2.f * u01f(r.z), &sp, &cp);
-                    hg_rotate<float>(k0, k1, k2, mu, sp, cp);
-                    stage = ST_START_DEP;
+            if (stage == ST_PEEL) {
+                const InstrDev& I = sins[C.peel_i[t]];
+                float w = L;  // isotropic emission: phase factor 1
+                if (C.peel_kind[t]) {
+                    const float mu = k0 * I.kobs_f[0] + k1 * I.kobs_f[1] + k2 * I.kobs_f[2];
+                    w = L * hg_phase<float>(gg, mu);
                 }
-                continue;
+                C.peel_w[t] = w;
+                stage = ST_PEEL_DONE;
+                nsteps = 0;
+                if (w > 0.f) {
+                    need = M_PEEL;
+                    w0 = I.kobs_f[0]; w1 = I.kobs_f[1]; w2 = I.kobs_f[2];
+                }
+            } else if (stage == ST_START_DEP) {
+                C.ev[t] += 1;
+                par = L * (1.f - C.alb[t]);
+                need = M_DEPOSIT;
+                w0 = k0; w1 = k1; w2 = k2;
+                stage = ST_DEPOSIT_DONE;
             }
-
-            // ST_END_PACKET
-            C.c_scat[t] += (unsigned long long)C.nscat[t];
-            const float pe = C.p_esc[t], pa = C.p_abs[t], pr = C.p_res[t], pp = C.p_peel[t];
-            C.l_abs[t] += f2d(pa);
-            C.l_esc[t] += f2d(pe);
-            C.l_res[t] += f2d(pr);
-            if (!isfinite(pe + pa + pr + pp)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
-            const unsigned pk = C.pk[t] - (unsigned)__ldg(A.pk_first + lam);  // index within this call
-            if (pk < (unsigned)A.nrec) {
-                double* rec = A.records + ((size_t)lam * A.nrec + pk) * SKIRT_REC_FIELDS;
-                rec[0] = (double)C.nscat[t];
-                rec[1] = f2d(pe);
-                rec[2] = f2d(pa);
-                rec[3] = f2d(pr);
-                rec[4] = f2d(pp);
-                rec[5] = f2d(x0) + f2d(C.xl0[t]);
-                rec[6] = f2d(x1) + f2d(C.xl1[t]);
-                rec[7] = f2d(x2) + f2d(C.xl2[t]);
-            }
-            stage = ST_NEW;
-        }
+            if (need != M_NONE) begin(need, w0, w1, w2);
+        } while (need == M_NONE);
     };
 
     for (;;) {
@@ -763,11 +843,12 @@ size_t trace_mixed_smem_bytes(int ninstr, int block)
 
 static cudaError_t set_smem_limit()
 {
-    cudaError_t e = cudaFuncSetAttribute(trace_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)trace_mixed_smem_bytes(16, MAXB));
+    const int bytes = (int)trace_mixed_smem_bytes(16, MAXB);
+    cudaError_t e = cudaFuncSetAttribute(trace_mixed_kernel<G_CART>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(trace_mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)trace_mixed_smem_bytes(16, MAXB));
+    e = cudaFuncSetAttribute(trace_mixed_kernel<G_CART_BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(trace_mixed_kernel<G_OCT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 cudaError_t launch_trace_mixed(const TraceArgs& a, int block, int grid, cudaStream_t s)
@@ -775,10 +856,13 @@ cudaError_t launch_trace_mixed(const TraceArgs& a, int block, int grid, cudaStre
     if (block > MAXB || block % 32) return cudaErrorInvalidValue;
     cudaError_t e = set_smem_limit();
     if (e != cudaSuccess) return e;
+    const size_t smem = trace_mixed_smem_bytes(a.ninstr, block);
     if (a.oct_levels > 0)
-        trace_mixed_kernel<true><<<grid, block, trace_mixed_smem_bytes(a.ninstr, block), s>>>(a);
+        trace_mixed_kernel<G_OCT><<<grid, block, smem, s>>>(a);
+    else if (a.nx < (1 << 23) && a.ny < (1 << 23) && a.nz < (1 << 23))
+        trace_mixed_kernel<G_CART><<<grid, block, smem, s>>>(a);
     else
-        trace_mixed_kernel<false><<<grid, block, trace_mixed_smem_bytes(a.ninstr, block), s>>>(a);
+        trace_mixed_kernel<G_CART_BIG><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -790,10 +874,9 @@ cudaError_t trace_mixed_occupancy(int block, int* blocks_per_sm, bool octree)
     }
     cudaError_t e = set_smem_limit();
     if (e != cudaSuccess) return e;
-    return octree ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_mixed_kernel<true>, block,
-                                                                  trace_mixed_smem_bytes(16, block))
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_mixed_kernel<false>, block,
-                                                                  trace_mixed_smem_bytes(16, block));
+    const size_t smem = trace_mixed_smem_bytes(16, block);
+    return octree ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_mixed_kernel<G_OCT>, block, smem)
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_mixed_kernel<G_CART>, block, smem);
 }
 
 }  // namespace skirt
