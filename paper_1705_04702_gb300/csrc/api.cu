@@ -113,6 +113,7 @@ void fill_instrument(const skirt_instrument& s, InstrDev& d, long long img_off)
         d.e1[a] = e1[a];
         d.e2[a] = e2[a];
         d.kobs_f[a] = (float)k[a];
+        d.ikobs_f[a] = d.kobs_f[a] != 0.f ? 1.f / d.kobs_f[a] : 0.f;
         d.e1_f[a] = (float)e1[a];
         d.e2_f[a] = (float)e2[a];
     }

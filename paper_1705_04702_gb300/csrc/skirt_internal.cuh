@@ -44,6 +44,7 @@ struct InstrDev {
     double kobs[3], e1[3], e2[3];
     double half_fov, inv_dpx, flux_norm;
     float kobs_f[3], e1_f[3], e2_f[3];
+    float ikobs_f[3];   // 1 / kobs_f, zero for zero components
     float half_fov_f, inv_dpx_f, flux_norm_f;
     int npx;
     long long img_off;  // element offset of this instrument in the images array

@@ -34,17 +34,21 @@
 //    om = 1 - e^{-tau_path}, so they add up to the packet luminosity.
 //  * Per-thread state used only at events lives in shared memory.
 //
-// What bounds it is instruction issue (72% of the cycles on the 256^3 disk),
+// What bounds it is instruction issue (71% of the cycles on the 256^3 disk),
 // so the crossing is written for few warp instructions: the exit axis's next
 // face is advanced under predicates from FP32 face indices, leaving the grid
-// is tested by one distance comparison, and the cell index moves by a signed
-// stride.  The lanes handle events in one pass over the stages with a single
-// copy of the traversal set-up and one random block per scattering, which
-// also keeps the loop inside the instruction cache.  Against selecting every
-// operand by axis and setting traversals up inside each stage: 1e7 packets on
-// the 256^3 disk 185.8 ms (250.4), 8e6 packets of 200 wavelengths on the 128^3
-// torus 135.9 ms (192.7), 3e6 packets on an octree of 8.3e5 leaves 63.6 ms
-// (94.6), the same histories bit for bit.
+// is tested by one distance comparison, the cell index moves by a signed
+// stride, and no branch separates the traversal kinds.  The lanes handle
+// events in one pass over the stages with a single copy of the traversal
+// set-up and one random block per scattering, which also keeps the loop inside
+// the instruction cache; the search for the interaction starts from the saved
+// start of the deposit traversal it repeats.  Against selecting every operand
+// by axis and setting traversals up inside each stage: 1e7 packets on the
+// 256^3 disk 172 ms (259), 8e6 packets of 200 wavelengths on the 128^3 torus
+// 117 ms (200), 3e6 packets on an octree of 8.3e5 leaves 58 ms (94), the same
+// histories bit for bit.  A crossing is now ~99 warp instructions for the
+// lanes of a warp (27 of them the deposit's); events take a fifth of the
+// instructions, run by 4 to 5 lanes at a time.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -151,14 +155,26 @@ __device__ __forceinline__ float face_t(float k, float d, float lo, float x, flo
 // Per-thread state used only at events, struct of arrays in shared memory.
 struct Cold {
     double l_emit[MAXB], l_abs[MAXB], l_esc[MAXB], l_res[MAXB];
-    unsigned long long q[MAXB], q_end[MAXB];
-    unsigned long long c_dep[MAXB], c_loc[MAXB], c_peel[MAXB], c_scat[MAXB];
+    unsigned long long q[MAXB];
+    unsigned left[MAXB];                                        // packets left of the last queue refill
+    unsigned c_dep[MAXB], c_loc[MAXB], c_peel[MAXB], c_scat[MAXB];  // added to the 64-bit counters below 2^32
     float L0[MAXB], p_esc[MAXB], p_abs[MAXB], p_res[MAXB], p_peel[MAXB], om[MAXB], peel_w[MAXB], alb[MAXB];
     float xl0[MAXB], xl1[MAXB], xl2[MAXB];  // low words of the double-float position
-    int lam[MAXB], led_lam[MAXB], nscat[MAXB], peel_i[MAXB], peel_kind[MAXB];
-    unsigned pk[MAXB], ev[MAXB], started[MAXB];
+    int lam[MAXB], nscat[MAXB], peel_i[MAXB];  // peel_i: instrument, + PEEL_SCATTER after a scattering
+    unsigned pk[MAXB], ev[MAXB];
     unsigned ry[MAXB], rz[MAXB];            // the event's second and third random words
+    // the deposit traversal's start, from which the search along the same ray
+    // starts again: distances to the first faces, face indices (octree: lattice
+    // corner), cell (node)
+    float b_t0[MAXB], b_t1[MAXB], b_t2[MAXB];
+    int b_k0[MAXB], b_k1[MAXB], b_k2[MAXB], b_m[MAXB];
+    float b_kr[MAXB];
+    // the search's interaction cell (octree: node; -1 before it is found), the
+    // distance at which it was entered, the length inside it, how it was entered
+    int f_m[MAXB], f_last[MAXB];
+    float f_t[MAXB], f_s[MAXB];
 };
+constexpr int PEEL_SCATTER = 16;  // at most 16 instruments
 
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
@@ -180,11 +196,10 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     for (int i = threadIdx.x; i < A.ninstr; i += blockDim.x) sins[i] = A.ins[i];
     const int t = threadIdx.x;
     C.l_emit[t] = C.l_abs[t] = C.l_esc[t] = C.l_res[t] = 0.0;
-    C.q[t] = C.q_end[t] = 0;
+    C.q[t] = 0;
+    C.left[t] = 0;
     C.c_dep[t] = C.c_loc[t] = C.c_peel[t] = C.c_scat[t] = 0;
     C.lam[t] = -1;
-    C.led_lam[t] = -1;
-    C.started[t] = 0;
     __syncthreads();
 
     const float INF = __int_as_float(0x7f800000);
@@ -205,9 +220,9 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     float tau_h = 0.f, tau_l = 0.f;  // running optical depth of the traversal (double-float)
     float par = 0.f;                 // deposit: L (1 - albedo); search: interaction optical depth
     unsigned nsteps = 0;
-    float s_found = 0.f, last_dusty_end = 0.f;
-    bool found = false;
-    int last_axis = -1;  // search: axis of the face through which the current cell was entered
+    float last_dusty_end = 0.f;  // search: where the last dusty cell crossed ended
+    int last = 0;        // search: how the current cell was entered (0: the start cell); Cartesian: the
+                         // stride of the crossing, octree: 1 + the face's axis
     int cur_m = 0;       // index of the current cell
     float kr_cur = 0.f;  // its extinction coefficient (loaded one crossing ahead)
     double* dep_base = nullptr;  // the absorbed table at (cell 0, the packet's wavelength)
@@ -215,6 +230,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     // node of the interaction leaf
     const int OL = A.oct_levels;
     const OctNode* __restrict__ nodes = A.oct_nodes;
+    bool started = false;  // per-wavelength schedule: this thread's packet is taken
     int onode = 0, olev = 0, pc_node = 0;
     float v0 = 0.f, v1 = 0.f, v2 = 0.f;
     // ---- packet state (registers)
@@ -254,40 +270,40 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         c2 = j2 & mask;
     };
 
-    // starts a traversal of kind m along (vx, vy, vz) from the packet's position
-    auto begin = [&](int m, float vx, float vy, float vz) {
+    // starts a traversal of kind m along (vx, vy, vz), whose reciprocals (zero
+    // for zero components) are (i0, i1, i2), from the packet's position
+    auto begin = [&](int m, float vx, float vy, float vz, float i0, float i1, float i2) {
         mode = m;
         const float2* __restrict__ fx = A.faces;
         const float2* __restrict__ fy = fx + (A.nx + 1);
         const float2* __restrict__ fz = fy + (A.ny + 1);
         const float l0 = C.xl0[t], l1 = C.xl1[t], l2 = C.xl2[t];
-        int b0 = pc0, b1 = pc1, b2 = pc2;
         if (!have_pc) {
-            b0 = axis_cell(x0, l0, A.lo_f[0], A.d_f[0], A.nx, fx);
-            b1 = axis_cell(x1, l1, A.lo_f[1], A.d_f[1], A.ny, fy);
-            b2 = axis_cell(x2, l2, A.lo_f[2], A.d_f[2], A.nz, fz);
+            pc0 = axis_cell(x0, l0, A.lo_f[0], A.d_f[0], A.nx, fx);
+            pc1 = axis_cell(x1, l1, A.lo_f[1], A.d_f[1], A.ny, fy);
+            pc2 = axis_cell(x2, l2, A.lo_f[2], A.d_f[2], A.nz, fz);
+            pc_node = 0;
+            have_pc = true;
         }
         if constexpr (OCT) {
-            oct_enter(have_pc ? pc_node : 0, 0, b0, b1, b2);
-            b0 = c0; b1 = c1; b2 = c2;
+            oct_enter(pc_node, 0, pc0, pc1, pc2);
+            pc0 = c0; pc1 = c1; pc2 = c2;
+            pc_node = onode;
             v0 = vx; v1 = vy; v2 = vz;
         }
         const int g0 = vx > 0.f ? 1 : (vx < 0.f ? -1 : 0);
         const int g1 = vy > 0.f ? 1 : (vy < 0.f ? -1 : 0);
         const int g2 = vz > 0.f ? 1 : (vz < 0.f ? -1 : 0);
-        iv0 = g0 ? 1.f / vx : 0.f;
-        iv1 = g1 ? 1.f / vy : 0.f;
-        iv2 = g2 ? 1.f / vz : 0.f;
+        iv0 = i0; iv1 = i1; iv2 = i2;
         // first faces from the exact face planes and the double-float position
         const int e = OCT ? 1 << (OL - olev) : 1;  // the cell's extent in lattice cells
-        const int n0 = b0 + (g0 > 0 ? e : 0), n1 = b1 + (g1 > 0 ? e : 0), n2 = b2 + (g2 > 0 ? e : 0);
+        const int n0 = pc0 + (g0 > 0 ? e : 0), n1 = pc1 + (g1 > 0 ? e : 0), n2 = pc2 + (g2 > 0 ? e : 0);
         tn0 = g0 ? df_diff(__ldg(fx + n0), x0, l0) * iv0 : INF;
         tn1 = g1 ? df_diff(__ldg(fy + n1), x1, l1) * iv1 : INF;
         tn2 = g2 ? df_diff(__ldg(fz + n2), x2, l2) * iv2 : INF;
         tcur = 0.f;
         tau_h = tau_l = 0.f;
         nsteps = 0;
-        last_axis = -1;
         if constexpr (OCT) {
             s0 = g0; s1 = g1; s2 = g2;
         } else {
@@ -303,18 +319,72 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
             const float u1 = n1 == m1 ? tn1 : face_t((float)m1, A.d_f[1], A.lo_f[1], x1, iv1);
             const float u2 = n2 == m2 ? tn2 : face_t((float)m2, A.d_f[2], A.lo_f[2], x2, iv2);
             t_end = fminf(g0 ? u0 : INF, fminf(g1 ? u1 : INF, g2 ? u2 : INF));
-            cur_m = (b2 * A.ny + b1) * A.nx + b0;
+            cur_m = (pc2 * A.ny + pc1) * A.nx + pc0;
             kr_cur = __ldg(kr + cur_m);
         }
     };
 
-    // deposit of one crossing
-    auto deposit = [&](int m, float tau_prev, float dtau) {
+    // keeps the start of a deposit traversal for the search that follows it
+    auto keep_start = [&]() {
+        C.b_t0[t] = tn0; C.b_t1[t] = tn1; C.b_t2[t] = tn2;
+        if constexpr (OCT) {
+            C.b_k0[t] = c0; C.b_k1[t] = c1; C.b_k2[t] = c2;
+            C.b_m[t] = onode;
+        } else {
+            if constexpr (BIG) { C.b_k0[t] = kf0; C.b_k1[t] = kf1; C.b_k2[t] = kf2; }
+            else { C.b_k0[t] = __float_as_int(kf0); C.b_k1[t] = __float_as_int(kf1); C.b_k2[t] = __float_as_int(kf2); }
+            C.b_m[t] = cur_m;
+            C.b_kr[t] = kr_cur;
+        }
+    };
+
+    // starts the search: the same position and direction as the deposit
+    // traversal just ended, so its direction state is still in place
+    auto begin_search = [&]() {
+        mode = M_LOCATE;
+        tn0 = C.b_t0[t]; tn1 = C.b_t1[t]; tn2 = C.b_t2[t];
+        if constexpr (OCT) {
+            c0 = C.b_k0[t]; c1 = C.b_k1[t]; c2 = C.b_k2[t];
+            onode = C.b_m[t];
+            const int2 h = __ldg(reinterpret_cast<const int2*>(nodes + onode));
+            olev = oct_leaf_level(h.x);
+            cur_m = oct_leaf_index(h.x);
+            kr_cur = __int_as_float(h.y);
+        } else {
+            if constexpr (BIG) { kf0 = C.b_k0[t]; kf1 = C.b_k1[t]; kf2 = C.b_k2[t]; }
+            else { kf0 = __int_as_float(C.b_k0[t]); kf1 = __int_as_float(C.b_k1[t]); kf2 = __int_as_float(C.b_k2[t]); }
+            cur_m = C.b_m[t];
+            kr_cur = C.b_kr[t];
+        }
+        tcur = 0.f;
+        tau_h = tau_l = 0.f;
+        nsteps = 0;
+        last = 0;
+        last_dusty_end = 0.f;
+        C.f_m[t] = -1;
+    };
+
+    // The work of one crossing in its cell, written without a branch per
+    // traversal kind: a warp's lanes are nearly always in several kinds, so the
+    // deposit's arithmetic is done by all of them and only its reduction is
+    // predicated; only the end of a search, once per scattering, branches.  (In
+    // the branched form the code after the branch ran once per kind.)
+    auto cell_work = [&](int m, float tmin, float dtau, float krl) {
+        const float tau_prev = tau_h + tau_l;
         const float dep = par * exp_neg(tau_prev) * one_minus_exp_neg(dtau);
-        if (dep >= 1.17549435e-38f)
+        if (mode == M_DEPOSIT && dep >= 1.17549435e-38f)
             atomicAdd(reinterpret_cast<double*>(reinterpret_cast<char*>(dep_base) +
                                                 (size_t)(unsigned)m * A.abs_cs8),
                       f2d_pos(dep));
+        if (mode == M_LOCATE && krl > 0.f && tau_h + (tau_l + dtau) >= par) {
+            C.f_m[t] = OCT ? onode : m;
+            C.f_t[t] = tcur;
+            C.f_s[t] = (par - tau_prev) / krl;  // distance inside the cell
+            C.f_last[t] = last;
+            mode = M_NONE;
+        }
+        last_dusty_end = krl > 0.f ? tmin : last_dusty_end;
+        df_accumulate(tau_h, tau_l, dtau);
     };
 
     // one leaf crossing of an octree traversal: the face neighbour and its
@@ -335,22 +405,9 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         const float krl = kr_cur * krs;
         const float dtau = krl * ds;
         ++nsteps;
-        bool done = false;
-        const float tau_prev = tau_h + tau_l;
-        if (mode == M_LOCATE) {
-            if (krl > 0.f) {
-                if (tau_h + (tau_l + dtau) >= par) {
-                    s_found = (par - tau_prev) / krl;
-                    found = true;
-                    done = true;
-                } else {
-                    last_dusty_end = tmin;
-                }
-            }
-        } else if (mode == M_DEPOSIT && dtau > 0.f) {
-            deposit(m, tau_prev, dtau);
-        }
-        df_accumulate(tau_h, tau_l, dtau);
+        const int run = mode;
+        cell_work(m, tmin, dtau, krl);
+        bool done = mode == M_NONE;
         if (!done) {
             tcur = tmin;
             if (out) {
@@ -393,88 +450,81 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                 tn0 = s0 ? face_t(i2f_small(c0 + (s0 > 0 ? en : 0)), A.d_f[0], A.lo_f[0], x0, iv0) : INF;
                 tn1 = s1 ? face_t(i2f_small(c1 + (s1 > 0 ? en : 0)), A.d_f[1], A.lo_f[1], x1, iv1) : INF;
                 tn2 = s2 ? face_t(i2f_small(c2 + (s2 > 0 ? en : 0)), A.d_f[2], A.lo_f[2], x2, iv2) : INF;
-                last_axis = axis;
+                last = axis + 1;
             }
         }
-        if (tau_h > A.tau_cut && mode != M_LOCATE) done = true;
+        if (tau_h > A.tau_cut && run != M_LOCATE) done = true;
         if (done) mode = M_NONE;
     };
 
     // one cell crossing of the current traversal (Cartesian)
     auto step = [&]() {
-        const float tmin = fminf(tn0, fminf(tn1, tn2));
-        const bool e0 = tn0 == tmin, e1 = tn1 == tmin;  // the exit axis: the first at tmin
-        // the next cell is known before the current one is processed: issue
-        // its density load now so that it overlaps with this crossing's work
-        const int mn = cur_m + (e0 ? st0 : (e1 ? st1 : st2));
-        bool out = false;
-        if (!(tmin < t_end)) {  // the last face of an axis, a tie with it, or a NaN
-            out = e0 ? kf0 == (KF)(sf0 > 0 ? A.nx : 0)
-                     : (e1 ? kf1 == (KF)(sf1 > 0 ? A.ny : 0) : kf2 == (KF)(sf2 > 0 ? A.nz : 0));
+        // the exit axis (the first at the smallest distance), the next cell, and
+        // the exit axis's next face.  Four instructions per axis under its
+        // predicate take the place of selecting nine operands by axis.
+        float tmin;
+        int str;
+        if constexpr (BIG) {
+            tmin = fminf(tn0, fminf(tn1, tn2));
+            if (tn0 == tmin) { str = st0; kf0 += sf0; tn0 = face_t((float)kf0, A.d_f[0], A.lo_f[0], x0, iv0); }
+            else if (tn1 == tmin) { str = st1; kf1 += sf1; tn1 = face_t((float)kf1, A.d_f[1], A.lo_f[1], x1, iv1); }
+            else { str = st2; kf2 += sf2; tn2 = face_t((float)kf2, A.d_f[2], A.lo_f[2], x2, iv2); }
+        } else {
+            asm("{\n\t"
+                ".reg .pred p0, p1, p2;\n\t"
+                "min.f32 %6, %1, %2;\n\t"
+                "min.f32 %6, %0, %6;\n\t"
+                "setp.eq.f32 p0, %0, %6;\n\t"
+                "setp.eq.and.f32 p1, %1, %6, !p0;\n\t"
+                "or.pred p2, p0, p1;\n\t"
+                "selp.b32 %7, %24, %25, p1;\n\t"
+                "selp.b32 %7, %23, %7, p0;\n\t"
+                "@p0 add.rn.f32 %3, %3, %8;\n\t"
+                "@p1 add.rn.f32 %4, %4, %9;\n\t"
+                "@!p2 add.rn.f32 %5, %5, %10;\n\t"
+                "@p0 fma.rn.f32 %0, %3, %11, %14;\n\t"
+                "@p1 fma.rn.f32 %1, %4, %12, %15;\n\t"
+                "@!p2 fma.rn.f32 %2, %5, %13, %16;\n\t"
+                "@p0 sub.rn.f32 %0, %0, %17;\n\t"
+                "@p1 sub.rn.f32 %1, %1, %18;\n\t"
+                "@!p2 sub.rn.f32 %2, %2, %19;\n\t"
+                "@p0 mul.rn.f32 %0, %0, %20;\n\t"
+                "@p1 mul.rn.f32 %1, %1, %21;\n\t"
+                "@!p2 mul.rn.f32 %2, %2, %22;\n\t"
+                "}"
+                : "+f"(tn0), "+f"(tn1), "+f"(tn2), "+f"(kf0), "+f"(kf1), "+f"(kf2), "=&f"(tmin), "=&r"(str)
+                : "f"(sf0), "f"(sf1), "f"(sf2), "f"(A.d_f[0]), "f"(A.d_f[1]), "f"(A.d_f[2]), "f"(A.lo_f[0]),
+                  "f"(A.lo_f[1]), "f"(A.lo_f[2]), "f"(x0), "f"(x1), "f"(x2), "f"(iv0), "f"(iv1), "f"(iv2), "r"(st0),
+                  "r"(st1), "r"(st2));
         }
-        const float kr_next = out ? 0.f : __ldg(kr + mn);
+        // the next cell's density, requested before the current cell is
+        // processed so that it arrives during this crossing's work
+        const int mn = cur_m + str;
+        const bool inside = tmin < t_end;
+        float kr_next = 0.f;
+        if (inside) kr_next = __ldg(kr + mn);
         const float ds = fmaxf(tmin - tcur, 0.f);
         const float krl = kr_cur * krs;
         const float dtau = krl * ds;
         ++nsteps;
-        if (mode != M_PEEL) {
-            const float tau_prev = tau_h + tau_l;
-            if (mode == M_DEPOSIT) {
-                if (dtau > 0.f) deposit(cur_m, tau_prev, dtau);
-            } else {
-                if (krl > 0.f) {
-                    if (tau_h + (tau_l + dtau) >= par) {
-                        s_found = (par - tau_prev) / krl;  // distance inside the current cell
-                        found = true;
-                        mode = M_NONE;
-                        return;  // the current cell stays
-                    }
-                    last_dusty_end = tmin;
-                }
-                last_axis = e0 ? 0 : (e1 ? 1 : 2);
-            }
-        }
-        df_accumulate(tau_h, tau_l, dtau);
+        cell_work(cur_m, tmin, dtau, krl);
+        last = str;
         tcur = tmin;
         cur_m = mn;
         kr_cur = kr_next;
-        if constexpr (BIG) {
-            if (e0) { kf0 += sf0; tn0 = face_t((float)kf0, A.d_f[0], A.lo_f[0], x0, iv0); }
-            else if (e1) { kf1 += sf1; tn1 = face_t((float)kf1, A.d_f[1], A.lo_f[1], x1, iv1); }
-            else { kf2 += sf2; tn2 = face_t((float)kf2, A.d_f[2], A.lo_f[2], x2, iv2); }
-        } else {
-            // the exit axis's next face: four instructions per axis under its
-            // predicate, in place of selecting nine operands by axis
-            asm("{\n\t"
-                ".reg .pred p0, p1, p2;\n\t"
-                ".reg .f32 u;\n\t"
-                "setp.eq.f32 p0, %0, %6;\n\t"
-                "setp.eq.and.f32 p1, %1, %6, !p0;\n\t"
-                "or.pred p2, p0, p1;\n\t"
-                "@p0 add.rn.f32 %3, %3, %7;\n\t"
-                "@p1 add.rn.f32 %4, %4, %8;\n\t"
-                "@!p2 add.rn.f32 %5, %5, %9;\n\t"
-                "@p0 fma.rn.f32 %0, %3, %10, %13;\n\t"
-                "@p1 fma.rn.f32 %1, %4, %11, %14;\n\t"
-                "@!p2 fma.rn.f32 %2, %5, %12, %15;\n\t"
-                "@p0 sub.rn.f32 %0, %0, %16;\n\t"
-                "@p1 sub.rn.f32 %1, %1, %17;\n\t"
-                "@!p2 sub.rn.f32 %2, %2, %18;\n\t"
-                "@p0 mul.rn.f32 %0, %0, %19;\n\t"
-                "@p1 mul.rn.f32 %1, %1, %20;\n\t"
-                "@!p2 mul.rn.f32 %2, %2, %21;\n\t"
-                "}"
-                : "+f"(tn0), "+f"(tn1), "+f"(tn2), "+f"(kf0), "+f"(kf1), "+f"(kf2)
-                : "f"(tmin), "f"(sf0), "f"(sf1), "f"(sf2), "f"(A.d_f[0]), "f"(A.d_f[1]), "f"(A.d_f[2]),
-                  "f"(A.lo_f[0]), "f"(A.lo_f[1]), "f"(A.lo_f[2]), "f"(x0), "f"(x1), "f"(x2), "f"(iv0), "f"(iv1),
-                  "f"(iv2));
-        }
         // Beyond tau = tau_cut (30) a line of sight transmits < e^-30 (1e-13) and a
         // deposit path has handed < e^-30 of the luminosity to its remaining
         // cells; 1 - e^-tau is 1 in FP32 from tau = 17 on, so the forced
         // scattering draw does not change: the traversal ends there (the search
         // never gets that far, since tau_int < 17 in FP32).
-        if (out || tau_h > A.tau_cut) mode = M_NONE;
+        if (!inside || tau_h > A.tau_cut) {
+            // at the last face of an axis (its index has moved one beyond), a tie
+            // with it, or a NaN
+            const bool out = kf0 == (KF)(sf0 > 0 ? A.nx + 1 : -1) || kf1 == (KF)(sf1 > 0 ? A.ny + 1 : -1) ||
+                             kf2 == (KF)(sf2 > 0 ? A.nz + 1 : -1);
+            if (out || tau_h > A.tau_cut) mode = M_NONE;
+            else kr_cur = __ldg(kr + mn);
+        }
     };
 
     auto draw = [&](uint32_t event, uint32_t block) -> uint4 {
@@ -482,7 +532,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     };
 
     auto flush_ledger = [&]() {
-        const int ll = C.led_lam[t];
+        const int ll = C.lam[t];
         if (ll >= 0) {
             double* lg = A.ledger + 4 * (size_t)ll;
             atomicAdd(lg + 0, C.l_emit[t]);
@@ -491,6 +541,14 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
             atomicAdd(lg + 3, C.l_res[t]);
         }
         C.l_emit[t] = C.l_abs[t] = C.l_esc[t] = C.l_res[t] = 0.0;
+    };
+
+    auto flush_counters = [&]() {
+        atomicAdd(A.counters + 0, (unsigned long long)C.c_scat[t]);
+        atomicAdd(A.counters + 1, (unsigned long long)C.c_dep[t]);
+        atomicAdd(A.counters + 2, (unsigned long long)C.c_loc[t]);
+        atomicAdd(A.counters + 3, (unsigned long long)C.c_peel[t]);
+        C.c_dep[t] = C.c_loc[t] = C.c_peel[t] = C.c_scat[t] = 0;
     };
 
     // Event handling, from the end of a traversal to the start of the next, as
@@ -504,10 +562,9 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         int need;
         do {
             need = M_NONE;
-            float w0 = k0, w1 = k1, w2 = k2;  // direction of the traversal to start
             if (stage == ST_PEEL_DONE) {
                 C.c_peel[t] += nsteps;
-                const int pi = C.peel_i[t];
+                const int pk = C.peel_i[t], pi = pk & (PEEL_SCATTER - 1);
                 const InstrDev& I = sins[pi];
                 const float w = C.peel_w[t];
                 if (w > 0.f) {
@@ -532,8 +589,8 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                         }
                     }
                 }
-                C.peel_i[t] = pi + 1;
-                stage = pi + 1 < A.ninstr ? ST_PEEL : (C.peel_kind[t] ? ST_AFTER_SCATTER : ST_START_DEP);
+                C.peel_i[t] = pk + 1;
+                stage = pi + 1 < A.ninstr ? ST_PEEL : (pk & PEEL_SCATTER ? ST_AFTER_SCATTER : ST_START_DEP);
             } else if (stage == ST_DEPOSIT_DONE) {
                 C.c_dep[t] += nsteps;
                 // om = 1 - e^{-tau_path}: from expm1 for small tau, from 1 - exp for
@@ -560,36 +617,47 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                     C.ry[t] = r.y;
                     C.rz[t] = r.z;
                     par = -log1pf(-u01f(r.x) * om);
-                    need = M_LOCATE;
-                    found = false;
-                    last_dusty_end = 0.f;
+                    begin_search();
                     stage = ST_LOCATE_DONE;
+                    break;
                 }
             } else if (stage == ST_LOCATE_DONE) {
                 C.c_loc[t] += nsteps;
                 float l0 = C.xl0[t], l1 = C.xl1[t], l2 = C.xl2[t];
-                have_pc = found;
-                if (found) {
+                const int fm = C.f_m[t];
+                have_pc = fm >= 0;
+                int axis = -1;  // of the face through which the interaction cell was entered
+                float s = last_dusty_end;
+                if (have_pc) {
+                    s = C.f_s[t];
+                    const int fl = C.f_last[t];
                     if constexpr (OCT) {
                         pc0 = c0; pc1 = c1; pc2 = c2;
-                        pc_node = onode;
+                        pc_node = fm;
+                        axis = fl - 1;
                     } else {
-                        pc0 = (int)kf0 - (sf0 > 0); pc1 = (int)kf1 - (sf1 > 0); pc2 = (int)kf2 - (sf2 > 0);
+                        const unsigned row = (unsigned)fm / (unsigned)A.nx;
+                        pc0 = (int)((unsigned)fm - row * (unsigned)A.nx);
+                        pc2 = (int)(row / (unsigned)A.ny);
+                        pc1 = (int)(row - (unsigned)pc2 * (unsigned)A.ny);
+                        // a stride names its axis, except along axes of one cell, which
+                        // no crossing inside the grid runs along
+                        if (fl != 0) axis = (fl == st0 && A.nx > 1) ? 0 : ((fl == st1 && A.ny > 1) ? 1 : 2);
                     }
                 }
-                float s = found ? s_found : last_dusty_end;
-                if (found && last_axis >= 0) {
+                if (axis >= 0) {
                     // entry point of the interaction cell, snapped onto the exact face plane
-                    df_add_prod(x0, l0, tcur, k0);
-                    df_add_prod(x1, l1, tcur, k1);
-                    df_add_prod(x2, l2, tcur, k2);
+                    const float ft = C.f_t[t];
+                    df_add_prod(x0, l0, ft, k0);
+                    df_add_prod(x1, l1, ft, k1);
+                    df_add_prod(x2, l2, ft, k2);
                     const int e = OCT ? 1 << (OL - olev) : 1;
-                    const float ka = last_axis == 0 ? k0 : (last_axis == 1 ? k1 : k2);
-                    const int ca = last_axis == 0 ? pc0 : (last_axis == 1 ? pc1 : pc2);
-                    const int off = last_axis == 0 ? 0 : (last_axis == 1 ? A.nx + 1 : A.nx + 1 + A.ny + 1);
+                    const float ka = axis == 0 ? k0 : (axis == 1 ? k1 : k2);
+                    const int ca = axis == 0 ? pc0 : (axis == 1 ? pc1 : pc2);
+                    const int off = axis == 0 ? 0 : (axis == 1 ? A.nx + 1 : A.nx + 1 + A.ny + 1);
                     const float2 f = __ldg(A.faces + off + ca + (ka < 0.f ? e : 0));
-                    if (last_axis == 0) { x0 = f.x; l0 = f.y; }
-                    else if (last_axis == 1) { x1 = f.x; l1 = f.y; }
+                    if (axis == 0) { x0 = f.x; l0 = f.y; }
+                    else if (axis == 1) { x1 = f.x; l1 = f.y; }
                     else { x2 = f.x; l2 = f.y; }
                 }
                 df_add_prod(x0, l0, s, k0);
@@ -599,8 +667,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                 L = L * C.alb[t] * C.om[t];
                 C.nscat[t] = (int)C.ev[t];
                 if (L > 0.f && A.peel && A.ninstr > 0) {
-                    C.peel_kind[t] = 1;
-                    C.peel_i[t] = 0;
+                    C.peel_i[t] = PEEL_SCATTER;
                     stage = ST_PEEL;
                 } else {
                     stage = ST_AFTER_SCATTER;
@@ -626,7 +693,8 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
             }
 
             if (stage == ST_END_PACKET) {
-                C.c_scat[t] += (unsigned long long)C.nscat[t];
+                C.c_scat[t] += (unsigned)C.nscat[t];
+                if ((C.c_scat[t] | C.c_dep[t] | C.c_loc[t] | C.c_peel[t]) >> 30) flush_counters();
                 const float pe = C.p_esc[t], pa = C.p_abs[t], pr = C.p_res[t], pp = C.p_peel[t];
                 C.l_abs[t] += f2d(pa);
                 C.l_esc[t] += f2d(pe);
@@ -648,14 +716,13 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
             }
 
             if (stage == ST_NEW) {
-                if (C.q[t] >= C.q_end[t]) {
+                if (C.left[t] == 0) {
                     if (!A.persistent) {
-                        if (C.started[t]) { alive = false; break; }
-                        C.started[t] = 1;
-                        const unsigned long long q = A.q_base + (unsigned long long)blockIdx.x * blockDim.x + t;
-                        C.q[t] = q;
-                        C.q_end[t] = (q < A.q_base + A.q_count) ? q + 1 : q;
-                        if (C.q[t] >= C.q_end[t]) { alive = false; break; }
+                        const unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + t;
+                        if (started || q >= A.q_count) { alive = false; break; }
+                        started = true;
+                        C.q[t] = A.q_base + q;
+                        C.left[t] = 1;
                     } else {
                         const unsigned mask = __activemask();
                         const int lane = t & 31;
@@ -668,9 +735,10 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                         const unsigned long long q = base + (unsigned long long)rank * A.chunk;
                         if (q >= A.total) { alive = false; break; }
                         C.q[t] = q;
-                        C.q_end[t] = q + A.chunk < A.total ? q + A.chunk : A.total;
+                        C.left[t] = (unsigned)(A.total - q < (unsigned long long)A.chunk ? A.total - q : A.chunk);
                     }
                 }
+                C.left[t] -= 1;
                 const unsigned long long qq = C.q[t]++;
                 int ll = C.lam[t];
                 if (ll < 0 || qq < __ldg(A.offsets + ll) || qq >= __ldg(A.offsets + ll + 1)) {
@@ -679,14 +747,11 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                         const int mid = (a + b + 1) >> 1;
                         if (__ldg(A.offsets + mid) <= qq) a = mid; else b = mid - 1;
                     }
+                    flush_ledger();
                     ll = a;
                     C.lam[t] = ll;
                     C.alb[t] = __ldg(A.albedo_f + ll);
                     C.L0[t] = __ldg(A.L0_f + ll);
-                    if (C.led_lam[t] != ll) {
-                        flush_ledger();
-                        C.led_lam[t] = ll;
-                    }
                 }
                 lam = ll;
                 dep_base = A.absorbed + (size_t)lam * A.abs_ls;
@@ -775,17 +840,18 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                     sincospif(2.f * u01f(r.y), &sp, &cp);
                     k0 = st * cp; k1 = st * sp; k2 = mu;
                     if (A.peel && A.ninstr > 0) {
-                        C.peel_kind[t] = 0;
                         C.peel_i[t] = 0;
                         stage = ST_PEEL;
                     }
                 }
             }
 
+            float w0 = k0, w1 = k1, w2 = k2, i0 = 0.f, i1 = 0.f, i2 = 0.f;  // the traversal to start
             if (stage == ST_PEEL) {
-                const InstrDev& I = sins[C.peel_i[t]];
+                const int pk = C.peel_i[t];
+                const InstrDev& I = sins[pk & (PEEL_SCATTER - 1)];
                 float w = L;  // isotropic emission: phase factor 1
-                if (C.peel_kind[t]) {
+                if (pk & PEEL_SCATTER) {
                     const float mu = k0 * I.kobs_f[0] + k1 * I.kobs_f[1] + k2 * I.kobs_f[2];
                     w = L * hg_phase<float>(gg, mu);
                 }
@@ -795,15 +861,21 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                 if (w > 0.f) {
                     need = M_PEEL;
                     w0 = I.kobs_f[0]; w1 = I.kobs_f[1]; w2 = I.kobs_f[2];
+                    i0 = I.ikobs_f[0]; i1 = I.ikobs_f[1]; i2 = I.ikobs_f[2];
                 }
             } else if (stage == ST_START_DEP) {
                 C.ev[t] += 1;
                 par = L * (1.f - C.alb[t]);
                 need = M_DEPOSIT;
-                w0 = k0; w1 = k1; w2 = k2;
+                i0 = k0 != 0.f ? 1.f / k0 : 0.f;
+                i1 = k1 != 0.f ? 1.f / k1 : 0.f;
+                i2 = k2 != 0.f ? 1.f / k2 : 0.f;
                 stage = ST_DEPOSIT_DONE;
             }
-            if (need != M_NONE) begin(need, w0, w1, w2);
+            if (need != M_NONE) {
+                begin(need, w0, w1, w2, i0, i1, i2);
+                if (need == M_DEPOSIT) keep_start();
+            }
         } while (need == M_NONE);
     };
 
@@ -813,13 +885,16 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         const unsigned wm = __ballot_sync(0xffffffffu, !stepping && alive);
         if (!(sm | wm)) break;
         if (sm && (__popc(sm) >= step_min || !wm)) {
+            // the barrier makes the lanes meet after every crossing: without it
+            // the rare branches of a crossing leave parts of the warp running
+            // their crossings apart (15 of 26 stepping lanes at a time)
 #pragma unroll 1
             for (int r = 0; r < ROUND; ++r) {
-                if constexpr (OCT) {
-                    if (mode != M_NONE) step_oct();
-                } else {
-                    if (mode != M_NONE) step();
+                if (mode != M_NONE) {
+                    if constexpr (OCT) step_oct();
+                    else step();
                 }
+                __syncwarp();
             }
             continue;
         }
@@ -827,10 +902,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     }
 
     flush_ledger();
-    atomicAdd(A.counters + 0, C.c_scat[t]);
-    atomicAdd(A.counters + 1, C.c_dep[t]);
-    atomicAdd(A.counters + 2, C.c_loc[t]);
-    atomicAdd(A.counters + 3, C.c_peel[t]);
+    flush_counters();
 }
 
 }  // namespace
