@@ -72,6 +72,10 @@ struct TraceArgs {
     const float* kr32;
     const double* kr64;
     int nx, ny, nz;
+    // mixed form, Cartesian: the traversal's cell order (kr32 and, where the
+    // deposits go to scratch, the absorbed table follow it): index strides of the
+    // axes, the fastest axis, the extents of the fastest and the middle one
+    int cst[3], fast, n_f, n_m;
     long long ncell;                       // nx*ny*nz, or the number of octree leaves
     double lo[3], d[3], hi[3];
     int nlambda;
@@ -134,10 +138,21 @@ size_t trace_smem_bytes(int ninstr, int block);
 cudaError_t launch_trace_mixed(const TraceArgs& a, int block, int grid, cudaStream_t s);
 cudaError_t trace_mixed_occupancy(int block, int* blocks_per_sm, bool octree);
 size_t trace_mixed_smem_bytes(int ninstr, int block);
-// out[cell][lambda] (+)= in[lambda][cell]: the absorbed table from the trace's
-// wavelength-major accumulation to the API's cell-major layout
+// The order in which the mixed form's Cartesian traversals number the cells:
+// fast = the axis along which consecutive numbers run (0: the API's order).
+struct CellOrder {
+    int n[3];       // cells per axis
+    int fast;
+    int st[3];      // stride of each axis
+    int n_f, n_m;   // extents of the fastest and the middle axis
+};
+CellOrder cell_order(int nx, int ny, int nz, int fast);
+// out[cell][lambda] (+)= in[lambda][number of the cell in order o]: the absorbed
+// table from the trace's wavelength-major accumulation to the API's layout
 cudaError_t launch_transpose_absorbed(const double* in, double* out, long long ncell, int nlambda, bool add,
-                                      cudaStream_t s);
+                                      const CellOrder& o, cudaStream_t s);
+// out[number of the cell in order o] = in[cell]
+cudaError_t launch_reorder_density(const float* in, float* out, const CellOrder& o, cudaStream_t s);
 // sed[q][lambda] += sign * (sum over the pixels of images_q) + oof[q][lambda] (oof may be NULL)
 cudaError_t launch_sed_finalize(const double* images, const double* oof, double* sed, int ninstr,
                                 const int* npx_host, int nlambda, double sign, cudaStream_t s);
@@ -223,7 +238,9 @@ struct skirt_grid_s {
     long long ncell = 0;
     double bbox[6] = {0, 0, 0, 0, 0, 0};
     float* kr32 = nullptr;
+    float* kr_fast = nullptr;  // kr32 in the traversal's cell order, if that is not the API's
     double* kr64 = nullptr;
+    int fast = 0;              // the traversal order's fastest axis
     float2* faces = nullptr;  // exact face planes as (hi, lo) FP32 pairs, x then y then z
     skirt::DevBuf scratch;  // per-call tables, accumulators, work queue
     skirt::DevBuf stage;    // device images of host outputs

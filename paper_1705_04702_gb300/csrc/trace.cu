@@ -594,12 +594,36 @@ cudaError_t trace_occupancy(int precision, int block, int* blocks_per_sm, bool o
                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_kernel<double, false>, block, smem);
 }
 
+CellOrder cell_order(int nx, int ny, int nz, int fast)
+{
+    CellOrder o;
+    o.n[0] = nx; o.n[1] = ny; o.n[2] = nz;
+    o.fast = fast;
+    const int mid = fast == 0 ? 1 : 0, slow = fast == 2 ? 1 : 2;
+    o.n_f = o.n[fast];
+    o.n_m = o.n[mid];
+    o.st[fast] = 1;
+    o.st[mid] = o.n_f;
+    o.st[slow] = (int)((long long)o.n_f * o.n_m);  // below the number of cells (< 2^31) if any axis is longer than one cell
+    return o;
+}
+
 namespace {
+
+// the API's cell number of number c in order o
+__device__ __forceinline__ unsigned api_cell(unsigned c, const CellOrder& o)
+{
+    if (o.fast == 0) return c;
+    const unsigned row = c / (unsigned)o.n_f, jf = c - row * (unsigned)o.n_f;
+    const unsigned js = row / (unsigned)o.n_m, jm = row - js * (unsigned)o.n_m;
+    const unsigned y = o.fast == 1 ? jf : js, z = o.fast == 2 ? jf : js;  // the middle axis is x
+    return (z * (unsigned)o.n[1] + y) * (unsigned)o.n[0] + jm;
+}
 
 // out[c][l] (+)= in[l][c], 32 x 32 tiles through shared memory (one padding
 // column): coalesced reads along the cells and writes along the wavelengths.
 __global__ void transpose_absorbed_kernel(const double* __restrict__ in, double* __restrict__ out, long long ncell,
-                                          int nl, int add)
+                                          int nl, int add, const CellOrder o)
 {
     __shared__ double tile[32][33];
     const long long c0 = (long long)blockIdx.x * 32;
@@ -614,21 +638,81 @@ __global__ void transpose_absorbed_kernel(const double* __restrict__ in, double*
         const long long c = c0 + k;
         const int l = l0 + threadIdx.x;
         if (c < ncell && l < nl) {
-            double* o = out + (size_t)c * nl + l;
-            *o = add ? *o + tile[threadIdx.x][k] : tile[threadIdx.x][k];
+            const long long m = o.fast ? (long long)api_cell((unsigned)c, o) : c;
+            double* p = out + (size_t)m * nl + l;
+            *p = add ? *p + tile[threadIdx.x][k] : tile[threadIdx.x][k];
         }
     }
+}
+
+// Reordering between the API's cell order (x fastest) and order o (axis o.fast
+// fastest), in 32 x 32 tiles of (x, fast axis) at one position of the third
+// axis: coalesced on both sides.  TO_API: out[api][lambda] (+)=
+// in[lambda][o], wavelength blockIdx.y of nl; otherwise out[o] = in[api].
+template <bool TO_API, typename T>
+__global__ void reorder_cells_kernel(const T* __restrict__ in, T* __restrict__ out, const CellOrder o,
+                                     long long ncell, int nl, int add)
+{
+    __shared__ T tile[32][33];
+    const int fa = o.fast, ta = 3 - fa;  // the fastest axis (1 or 2) and the third one
+    const int nx = o.n[0], nf = o.n[fa], nt = o.n[ta];
+    const size_t api_f = fa == 1 ? (size_t)nx : (size_t)nx * o.n[1], api_t = fa == 1 ? (size_t)nx * o.n[1] : (size_t)nx;
+    const size_t o_x = (size_t)o.st[0], o_t = (size_t)o.st[ta];
+    const long long tx = (nx + 31) / 32, tf = (nf + 31) / 32, total = tx * tf * nt;
+    const int l = blockIdx.y;
+    for (long long b = blockIdx.x; b < total; b += gridDim.x) {
+        const int x0 = (int)(b % tx) * 32, f0 = (int)((b / tx) % tf) * 32, it = (int)(b / (tx * tf));
+        for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+            const int x = x0 + (TO_API ? k : (int)threadIdx.x), f = f0 + (TO_API ? (int)threadIdx.x : k);
+            if (x < nx && f < nf)
+                tile[k][threadIdx.x] = TO_API ? in[(size_t)l * ncell + f + x * o_x + it * o_t]
+                                              : in[x + f * api_f + it * api_t];
+        }
+        __syncthreads();
+        for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+            const int x = x0 + (TO_API ? (int)threadIdx.x : k), f = f0 + (TO_API ? k : (int)threadIdx.x);
+            if (x < nx && f < nf) {
+                const T v = tile[threadIdx.x][k];
+                if constexpr (TO_API) {
+                    T* p = out + (x + f * api_f + it * api_t) * nl + l;
+                    *p = add ? *p + v : v;
+                } else {
+                    out[f + x * o_x + it * o_t] = v;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+int reorder_blocks(const CellOrder& o)
+{
+    const long long b = (long long)((o.n[0] + 31) / 32) * ((o.n[o.fast] + 31) / 32) * o.n[3 - o.fast];
+    return (int)(b < 65536 ? b : 65536);
 }
 
 }  // namespace
 
 cudaError_t launch_transpose_absorbed(const double* in, double* out, long long ncell, int nlambda, bool add,
-                                      cudaStream_t s)
+                                      const CellOrder& o, cudaStream_t s)
 {
+    if (o.fast != 0 && nlambda < 4) {
+        // too few wavelengths for the tiles below: 32-byte runs of the output from four on
+        reorder_cells_kernel<true, double><<<dim3(reorder_blocks(o), nlambda), dim3(32, 8), 0, s>>>(in, out, o, ncell,
+                                                                                                    nlambda, add ? 1 : 0);
+        return cudaGetLastError();
+    }
     const long long bx = (ncell + 31) / 32;
     if (bx > 0x7fffffffLL) return cudaErrorInvalidValue;
     transpose_absorbed_kernel<<<dim3((unsigned)bx, (unsigned)((nlambda + 31) / 32)), dim3(32, 8), 0, s>>>(
-        in, out, ncell, nlambda, add ? 1 : 0);
+        in, out, ncell, nlambda, add ? 1 : 0, o);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reorder_density(const float* in, float* out, const CellOrder& o, cudaStream_t s)
+{
+    reorder_cells_kernel<false, float><<<reorder_blocks(o), dim3(32, 8), 0, s>>>(
+        in, out, o, (long long)o.n[0] * o.n[1] * o.n[2], 1, 0);
     return cudaGetLastError();
 }
 

@@ -309,9 +309,9 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         } else {
             kf0 = (KF)n0; kf1 = (KF)n1; kf2 = (KF)n2;
             sf0 = (KF)g0; sf1 = (KF)g1; sf2 = (KF)g2;
-            st0 = g0;
-            st1 = g1 * A.nx;
-            st2 = g2 * (A.nx * A.ny);
+            st0 = g0 * A.cst[0];
+            st1 = g1 * A.cst[1];
+            st2 = g2 * A.cst[2];
             // the distance to each axis's last face by the crossing's own
             // formula: the crossing that leaves the grid lies at one of them
             const int m0 = g0 > 0 ? A.nx : 0, m1 = g1 > 0 ? A.ny : 0, m2 = g2 > 0 ? A.nz : 0;
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
             const float u1 = n1 == m1 ? tn1 : face_t((float)m1, A.d_f[1], A.lo_f[1], x1, iv1);
             const float u2 = n2 == m2 ? tn2 : face_t((float)m2, A.d_f[2], A.lo_f[2], x2, iv2);
             t_end = fminf(g0 ? u0 : INF, fminf(g1 ? u1 : INF, g2 ? u2 : INF));
-            cur_m = (pc2 * A.ny + pc1) * A.nx + pc0;
+            cur_m = pc0 * A.cst[0] + pc1 * A.cst[1] + pc2 * A.cst[2];
             kr_cur = __ldg(kr + cur_m);
         }
     };
@@ -636,10 +636,12 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                         pc_node = fm;
                         axis = fl - 1;
                     } else {
-                        const unsigned row = (unsigned)fm / (unsigned)A.nx;
-                        pc0 = (int)((unsigned)fm - row * (unsigned)A.nx);
-                        pc2 = (int)(row / (unsigned)A.ny);
-                        pc1 = (int)(row - (unsigned)pc2 * (unsigned)A.ny);
+                        const unsigned row = (unsigned)fm / (unsigned)A.n_f, is = row / (unsigned)A.n_m;
+                        const int jf = (int)((unsigned)fm - row * (unsigned)A.n_f);
+                        const int jm = (int)(row - is * (unsigned)A.n_m);
+                        pc0 = A.fast == 0 ? jf : jm;
+                        pc1 = A.fast == 1 ? jf : (A.fast == 0 ? jm : (int)is);
+                        pc2 = A.fast == 2 ? jf : (int)is;
                         // a stride names its axis, except along axes of one cell, which
                         // no crossing inside the grid runs along
                         if (fl != 0) axis = (fl == st0 && A.nx > 1) ? 0 : ((fl == st1 && A.ny > 1) ? 1 : 2);

@@ -58,3 +58,40 @@ def test_beams_leave_the_grid_where_the_oracle_does(S, oracle_lib, pos, directio
     g = S.run_problem(prob, nrec=3)
     np.testing.assert_allclose(g["absorbed"].cpu().numpy(), ref["absorbed"], rtol=0, atol=1e-5)
     np.testing.assert_allclose(g["records"].cpu().numpy()[..., :4], ref["records"][..., :4], rtol=0, atol=1e-5)
+
+
+@pytest.mark.parametrize("nxyz,ext", [
+    ((33, 5, 41), (4.0, 2.0, 0.5)),     # z cells the smallest: z runs fastest
+    ((7, 40, 3), (2.0, 1.0, 3.0)),      # y cells
+    ((1, 70, 9), (1.0, 1.0, 3.0)),      # y cells, one cell along x
+    ((65, 3, 1), (6.5, 0.1, 3.0)),      # y cells, one cell along z
+    ((64, 32, 33), (2.0, 2.0, 0.4)),
+])
+@pytest.mark.parametrize("nl", [1, 3, 4, 37])
+def test_cell_orders_give_the_api_tables(S, nxyz, ext, nl):
+    """Grids whose thinnest cells lie along y or z are traversed with that
+    axis fastest.  The tables come back in the API's order: the FP64 form,
+    which never reorders, gives them up to the <= 0.1% of packets whose FP32
+    histories differ (each moves its luminosity once on either side: L1 2e-3),
+    and an accumulating second call doubles them."""
+    import torch
+    nx, ny, nz = nxyz
+    x = (np.arange(nx) + 0.5) / nx
+    y = (np.arange(ny) + 0.5) / ny
+    z = (np.arange(nz) + 0.5) / nz
+    kr = (0.5 + 2.0 * x[None, None, :] + y[None, :, None] ** 2 + 0.3 * z[:, None, None]).astype(np.float32)
+    ex, ey, ez = ext
+    grid = W.Grid(nx, ny, nz, (0.0, ex, -ey, 0.0, 0.0, ez), kr)
+    wl = W.single_wavelength() if nl == 1 else W.powerlaw_wavelengths(nl, 0.3, 3.0)
+    prob = W.Problem("order", grid, W.Source(W.SRC_POINT, (0.31 * ex, -0.43 * ey, 0.57 * ez)), wl,
+                     np.full(nl, 3000, dtype=np.uint64), [W.Instrument(100.0, 40.0, 20.0, 10.0, 8)], seed=11)
+    a = S.run_problem(prob, precision=S.PREC_MIXED)
+    b = S.run_problem(prob, precision=S.PREC_FP64)
+    ta, tb = a["absorbed"].cpu().numpy(), b["absorbed"].cpu().numpy()
+    assert np.abs(ta - tb).sum() <= 2e-3 * tb.sum()
+    g = S.Grid(grid)
+    outs = (torch.zeros_like(a["absorbed"]), torch.zeros_like(a["images_flat"]), torch.zeros_like(a["sed"]))
+    S.run_problem(prob, grid=g, outputs=outs)
+    S.run_problem(prob, grid=g, outputs=outs, accumulate=True, use_graph=True)
+    np.testing.assert_allclose(outs[0].cpu().numpy(), 2.0 * ta, rtol=1e-12)
+    g.close()
