@@ -602,7 +602,17 @@ extern "C" int skirt_trace(skirt_grid_t g, const skirt_source* src, const skirt_
         if (bps < 1) bps = 1;
     }
     const int pgrid = g->sm_count * bps;
+    // Packets a thread takes per queue refill: what was asked for, but no more than
+    // leaves every thread eight refills.  Fewer starve the launch's end, or, below a
+    // refill per thread, most of the launch: 1e5 packets in the sphere took 1.68 ms by
+    // fours and take 1.00 ms one by one, 3e5 on an octree 12.6 and 7.8 ms; where there
+    // is work for many refills, single packets cost more in queue traffic (2e6 dust
+    // packets 14.9 ms against 13.8 ms by twos).
     A.chunk = opts->chunk > 0 ? opts->chunk : 4;
+    {
+        const unsigned long long fair = P.total / (8ull * (unsigned long long)pgrid * (unsigned long long)block);
+        if ((unsigned long long)A.chunk > fair) A.chunk = fair > 0 ? (int)fair : 1;
+    }
     if (opts->precision == SKIRT_PREC_FP64 && trace_smem_bytes(A.ninstr, block) > 48 * 1024)
         return fail(SKIRT_ERR_INVALID_ARG, "block too large for the shared-memory budget");
 
