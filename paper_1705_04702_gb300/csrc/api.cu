@@ -267,7 +267,7 @@ extern "C" int skirt_emission_totals(skirt_grid_t g, const double* emission, int
     if (!is_device_ptr(emission)) return fail(SKIRT_ERR_INVALID_ARG, "emission must be device memory");
     const std::vector<uint64_t> none((size_t)nlambda, 0);
     std::vector<double> t;
-    if (int r = build_dust_cdf(g, emission, nlambda, none.data(), (cudaStream_t)stream, &t)) return r;
+    if (int r = build_dust_cdf(g, emission, nlambda, none.data(), (cudaStream_t)stream, &t, false)) return r;
     std::memcpy(totals, t.data(), sizeof(double) * (size_t)nlambda);
     return SKIRT_OK;
 }
@@ -548,6 +548,8 @@ extern "C" int skirt_trace(skirt_grid_t g, const skirt_source* src, const skirt_
     A.h_R = src->h_R;
     A.h_z = src->h_z;
     A.cdf = d_cdf;
+    A.cdf_off = d_cdf ? (const double*)g->cdf_aux.p : nullptr;
+    A.dust_tiles = (g->ncell + DUST_TILE - 1) / DUST_TILE;
     A.ninstr = peel ? ninstr : 0;
     A.ins = (const InstrDev*)(dp + L.ins);
     // With more than one wavelength the packets deposit into a wavelength-major

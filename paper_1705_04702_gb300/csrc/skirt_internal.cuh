@@ -68,6 +68,8 @@ constexpr int OCT_LEAF_BITS = 27;
 __host__ __device__ __forceinline__ int oct_leaf_index(int ref) { return (~ref) & ((1 << OCT_LEAF_BITS) - 1); }
 __host__ __device__ __forceinline__ int oct_leaf_level(int ref) { return (~ref) >> OCT_LEAF_BITS; }
 
+constexpr int DUST_TILE = 256;  // cells per tile of the dust source's cumulative distribution
+
 struct TraceArgs {
     const float* kr32;
     const double* kr64;
@@ -97,7 +99,9 @@ struct TraceArgs {
     unsigned long long total;
     int src_kind;
     double src_pos[3], src_dir[3], h_R, h_z;
-    const double* cdf;                     // dust source: [nlambda][ncell] cumulative, normalised
+    const double* cdf;                     // dust source: [nlambda][ncell] running sums within tiles of DUST_TILE cells
+    const double* cdf_off;                 // [nlambda][dust_tiles + 1] offsets of the tiles, then the total
+    long long dust_tiles;
     int ninstr;
     const InstrDev* ins;
     double* absorbed;                      // element (cell, lambda) at cell * abs_cs + lambda * abs_ls
@@ -244,8 +248,8 @@ struct skirt_grid_s {
     float2* faces = nullptr;  // exact face planes as (hi, lo) FP32 pairs, x then y then z
     skirt::DevBuf scratch;  // per-call tables, accumulators, work queue
     skirt::DevBuf stage;    // device images of host outputs
-    skirt::DevBuf cdf;      // dust source: [nlambda][ncell] cumulative distributions
-    skirt::DevBuf cdf_aux;  // dust source: tile sums and totals
+    skirt::DevBuf cdf;      // dust source: [nlambda][ncell] running sums within tiles
+    skirt::DevBuf cdf_aux;  // dust source: tile offsets, totals and tile sums
     skirt::DevBuf abs_lmajor;  // wavelength-major absorbed table of the current call
     int oct_levels = 0;              // octree grid: finest lattice 2^oct_levels per axis
     long long oct_nnode = 0;
@@ -278,9 +282,10 @@ int launch_exact_emission(const double* absorbed, int n_in, const double* w_dev,
                           cudaStream_t s, const double* absorbed2 = nullptr, int n2 = 0,
                           const double* w2_dev = nullptr);
 // dust_source.cu: per-wavelength cumulative distribution of emission[cell][lambda]
-// over the cells, normalised to 1, into grid->cdf; the per-wavelength totals
-// into *totals_out (may be NULL).  INVALID_ARG when a wavelength with packets
-// has no (or non-finite / negative) emission.
+// over the cells into grid->cdf (running sums within tiles) and grid->cdf_aux
+// (tile offsets); the per-wavelength totals into *totals_out (may be NULL), and
+// nothing but them when the distribution is not wanted.  INVALID_ARG when a
+// wavelength with packets has no (or non-finite / negative) emission.
 int build_dust_cdf(skirt_grid_s* g, const double* emission, int nlambda, const uint64_t* npk, cudaStream_t s,
-                   std::vector<double>* totals_out);
+                   std::vector<double>* totals_out, bool rows_wanted = true);
 }  // namespace skirt

@@ -347,14 +347,7 @@ __global__ void __launch_bounds__(512) trace_kernel(const TraceArgs A)
                 }
             } else if (A.src_kind == SKIRT_SRC_DUST) {
                 const uint4 r = draw(0u, 0u);
-                const long long ncell = A.ncell;
-                const double* cdf = A.cdf + (size_t)lam * ncell;
-                const double u0 = (double)u01f(r.x);
-                long long a = 0, b = ncell - 1;  // first cell with cdf > u0
-                while (a < b) {
-                    const long long mid = (a + b) >> 1;
-                    if (__ldg(cdf + mid) > u0) b = mid; else a = mid + 1;
-                }
+                const long long a = dust_cell(A, lam, (double)u01f(r.x));
                 if (OCT) {
                     // uniform point in the leaf's box
                     const int4 lf = __ldg(&A.oct_leaf[a]);

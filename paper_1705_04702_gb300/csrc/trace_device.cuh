@@ -59,6 +59,34 @@ __device__ __forceinline__ void hg_rotate(R& k0, R& k1, R& k2, R mu, R sp, R cp)
     k2 = n2;
 }
 
+// The dust-source cell of uniform number u (0 < u < 1) at wavelength lam: the
+// first whose cumulative emission exceeds u times the total, found by bisecting
+// the tiles' offsets and then the running sums of one tile.  All values are
+// non-negative, so they compare as integers, off the FP64 pipe.
+__device__ __forceinline__ long long dust_cell(const TraceArgs& A, int lam, double u)
+{
+    const double* off = A.cdf_off + (size_t)lam * (A.dust_tiles + 1);
+    const double target = u * __ldg(off + A.dust_tiles);
+    long long key = __double_as_longlong(target);
+    long long a = 0, b = A.dust_tiles - 1;  // first tile that ends beyond the target
+    while (a < b) {
+        const long long mid = (a + b) >> 1;
+        if (__double_as_longlong(__ldg(off + mid + 1)) > key) b = mid; else a = mid + 1;
+    }
+    const long long m0 = a * DUST_TILE;
+    const double* row = A.cdf + (size_t)lam * A.ncell + m0;
+    int lo = 0, hi = (int)(A.ncell - m0 < DUST_TILE ? A.ncell - m0 : DUST_TILE) - 1;
+    key = __double_as_longlong(target - __ldg(off + a));
+    // where rounding leaves nothing of the tile beyond the rest, its last emitting cell
+    const long long last = __double_as_longlong(__ldg(row + hi));
+    if (last <= key) key = last - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__double_as_longlong(__ldg(row + mid)) > key) hi = mid; else lo = mid + 1;
+    }
+    return m0 + lo;
+}
+
 // Cell index along one axis: floor((x - lo) / d) clamped to [0, n-1].
 template <typename R>
 __device__ __forceinline__ int cell_index(R x, R lo, R d, int n)
