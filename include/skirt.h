@@ -444,7 +444,7 @@ int skirt_dust_emission_pair(const double* absorbed_a, long long ncell, int n_a,
  * Same result as skirt_dust_emission in SKIRT_EMIT_EXACT mode, same argument
  * meaning (all arrays device memory, lambda_in host, temperature may be NULL),
  * no statistics.  Its only working table, the absorption shares of the input
- * wavelengths, lives in a fixed device array of 3 x 4096 doubles (96 KiB) that
+ * wavelengths, lives in a fixed device array of 8 x 4096 doubles (256 KiB) that
  * every device loading the library holds until the process exits: n_in above
  * 4096 is rejected with SKIRT_ERR_INVALID_ARG.  The first call on a device
  * looks up the array's device address (once per device, with that device

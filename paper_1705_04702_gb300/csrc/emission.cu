@@ -5,14 +5,16 @@
 //  * band_features_kernel  32 log-spaced band sums per unit mass (log10) and
 //                          the total absorbed power, one cell per lane
 //  * exact_kernel          equilibrium temperatures of three grain
-//                          populations by bracketed Newton on ln T (FP64
-//                          per population, Planck terms in double-float),
-//                          then the energy-conserving emission spectrum
+//                          populations by bracketed Newton on ln T (powers
+//                          in 64-bit integers, FP64 per population, Planck
+//                          terms in double-float), then the energy-conserving
+//                          emission spectrum
 // and skirt_dust_emission, which runs either the exact solver on every cell
 // or the MLP surrogate (mlp.cu) with the exact solver as the fallback for
 // cells outside the network's training hull.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -34,26 +36,28 @@ const double BETA[NPOP] = {1.5, 2.0, 2.0};
 // h c / k_B in micron kelvin from the exact SI constants
 const double HCK_UM = 6.62607015e-34 * 299792458.0 / 1.380649e-23 * 1e6;
 
-__constant__ double c_a[NOUT];          // hc/(k lambda_l)
-__constant__ double c_K[NPOP][NOUT];    // W_l kappa_i(lambda_l) lambda_l^-5
 __constant__ double c_lnc[NPOP];        // ln c_i = -ln G_i(30 K)
+__constant__ double c_Gref[NPOP];       // 1 / c_i
 __constant__ double c_lnG_lo[NPOP];     // ln G_i(3 K)
 __constant__ double c_lnG_hi[NPOP];     // ln G_i(2000 K)
-__constant__ double c_beta[NPOP];
-// ln G_i and d ln G_i / d ln T at NTAB log-spaced temperatures over [T_LO,
-// T_HI]: the starting point of the Newton solve (read through the L1 path);
-// 4096 intervals, so that every 2^k-th point also spans [T_LO, T_HI]
-constexpr int NTAB = 4097;
-__device__ double g_lnG_tab[NPOP][NTAB];
-__device__ double g_dlnG_tab[NPOP][NTAB];
-// (a_l, K_il) of slot s = i * NOUT + l as double-float pairs (the exact solve's terms)
+__constant__ double c_h[NPOP], c_inv_h[NPOP];  // spacing of the table below in ln G_i, and its reciprocal
+// 1/T and d(1/T)/d ln G_i times the spacing at NTAB values of ln G_i equally
+// spaced over [ln G_i(3 K), ln G_i(2000 K)]: the start of the Newton solve (read
+// through the L1 path); 8192 intervals, so that every 2^k-th point also spans
+// the range
+constexpr int NTAB = 8193;
+__device__ double2 g_invT_tab[NPOP][NTAB];
+// (256/ln 2 a_l, K_il) of slot s = i * NOUT + l as double-float pairs (the exact
+// solve's terms), and the exponential's table
 __device__ float4 g_slot[NPOP * NOUT];
+__device__ float2 g_exp[DF_EXP_N];
 
 struct HostModel {
     double lam[NOUT], W[NOUT], a[NOUT], K[NPOP][NOUT];
-    double lnc[NPOP], lnG_lo[NPOP], lnG_hi[NPOP];
-    double tab[NPOP][NTAB], dtab[NPOP][NTAB];
-    float slot[NPOP * NOUT][4];  // (a_l, K_il) of slot i * NOUT + l as double-float pairs
+    double lnc[NPOP], Gref[NPOP], lnG_lo[NPOP], lnG_hi[NPOP], h[NPOP], inv_h[NPOP];
+    double tab[NPOP][NTAB][2];
+    float slot[NPOP * NOUT][4];
+    float exp_tab[DF_EXP_N][2];
 };
 
 // v = hi + lo with hi = v rounded to binary32, lo = the rest rounded
@@ -63,11 +67,20 @@ void split_float(double v, float& hi, float& lo)
     lo = (float)(v - (double)hi);
 }
 
-double host_G(const HostModel& h, int i, double T)
+// ln G_i at T = e^y and its derivative by y
+double host_lnG(const HostModel& h, int i, double y, double& slope)
 {
-    double g = 0.0;
-    for (int l = 0; l < NOUT; ++l) g += h.K[i][l] / std::expm1(h.a[l] / T);
-    return g;
+    const double T = std::exp(y);
+    double g = 0.0, d = 0.0;
+    for (int l = 0; l < NOUT; ++l) {
+        const double x = h.a[l] / T;
+        if (x > 700.0) continue;
+        const double q = 1.0 / std::expm1(x);
+        g += h.K[i][l] * q;
+        d += h.K[i][l] * q * x * (1.0 + q);
+    }
+    slope = d / g;
+    return std::log(g);
 }
 
 const HostModel& host_model()
@@ -86,47 +99,82 @@ const HostModel& host_model()
                 h.K[i][l] = h.W[l] * std::pow(h.lam[l] / 100.0, -BETA[i]) * std::pow(h.lam[l], -5.0);
         }
         for (int i = 0; i < NPOP; ++i) {
-            h.lnc[i] = -std::log(host_G(h, i, T_REF));
-            h.lnG_lo[i] = std::log(host_G(h, i, T_LO));
-            h.lnG_hi[i] = std::log(host_G(h, i, T_HI));
+            if (i > 0 && BETA[i] == BETA[i - 1]) {  // the same G
+                h.lnc[i] = h.lnc[i - 1];
+                h.Gref[i] = h.Gref[i - 1];
+                h.lnG_lo[i] = h.lnG_lo[i - 1];
+                h.lnG_hi[i] = h.lnG_hi[i - 1];
+                h.h[i] = h.h[i - 1];
+                h.inv_h[i] = h.inv_h[i - 1];
+                std::memcpy(h.tab[i], h.tab[i - 1], sizeof h.tab[i]);
+                continue;
+            }
+            double slope;
+            h.lnc[i] = -host_lnG(h, i, std::log(T_REF), slope);
+            h.Gref[i] = std::exp(-h.lnc[i]);
+            h.lnG_hi[i] = host_lnG(h, i, std::log(T_HI), slope);
+            h.lnG_lo[i] = host_lnG(h, i, std::log(T_LO), slope);
+            h.h[i] = (h.lnG_hi[i] - h.lnG_lo[i]) / (NTAB - 1);
+            h.inv_h[i] = 1.0 / h.h[i];
+            // ln T of every point by Newton from the extrapolated previous ones
+            double y = std::log(T_LO), y1 = y, y2 = y;
             for (int k = 0; k < NTAB; ++k) {
-                const double T = std::exp(std::log(T_LO) + (std::log(T_HI) - std::log(T_LO)) * k / (NTAB - 1));
-                double g = 0.0, d = 0.0;
-                for (int l = 0; l < NOUT; ++l) {
-                    const double x = h.a[l] / T;
-                    if (x > 700.0) continue;
-                    const double q = 1.0 / std::expm1(x);
-                    g += h.K[i][l] * q;
-                    d += h.K[i][l] * q * x * (1.0 + q);
+                const double t = h.lnG_lo[i] + k * h.h[i];
+                if (k == 1) y = y1 + h.h[i] / slope;
+                if (k > 1) y = 2.0 * y1 - y2;
+                for (int it = 0; it < 8; ++it) {
+                    const double step = (t - host_lnG(h, i, y, slope)) / slope;
+                    y += step;
+                    // quadratic convergence: the next step would be below 1e-16
+                    if (std::fabs(step) < 1e-8) break;
                 }
-                h.tab[i][k] = std::log(g);
-                h.dtab[i][k] = d / g;
+                y2 = y1;
+                y1 = y;
+                h.tab[i][k][0] = std::exp(-y);
+                h.tab[i][k][1] = -std::exp(-y) / slope * h.h[i];
             }
         }
         for (int i = 0; i < NPOP; ++i)
             for (int l = 0; l < NOUT; ++l) {
                 float* q = h.slot[i * NOUT + l];
-                split_float(h.a[l], q[0], q[1]);
+                split_float(h.a[l] * DF_Z_PER_X, q[0], q[1]);
                 split_float(h.K[i][l], q[2], q[3]);
             }
+        for (int j = 0; j < DF_EXP_N; ++j) {
+            const dfl::df2 v = dfl::exp_table_entry(j);
+            h.exp_tab[j][0] = v.hi;
+            h.exp_tab[j][1] = v.lo;
+        }
         ready = true;
     }
     return h;
 }
 
-cudaError_t upload_model(cudaStream_t s)
+// The model's tables on the current device: constants of the library, put there
+// once per device (nine copies from pageable memory took 60 us of every call).
+cudaError_t upload_model()
 {
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
     const HostModel& h = host_model();
-    cudaError_t e;
-    if ((e = cudaMemcpyToSymbolAsync(c_a, h.a, sizeof h.a, 0, cudaMemcpyHostToDevice, s))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(c_K, h.K, sizeof h.K, 0, cudaMemcpyHostToDevice, s))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(c_lnc, h.lnc, sizeof h.lnc, 0, cudaMemcpyHostToDevice, s))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(c_lnG_lo, h.lnG_lo, sizeof h.lnG_lo, 0, cudaMemcpyHostToDevice, s))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(c_lnG_hi, h.lnG_hi, sizeof h.lnG_hi, 0, cudaMemcpyHostToDevice, s))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(g_lnG_tab, h.tab, sizeof h.tab, 0, cudaMemcpyHostToDevice, s))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(g_dlnG_tab, h.dtab, sizeof h.dtab, 0, cudaMemcpyHostToDevice, s))) return e;
-    if ((e = cudaMemcpyToSymbolAsync(g_slot, h.slot, sizeof h.slot, 0, cudaMemcpyHostToDevice, s))) return e;
-    return cudaMemcpyToSymbolAsync(c_beta, BETA, sizeof BETA, 0, cudaMemcpyHostToDevice, s);
+    if ((e = cudaMemcpyToSymbol(c_lnc, h.lnc, sizeof h.lnc))) return e;
+    if ((e = cudaMemcpyToSymbol(c_Gref, h.Gref, sizeof h.Gref))) return e;
+    if ((e = cudaMemcpyToSymbol(c_lnG_lo, h.lnG_lo, sizeof h.lnG_lo))) return e;
+    if ((e = cudaMemcpyToSymbol(c_lnG_hi, h.lnG_hi, sizeof h.lnG_hi))) return e;
+    if ((e = cudaMemcpyToSymbol(c_h, h.h, sizeof h.h))) return e;
+    if ((e = cudaMemcpyToSymbol(c_inv_h, h.inv_h, sizeof h.inv_h))) return e;
+    if ((e = cudaMemcpyToSymbol(g_invT_tab, h.tab, sizeof h.tab))) return e;
+    if ((e = cudaMemcpyToSymbol(g_slot, h.slot, sizeof h.slot))) return e;
+    if ((e = cudaMemcpyToSymbol(g_exp, h.exp_tab, sizeof h.exp_tab))) return e;
+    // pageable copies may return before they have arrived; other streams use the tables next
+    if ((e = cudaStreamSynchronize(cudaStreamLegacy))) return e;
+    if (dev >= 0 && dev < 64) done[dev] = true;
+    return cudaSuccess;
 }
 
 // vol: the cell volume; on an octree (leaf != NULL) the finest-lattice cell
@@ -269,35 +317,52 @@ int band_blocks(long long ncell)
     return (int)(b < 1 ? 1 : b);
 }
 
-// The exact solve, one warp per batch of EX_BATCH rows.
+// The exact solve, one warp per batch of up to EX_BATCH rows.
 //
 // Per row and population i the solve needs P_i = sum_j w_ij A_j, the target
-// ln G_i(T_i) = ln(P_i / M) - ln c_i, a start and bracket for T_i, one
-// evaluation of G_i(T_i) = sum_l K_il / expm1(a_l / T_i) with T dG_i/dT, and
-// a Newton test; the emission row is e_l = sum_i (P_i / G_i) K_il / expm1(a_l / T_i).
+// ln G_i(T_i) = ln(P_i / M) - ln c_i, a start for T_i, one evaluation of
+// G_i(T_i) = sum_l K_il / expm1(a_l / T_i), and a Newton test;
+// the emission row is e_l = sum_i (P_i / G_i) K_il / expm1(a_l / T_i).
 //
-//  * Per population (FP64, lane 3r + i holds row r's population i, so the
-//    EX_BATCH rows share each FP64 instruction): the target, the clamp to
-//    3 or 2000 K, the table start, T_i, and after the evaluation the Newton
-//    test on ln T.
+// An FP64 warp instruction holds the SM's FP64 pipe for as long as 78 other
+// instructions take to issue, so FP64 does only what has to be FP64:
+//
+//  * The powers are sums in 64-bit integers.  The inputs of a block of 256
+//    columns become fixed-point numbers relative to the largest (59 bits), the
+//    shares carry 58 bits, and a product is three 32-bit multiply-adds into
+//    64-bit sums; what is cut off stays below 2^-57 of the largest product, so
+//    the sums are as exact as FP64 ones and do not depend on their order.  A
+//    block with a negative or non-finite entry, or none above 2^-895, is summed
+//    in FP64 instead.
+//  * Per population (FP64, lane 3r + i holds row r's population i, so the rows
+//    share each FP64 instruction): the target, the clamp to 3 or 2000 K, the
+//    start 1/T_i (cubic Hermite in ln G, on points equally spaced in it: no
+//    search, no division) and after the evaluation the Newton test, which
+//    compares G_i with P_i / (M c_i) itself.
 //  * Per term (double-float, FP32 pipe; dfloat.cuh): the 300 terms of a row,
 //    slots s = i * NOUT + l, lane j holding slots j + 32 k.  x = a_l / T_i,
-//    expm1(x), its reciprocal, the term t = K_il q and its T dG/dT part
-//    t x (1 + q) (binary32: it only sets the Newton step).  Terms with x > 70
-//    are left out: over 3..2000 K they carry less than 4e-23 of G_i.
+//    expm1(x), its reciprocal, the term t = K_il q.  Terms with x > 70 are left
+//    out: over 3..2000 K they carry less than 4e-23 of G_i.
 //  * The output row: with E the binary exponent of max_i P_i, the scaled
 //    P_i 2^-E over G_i times each term, summed over the populations in
-//    double-float, widened to FP64 and scaled by 2^E: every row sums to
-//    sum_i P_i to the double-float rounding (~1e-14).
-// The table start is within a few 1e-14 of the root, so the first evaluation
-// passes the 1e-13 convergence test; a population that does not (the coarse-
-// start diagnostic, or a rare target) continues Newton over the whole warp,
-// and its row is evaluated and written again.
+//    double-float, widened to FP64 by integers and scaled by 2^E: every row sums
+//    to sum_i P_i to the double-float rounding (~1e-14).
+// The start is within 5e-15 of the root, so the first evaluation passes the
+// 1e-13 convergence test; a population that does not (the coarse-start
+// diagnostic, or a rare target) continues Newton over the whole warp, and its
+// row is evaluated and written again.
+//
+// What bounds it is instruction issue (80%): 2480 warp instructions per row, of
+// which the powers take 660, the output 340 and the terms most of the rest, at
+// 72 registers and 28 warps per SM.  1e6 rows of 200 wavelengths take 2.7 ms
+// (5.3 with FP64 power sums, a start table searched in ln G and Taylor-series
+// exponentials: FP64 pipe 62% busy, 4270 instructions per row), 2.1e6 rows of
+// 200 + 100 wavelengths 6.5 ms (12.5).
 constexpr int NS = NPOP * NOUT;
 constexpr int EX_SLOTS = (NS + 31) / 32;
 constexpr int EX_WARPS = 4;   // warps per block
-constexpr int EX_BATCH = 10;  // rows per warp batch: lanes 3r + i, r < 10
-constexpr float X_CUT = 70.f;
+constexpr int EX_BATCH = 10;  // most rows per warp batch: lanes 3r + i, r < 10
+constexpr float Z_CUT = 70.f * (float)DF_Z_PER_X;
 
 // binary32 -> FP64 on the integer pipe: exact for normal numbers, zero for
 // zero and subnormals (which the double-float terms only reach below 1e-23
@@ -312,7 +377,30 @@ __device__ __forceinline__ double widen(float f)
 
 __device__ __forceinline__ double df_to_double(dfl::df2 v) { return widen(v.hi) + widen(v.lo); }
 
-// v * 2^e for a normal v: the exponent field moved on the integer pipe; a
+// (hi + lo) 2^E for a normalised pair with hi >= 0, on the integer pipe: the
+// low word's bits added to the high word's significand (cut below 2^-52); a
+// result that would leave the normal range takes the multiplication
+__device__ __forceinline__ double df_scaled(dfl::df2 v, int E)
+{
+    const unsigned uh = __float_as_uint(v.hi), ul = __float_as_uint(v.lo);
+    if (uh < 0x00800000u) return 0.0;
+    int eh = (int)(uh >> 23);
+    const int el = (int)((ul >> 23) & 0xFFu), d = eh - el;  // d >= 24 where lo counts
+    const unsigned ml = el ? (ul & 0x7FFFFFu) | 0x800000u : 0u;
+    const unsigned t = d <= 29 ? ml << (29 - d) : (d < 61 ? ml >> (d - 29) : 0u);
+    long long m = (long long)((uh & 0x7FFFFFu) | 0x800000u) << 29;
+    m += (ul >> 31) ? -(long long)t : (long long)t;
+    if (m < (1ll << 52)) {  // the low word took the leading bit
+        m <<= 1;
+        --eh;
+    }
+    const int e = eh + 896 + E;
+    if (e <= 0 || e >= 0x7FF)
+        return __longlong_as_double(m + ((long long)(eh + 895) << 52)) * __longlong_as_double((long long)(E + 1023) << 52);
+    return __longlong_as_double(m + ((long long)(e - 1) << 52));
+}
+
+// v 2^e for a normal v (or 0): the exponent field moved on the integer pipe; a
 // result that would leave the normal range takes the multiplication
 __device__ __forceinline__ double scale_pow2(double v, int e)
 {
@@ -323,26 +411,46 @@ __device__ __forceinline__ double scale_pow2(double v, int e)
 }
 
 // the warp sums of three values on every lane: one butterfly that halves the
-// set of partial sums a lane carries at the first two levels (6 FP64 adds
+// set of partial sums a lane carries at the first two levels (6 additions
 // instead of 15); lanes 8k .. 8k+7 end with the sum of value k, broadcast
-__device__ __forceinline__ void warp_sum3(double& a, double& b, double& c)
+template <typename T, typename Shfl, typename Add>
+__device__ __forceinline__ void warp_sum3(T& a, T& b, T& c, const T zero, const Shfl& xor_, const Shfl& from,
+                                          const Add& add)
 {
     const int lane = threadIdx.x & 31;
     const bool up = lane & 16;
     // level 16: the lower half keeps (a, b), the upper half (c, 0)
-    double k0 = up ? c : a, k1 = up ? 0.0 : b;
-    const double s0 = up ? a : c, s1 = up ? b : 0.0;
-    k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-    k1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+    T k0 = up ? c : a, k1 = up ? zero : b;
+    const T s0 = up ? a : c, s1 = up ? b : zero;
+    k0 = add(k0, xor_(s0, 16, true));
+    k1 = add(k1, xor_(s1, 16, true));
     // level 8: lanes with bit 3 keep the second value
     const bool hi8 = lane & 8;
-    double k = hi8 ? k1 : k0;
-    k += __shfl_xor_sync(0xffffffffu, hi8 ? k0 : k1, 8);
+    T k = add(hi8 ? k1 : k0, xor_(hi8 ? k0 : k1, 8, true));
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-    a = __shfl_sync(0xffffffffu, k, 0);
-    b = __shfl_sync(0xffffffffu, k, 8);
-    c = __shfl_sync(0xffffffffu, k, 16);
+    for (int o = 4; o > 0; o >>= 1) k = add(k, xor_(k, o, true));
+    a = from(k, 0, false);
+    b = from(k, 8, false);
+    c = from(k, 16, false);
+}
+
+template <typename T>
+__device__ __forceinline__ void warp_sum3(T& a, T& b, T& c)
+{
+    const auto sh = [](T v, int o, bool x) {
+        return x ? __shfl_xor_sync(0xffffffffu, v, o) : __shfl_sync(0xffffffffu, v, o);
+    };
+    warp_sum3(a, b, c, T(0), sh, sh, [](T x, T y) { return x + y; });
+}
+
+__device__ __forceinline__ void warp_sum3(dfl::df2& a, dfl::df2& b, dfl::df2& c)
+{
+    const auto sh = [](dfl::df2 v, int o, bool x) {
+        return x ? dfl::make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o))
+                 : dfl::make(__shfl_sync(0xffffffffu, v.hi, o), __shfl_sync(0xffffffffu, v.lo, o));
+    };
+    // add(x, y) == add(y, x) bit for bit: every lane ends with the same sums
+    warp_sum3(a, b, c, dfl::make(0.f, 0.f), sh, sh, [](dfl::df2 x, dfl::df2 y) { return dfl::add(x, y); });
 }
 
 __device__ __forceinline__ dfl::df2 df_from_double(double v)
@@ -351,234 +459,358 @@ __device__ __forceinline__ dfl::df2 df_from_double(double v)
     return dfl::make(h, __double2float_rn(v - (double)h));
 }
 
-// a / b for b > 0 (double-float): the binary32 quotient and one correction
-__device__ __forceinline__ dfl::df2 df_div(dfl::df2 a, dfl::df2 b)
+// 1 / a for a = hi + lo > 0 (lo a few ulp of hi at most) in double-float: the
+// approximate binary32 reciprocal corrected to its last bit, then the exact
+// residual 1 - a y
+__device__ __forceinline__ dfl::df2 df_recip(float hi, float lo)
 {
-    const float q1 = __fdiv_rn(a.hi, b.hi);
-    float p, e;
-    dfl::two_prod(b.hi, q1, p, e);
-    float r = __fsub_rn(a.hi, p);  // exact: q1 b.hi is within an ulp of a.hi
-    r = __fsub_rn(r, e);
-    r = __fadd_rn(r, a.lo);
-    r = fmaf(-b.lo, q1, r);
-    return dfl::renorm(q1, __fdiv_rn(r, b.hi));
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(hi));
+    y = fmaf(y, fmaf(-hi, y, 1.0f), y);
+    const float r = fmaf(-lo, y, fmaf(-hi, y, 1.0f));
+    const float yr = __fmul_rn(y, r);
+    return dfl::make(y, fmaf(yr, r, yr));
 }
 
-struct TermOut {
-    float th, tl, d;
-};
-
-// term of slot (a, K) at 1/T (double-float): t = K / expm1(a / T), and d =
-// t x (1 + q) in binary32 (one copy of the code for every caller)
-__device__ __noinline__ TermOut slot_term(float4 aK, float ih, float il)
+// Term of slot (z, K) at 1/T: t = K / expm1(a / T) as hi + lo.  Sums and products
+// here stay unevaluated (lo a few ulp of hi at most), which the next step allows.
+__device__ __forceinline__ dfl::df2 slot_term(float4 aK, float ih, float il, const float2* __restrict__ exp_tab)
 {
-    const dfl::df2 x = dfl::mul(dfl::make(aK.x, aK.y), dfl::make(ih, il));
-    TermOut o = {0.f, 0.f, 0.f};
-    if (x.hi <= X_CUT) {
-        const dfl::df2 q = dfl::recip(dfl::expm1(x));
-        const dfl::df2 t = dfl::mul(dfl::make(aK.z, aK.w), q);
-        o.th = t.hi;
-        o.tl = t.lo;
-        o.d = t.hi * x.hi * (1.f + q.hi);
-    }
-    return o;
+    float zh, zl;
+    dfl::two_prod(aK.x, ih, zh, zl);
+    zl = fmaf(aK.y, ih, fmaf(aK.x, il, zl));
+    if (!(zh <= Z_CUT)) return dfl::make(0.f, 0.f);
+    const dfl::df2 q0 = dfl::expm1_z(dfl::make(zh, zl), [&](int j) {
+        const float2 e = exp_tab[j];
+        return dfl::make(e.x, e.y);
+    });
+    const dfl::df2 q = df_recip(q0.hi, q0.lo);
+    float th, tl;
+    dfl::two_prod(aK.z, q.hi, th, tl);
+    return dfl::make(th, fmaf(aK.w, q.hi, fmaf(aK.z, q.lo, tl)));
 }
 
-__device__ __forceinline__ void warp_sum_df(dfl::df2& v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const dfl::df2 w = dfl::make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
-        v = dfl::add(v, w);  // add(a, b) == add(b, a) bit for bit: every lane ends with the same sum
-    }
-}
-
-__device__ __forceinline__ float warp_sum_f(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// One row: every slot at its population's 1/T (populations with on bit i),
-// G_i (double-float) and T dG_i/dT (binary32) over the warp, and the output
-// row written from the same terms (staged in buf) with the scaled powers
-// Pp_i (P_i 2^-E).  The slot loop is not unrolled and the term is one
-// non-inlined routine: unrolled, the solve's code outgrew the instruction
-// cache and the warps stalled on instruction fetch.
-__device__ __forceinline__ void eval_row(const float4* __restrict__ slot, const dfl::df2 (&iT)[NPOP], unsigned on,
-                                         const dfl::df2 (&Pp)[NPOP], int scale_e, double* __restrict__ out,
-                                         float2* __restrict__ buf, int lane, dfl::df2 (&G)[NPOP], float (&D)[NPOP])
+// One row: every slot at its population's 1/T (populations with on bit i), G_i
+// over the warp, and the output row written from the same terms (staged in
+// buf) with the scaled powers Pp_i (P_i 2^-E).  The slot loop is not unrolled:
+// the solve's code has to stay in the instruction cache.
+__device__ __forceinline__ void eval_row(const float4* __restrict__ slot, const float2* __restrict__ exp_tab,
+                                         const dfl::df2 (&iT)[NPOP], unsigned on, const dfl::df2 (&Pp)[NPOP],
+                                         int scale_e, double* __restrict__ out, float2* __restrict__ buf, int lane,
+                                         dfl::df2 (&G)[NPOP])
 {
     if (on == 0u) {  // no population absorbs (a dust-free or unheated cell): a zero row
 #pragma unroll
-        for (int i = 0; i < NPOP; ++i) {
-            G[i] = dfl::make(0.f, 0.f);
-            D[i] = 0.f;
-        }
+        for (int i = 0; i < NPOP; ++i) G[i] = dfl::make(0.f, 0.f);
         for (int l = lane; l < NOUT; l += 32) __stcs(out + l, 0.0);
         return;
     }
-    dfl::df2 g0 = dfl::make(0.f, 0.f), g1 = g0, g2 = g0;
-    float d0 = 0.f, d1 = 0.f, d2 = 0.f;
+    // a lane meets its populations' slots one population after the other: the
+    // running sum is set aside where the next one starts
+    dfl::df2 g0 = dfl::make(0.f, 0.f), g1 = g0, it = iT[0];
+    float gh = 0.f, gl = 0.f;
+    bool act = on & 1u;
+    int next = NOUT;  // first slot of the next population
 #pragma unroll 1
-    for (int j = 0; j < EX_SLOTS; ++j) {
-        const int s = lane + 32 * j;
-        const int i = s < NOUT ? 0 : (s < 2 * NOUT ? 1 : 2);
-        TermOut o = {0.f, 0.f, 0.f};
-        if (s < NS && ((on >> i) & 1u)) {
-            const dfl::df2 it = i == 0 ? iT[0] : (i == 1 ? iT[1] : iT[2]);
-            o = slot_term(slot[s], it.hi, it.lo);
+    for (int s = lane; s < EX_SLOTS * 32; s += 32) {
+        if (s >= next) {
+            const bool first = next == NOUT;
+            if (first) g0 = dfl::renorm(gh, gl); else g1 = dfl::renorm(gh, gl);
+            it = first ? iT[1] : iT[2];
+            act = on & (first ? 2u : 4u);
+            next = first ? 2 * NOUT : EX_SLOTS * 32;
+            gh = gl = 0.f;
         }
-        if (s < NS) buf[s] = make_float2(o.th, o.tl);
-        const dfl::df2 tt = dfl::make(o.th, o.tl);
-        if (i == 0) { g0 = dfl::add(g0, tt); d0 += o.d; }
-        else if (i == 1) { g1 = dfl::add(g1, tt); d1 += o.d; }
-        else { g2 = dfl::add(g2, tt); d2 += o.d; }
+        dfl::df2 o = dfl::make(0.f, 0.f);
+        if (act && s < NS) o = slot_term(slot[s], it.hi, it.lo, exp_tab);
+        if (s < NS) buf[s] = make_float2(o.hi, o.lo);
+        float e;
+        dfl::two_sum(gh, o.hi, gh, e);
+        gl = __fadd_rn(gl, __fadd_rn(e, o.lo));
     }
-    warp_sum_df(g0); warp_sum_df(g1); warp_sum_df(g2);
+    dfl::df2 g2 = dfl::renorm(gh, gl);
+    warp_sum3(g0, g1, g2);
     G[0] = g0; G[1] = g1; G[2] = g2;
-    D[0] = warp_sum_f(d0); D[1] = warp_sum_f(d1); D[2] = warp_sum_f(d2);
+    // P_i / G_i, population i on the lanes that are i modulo 3
+    const int i3 = lane % NPOP;
+    const dfl::df2 gi = i3 == 0 ? g0 : (i3 == 1 ? g1 : g2), pi = i3 == 0 ? Pp[0] : (i3 == 1 ? Pp[1] : Pp[2]);
+    const dfl::df2 ri = gi.hi > 0.f ? dfl::mul(pi, df_recip(gi.hi, gi.lo)) : dfl::make(0.f, 0.f);
     dfl::df2 PS[NPOP];
 #pragma unroll
     for (int i = 0; i < NPOP; ++i)
-        PS[i] = (((on >> i) & 1u) && G[i].hi > 0.f) ? df_div(Pp[i], G[i]) : dfl::make(0.f, 0.f);
+        PS[i] = dfl::make(__shfl_sync(0xffffffffu, ri.hi, i), __shfl_sync(0xffffffffu, ri.lo, i));
     __syncwarp();
+#pragma unroll 1
     for (int l = lane; l < NOUT; l += 32) {
-        const float2 b0 = buf[l], b1 = buf[NOUT + l], b2 = buf[2 * NOUT + l];
-        const dfl::df2 e = dfl::add(dfl::add(dfl::mul(PS[0], dfl::make(b0.x, b0.y)), dfl::mul(PS[1], dfl::make(b1.x, b1.y))),
-                                    dfl::mul(PS[2], dfl::make(b2.x, b2.y)));
-        __stcs(out + l, scale_pow2(df_to_double(e), scale_e));
+        float h[NPOP], e[NPOP];
+#pragma unroll
+        for (int i = 0; i < NPOP; ++i) {
+            const float2 b = buf[i * NOUT + l];
+            dfl::two_prod(PS[i].hi, b.x, h[i], e[i]);
+            e[i] = fmaf(PS[i].lo, b.x, fmaf(PS[i].hi, b.y, e[i]));
+        }
+        float u, ue, v, ve;
+        dfl::two_sum(h[0], h[1], u, ue);
+        dfl::two_sum(u, h[2], v, ve);
+        const float lo = __fadd_rn(__fadd_rn(__fadd_rn(e[0], e[1]), e[2]), __fadd_rn(ue, ve));
+        __stcs(out + l, df_scaled(dfl::renorm(v, lo), scale_e));
     }
     __syncwarp();
 }
 
 // G_i and T dG_i/dT at 1/T for one population, the lanes splitting the
 // wavelengths (the rare Newton solve that needs more than one evaluation)
-__device__ void pop_G_warp(const float4* __restrict__ slot, int i, dfl::df2 iT, int lane, double& G, double& D)
+__device__ __noinline__ void pop_G_warp(const float4* __restrict__ slot, const float2* __restrict__ exp_tab, int i,
+                                        dfl::df2 iT, int lane, double& G, double& D)
 {
-    dfl::df2 g = dfl::make(0.f, 0.f);
-    float d = 0.f;
+    dfl::df2 g = dfl::make(0.f, 0.f), z0 = g, z1 = g;
+    float d = 0.f, y0 = 0.f, y1 = 0.f;
     for (int l = lane; l < NOUT; l += 32) {
-        const TermOut o = slot_term(slot[i * NOUT + l], iT.hi, iT.lo);
-        g = dfl::add(g, dfl::make(o.th, o.tl));
-        d += o.d;
+        const float4 aK = slot[i * NOUT + l];
+        const dfl::df2 t = slot_term(aK, iT.hi, iT.lo, exp_tab);
+        g = dfl::add(g, dfl::renorm(t.hi, t.lo));
+        // t x (1 + q), q = t / K
+        d += t.hi * (aK.x * iT.hi * (float)(1.0 / DF_Z_PER_X)) * (1.f + t.hi / aK.z);
     }
-    warp_sum_df(g);
+    warp_sum3(g, z0, z1);
+    warp_sum3(d, y0, y1);
     G = df_to_double(g);
-    D = (double)warp_sum_f(d);
+    D = (double)d;
 }
 
-// Starting point and bracket of the Newton solve for ln G_i(e^y) = target:
-// the table interval holding the target (binary search), and the cubic
-// Hermite inverse of ln G on it (slopes dy/d lnG = 1 / (d lnG / dy)).  With
-// 4096 intervals over [ln 3, ln 2000] the start is within a few 1e-14 of the
-// root (the Hermite error falls as the fourth power of the spacing).  stride
-// > 1 uses every stride-th point only (a coarser start that needs further
-// Newton steps; a diagnostic setting).
-__device__ __forceinline__ void start_T(int i, double target, int stride, double& y, double& lo, double& hi)
+// Start of the Newton solve for ln G_i = target: 1/T from the cubic Hermite
+// polynomial of the table's interval k that holds the target.  With 8192
+// intervals it is within 5e-15 of the root (the error falls as the fourth
+// power of the spacing; 4096 intervals leave 2e-14, which shows in the rows).  stride > 1 uses every stride-th point only (a
+// coarser start that needs further Newton steps; a diagnostic setting).
+__device__ __forceinline__ double start_invT(int i, double target, int stride, int& k, float& slope)
 {
-    const double* tab = &g_lnG_tab[i][0];
-    const double* dtab = &g_dlnG_tab[i][0];
-    int a = 0, b = (NTAB - 1) / stride;  // tab[a stride] <= target < tab[b stride]
-    while (b - a > 1) {
-        const int mid = (a + b) >> 1;
-        if (__ldg(tab + mid * stride) <= target) a = mid; else b = mid;
+    const double t = target - c_lnG_lo[i];
+    const int lg = 31 - __clz(stride);  // stride = 2^lg
+    const int a = min((int)__double2float_rn(t * c_inv_h[i]) >> lg, ((NTAB - 1) >> lg) - 1);
+    k = a << lg;
+    // u = position within the interval; k as a double through the 2^52 offset
+    double u = fma(-(__hiloint2double(0x43300000, k) - 4503599627370496.0), c_h[i], t) * c_inv_h[i];
+    const double2 pa = __ldg(&g_invT_tab[i][k]), pb = __ldg(&g_invT_tab[i][k + stride]);
+    double sa = pa.y, sb = pb.y;
+    if (lg > 0) {
+        const double st = __hiloint2double((1023 + lg) << 20, 0);
+        sa *= st;
+        sb *= st;
+        u *= __hiloint2double((1023 - lg) << 20, 0);
     }
-    const double dy = (log(T_HI) - log(T_LO)) / (NTAB - 1) * stride;
-    lo = log(T_LO) + a * dy;
-    hi = lo + dy;
-    a *= stride;
-    b *= stride;
-    const double ga = __ldg(tab + a), gb = __ldg(tab + b);
-    const double h = gb - ga, u = (target - ga) / h;
-    const double sa = 1.0 / __ldg(dtab + a), sb = 1.0 / __ldg(dtab + b);
-    const double u2 = u * u, u3 = u2 * u;
-    y = (2.0 * u3 - 3.0 * u2 + 1.0) * lo + (u3 - 2.0 * u2 + u) * h * sa + (3.0 * u2 - 2.0 * u3) * hi +
-        (u3 - u2) * h * sb;
-    if (!(y > lo && y < hi)) y = 0.5 * (lo + hi);
+    const double dx = pb.x - pa.x;
+    // d ln T / d ln G at the interval's start (it only sets the Newton test's step)
+    slope = -__double2float_rn(pa.y * c_inv_h[i]) / __double2float_rn(pa.x);
+    const double c2 = fma(3.0, dx, fma(-2.0, sa, -sb)), c3 = fma(-2.0, dx, sa + sb);
+    return fma(u, fma(u, fma(u, c3, c2), sa), pa.x);
 }
 
-// Exact emission for rows m = rows ? rows[k] : k, k < nrows.  A second
-// absorbed table A2 [ncell][n2] with its shares w2 (may be NULL) adds its
+// The sums of a block of up to 256 columns of a row, sum_j w_ij A_j of the three
+// populations, in fixed point: value = s 2^(e - 1078), e the biased exponent of
+// the block's largest entry.  False (nothing summed) for a block with a negative or
+// non-finite entry, or none above 2^-895 but one above zero.
+constexpr int EX_COLS = 256;
+
+__device__ __forceinline__ void mad_wide(unsigned long long& acc, unsigned a, int b)
+{
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
+
+__device__ __forceinline__ void mad_wide(long long& acc, unsigned a, int b)
+{
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
+
+// v >> s for any s (the instruction's clamped shift)
+__device__ __forceinline__ unsigned shr_clamped(unsigned v, unsigned s)
+{
+    unsigned r;
+    asm("shr.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
+    return r;
+}
+
+// wq: the shares' fixed-point pairs, 32 bytes per wavelength: hi, lo of the three
+// populations, 8 bytes of padding (two 16-byte loads)
+__device__ __forceinline__ bool block_powers(const double* __restrict__ row, int n, const int4* __restrict__ wq,
+                                             int lane, unsigned long long& s0, unsigned long long& s1,
+                                             unsigned long long& s2, int& e)
+{
+    double v[EX_COLS / 32];
+    unsigned mx = 0u, any = 0u;
+#pragma unroll
+    for (int k = 0; k < EX_COLS / 32; ++k) {
+        v[k] = lane + 32 * k < n ? __ldcs(row + lane + 32 * k) : 0.0;
+        mx = max(mx, (unsigned)__double2hiint(v[k]));
+        any |= (unsigned)__double2loint(v[k]);
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    s0 = s1 = s2 = 0ull;
+    e = 1;
+    if (mx >= 0x7FF00000u) return false;
+    // all zero, or too small for a subnormal entry to shift out
+    if (mx < 0x08000000u) return mx == 0u && __reduce_or_sync(0xffffffffu, any) == 0u;
+    e = (int)(mx >> 20);
+    // products a w: a = v 2^(1081 - e) as hi (27 bits) and lo (32 bits), w 2^58 as
+    // hi (29 bits, unsigned) and lo (28 bits and sign); partial sums of up to 8
+    unsigned long long hh0 = 0, hh1 = 0, hh2 = 0, lh0 = 0, lh1 = 0, lh2 = 0;
+    long long hl0 = 0, hl1 = 0, hl2 = 0;
+#pragma unroll
+    for (int k = 0; k < EX_COLS / 32; ++k) {
+        if (32 * k < n) {
+            int4 wa = make_int4(0, 0, 0, 0), wb = wa;
+            if (lane + 32 * k < n) {
+                wa = __ldg(wq + 2 * lane + 64 * k);
+                wb = __ldg(wq + 2 * lane + 64 * k + 1);
+            }
+            const unsigned hi = (unsigned)__double2hiint(v[k]), lo = (unsigned)__double2loint(v[k]);
+            const unsigned ex = hi >> 20;
+            const unsigned mh = (hi & 0xFFFFFu) | (ex ? 0x100000u : 0u), sh = (unsigned)e - ex;
+            const unsigned ah0 = __funnelshift_l(lo, mh, 6), al0 = lo << 6;
+            const unsigned al1 = __funnelshift_rc(al0, ah0, sh);
+            const unsigned ah = shr_clamped(ah0, sh), al = shr_clamped(al1, (unsigned)max((int)sh - 32, 0));
+            mad_wide(hh0, ah, wa.x);
+            mad_wide(hl0, ah, wa.y);
+            mad_wide(lh0, al, wa.x);
+            mad_wide(hh1, ah, wa.z);
+            mad_wide(hl1, ah, wa.w);
+            mad_wide(lh1, al, wa.z);
+            mad_wide(hh2, ah, wb.x);
+            mad_wide(hl2, ah, wb.y);
+            mad_wide(lh2, al, wb.x);
+        }
+    }
+    // in units of hi x hi, rounded
+    s0 = hh0 + (unsigned long long)((hl0 + (1ll << 28)) >> 29) + ((lh0 + (1ull << 31)) >> 32);
+    s1 = hh1 + (unsigned long long)((hl1 + (1ll << 28)) >> 29) + ((lh1 + (1ull << 31)) >> 32);
+    s2 = hh2 + (unsigned long long)((hl2 + (1ll << 28)) >> 29) + ((lh2 + (1ull << 31)) >> 32);
+    warp_sum3(s0, s1, s2);
+    return true;
+}
+
+// s 2^(e - 1078)
+__device__ __forceinline__ double fixed_to_double(unsigned long long s, int e)
+{
+    if (s == 0ull) return 0.0;
+    const int x = e - 1078, h = x / 2;
+    return scale_pow2(scale_pow2(__ull2double_rn(s), h), x - h);
+}
+
+// the same sums in FP64
+__device__ __noinline__ void block_powers_fp64(const double* __restrict__ row, int n, const double* __restrict__ w,
+                                               int nw, int lane, double& p0, double& p1, double& p2)
+{
+    p0 = p1 = p2 = 0.0;
+    for (int j = lane; j < n; j += 32) {
+        const double v = __ldcs(row + j);
+        p0 += __ldg(w + j) * v;
+        p1 += __ldg(w + nw + j) * v;
+        p2 += __ldg(w + 2 * nw + j) * v;
+    }
+    warp_sum3(p0, p1, p2);
+}
+
+// Exact emission for rows m = rows ? rows[k] : k, k < nrows.  w: the absorption
+// shares as fill_shares lays them out (16-byte aligned).  A
+// second absorbed table A2 [ncell][n2] with its shares w2 (may be NULL) adds its
 // power to each population's.
-__global__ void __launch_bounds__(32 * EX_WARPS) exact_kernel(
+__global__ void __launch_bounds__(32 * EX_WARPS, 7) exact_kernel(
     const double* __restrict__ A, int n_in, const double* __restrict__ w, const double* __restrict__ A2, int n2,
     const double* __restrict__ w2, const float* __restrict__ mass, const unsigned* __restrict__ rows, long long nrows,
-    double* __restrict__ emission, float* __restrict__ temperature, int stride)
+    double* __restrict__ emission, float* __restrict__ temperature, int stride, int batch)
 {
     __shared__ float4 s_slot[NS];
+    __shared__ float2 s_exp[DF_EXP_N];
     __shared__ float2 s_buf[EX_WARPS][NS];
     for (int s = threadIdx.x; s < NS; s += blockDim.x) s_slot[s] = g_slot[s];
+    for (int j = threadIdx.x; j < DF_EXP_N; j += blockDim.x) s_exp[j] = g_exp[j];
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float2* buf = s_buf[warp];
     const int my_r = lane / NPOP, my_i = lane - NPOP * (lane / NPOP);  // this lane's (row, population)
-    for (long long base = ((long long)blockIdx.x * EX_WARPS + warp) * EX_BATCH; base < nrows;
-         base += (long long)gridDim.x * EX_WARPS * EX_BATCH) {
-        const int nb = nrows - base < EX_BATCH ? (int)(nrows - base) : EX_BATCH;
+    for (long long base = ((long long)blockIdx.x * EX_WARPS + warp) * batch; base < nrows;
+         base += (long long)gridDim.x * EX_WARPS * batch) {
+        const int nb = nrows - base < batch ? (int)(nrows - base) : batch;
         const bool mine = my_r < nb;
         const long long my_m = mine ? (rows ? (long long)rows[base + my_r] : base + my_r) : 0;
-        // ---- population powers, one row at a time over the lanes (FP64)
-        double P = 0.0;
-        int E = 0;
+        // ---- population powers, one row at a time over the lanes: the first
+        // block of each table as an integer, converted once for all rows; what
+        // else there is is added in FP64
+        unsigned long long sa = 0, sb = 0;
+        int ea = 1, eb = 1;
+        double rest = 0.0;
+        bool more = false;
+#pragma unroll 1
         for (int r = 0; r < nb; ++r) {
             const long long m = rows ? (long long)rows[base + r] : base + r;
-            const double* row = A + (size_t)m * n_in;
-            double p0 = 0.0, p1 = 0.0, p2 = 0.0;
-            for (int j = lane; j < n_in; j += 32) {
-                const double v = __ldcs(row + j);
-                p0 += __ldg(w + j) * v;
-                p1 += __ldg(w + n_in + j) * v;
-                p2 += __ldg(w + 2 * n_in + j) * v;
-            }
-            if (A2) {
-                const double* row2 = A2 + (size_t)m * n2;
-                for (int j = lane; j < n2; j += 32) {
-                    const double v = __ldcs(row2 + j);
-                    p0 += __ldg(w2 + j) * v;
-                    p1 += __ldg(w2 + n2 + j) * v;
-                    p2 += __ldg(w2 + 2 * n2 + j) * v;
+#pragma unroll 1
+            for (int tab = 0; tab < (A2 ? 2 : 1); ++tab) {
+                const int nw = tab ? n2 : n_in;
+                const double* row = (tab ? A2 : A) + (size_t)m * nw;
+                const int4* wq = reinterpret_cast<const int4*>(tab ? w2 : w);
+#pragma unroll 1
+                for (int c = 0; c < nw; c += EX_COLS) {
+                    const int n = min(nw - c, EX_COLS);
+                    unsigned long long s0, s1, s2;
+                    int e;
+                    if (block_powers(row + c, n, wq + 2 * c, lane, s0, s1, s2, e)) {
+                        const unsigned long long sv = my_i == 0 ? s0 : (my_i == 1 ? s1 : s2);
+                        if (c > 0) {
+                            more = true;
+                            if (my_r == r) rest += fixed_to_double(sv, e);
+                        } else if (my_r == r) {
+                            if (tab) { sb = sv; eb = e; } else { sa = sv; ea = e; }
+                        }
+                    } else {
+                        double p0, p1, p2;
+                        block_powers_fp64(row + c, n, (tab ? w2 : w) + 4 * (size_t)nw + c, nw, lane, p0, p1, p2);
+                        more = true;
+                        if (my_r == r) rest += my_i == 0 ? p0 : (my_i == 1 ? p1 : p2);
+                    }
                 }
             }
-            warp_sum3(p0, p1, p2);
-            if (my_r == r) {
-                P = my_i == 0 ? p0 : (my_i == 1 ? p1 : p2);
-                // binary exponent of the row's largest population power (0 if none is positive)
-                const double pm = fmax(fmax(p0, p1), p2);
-                E = pm > 0.0 ? ((__double2hiint(pm) >> 20) & 0x7FF) - 1023 : 0;
-                E = E < -1000 ? -1000 : (E > 1000 ? 1000 : E);
-            }
         }
+        double P = fixed_to_double(sa, ea);
+        if (A2) P += fixed_to_double(sb, eb);
+        if (more) P += rest;
+        // binary exponent of the row's largest population power (0 if none is positive)
+        const int xe = P > 0.0 ? (__double2hiint(P) >> 20) + 1 : 0;
+        const int l3 = min(lane - my_i, 29);
+        int E = max(__shfl_sync(0xffffffffu, xe, l3),
+                    max(__shfl_sync(0xffffffffu, xe, l3 + 1), __shfl_sync(0xffffffffu, xe, l3 + 2)));
+        E = E > 0 ? E - 1024 : 0;
+        E = E < -1000 ? -1000 : (E > 1000 ? 1000 : E);
         // ---- per population (FP64): target, clamp or table start, 1/T, scaled power
         const float M = mine ? mass[my_m] : 0.f;
-        int kind = 0;  // 0 no power, 1 clamped, 2 Newton
-        double tg = 0.0, y = 0.0, lo = 0.0, hi = 0.0, T = 0.0;
+        int kind = 0;  // 0 no power, 1 at 3 K, 2 at 2000 K, 3 Newton
+        int k_tab = 0;
+        float slope = 0.f;
+        double Gt = 0.0;
         dfl::df2 iT = dfl::make(0.f, 0.f), Pp = dfl::make(0.f, 0.f);
         if (mine && P > 0.0 && M > 0.f) {
-            tg = log(P / (double)M) - c_lnc[my_i];
+            const double ratio = P / (double)M;
+            const double tg = log(ratio) - c_lnc[my_i];
+            double x;
             if (c_lnG_lo[my_i] - tg >= 0.0) {
                 kind = 1;
-                T = T_LO;
+                x = 1.0 / T_LO;
             } else if (c_lnG_hi[my_i] - tg <= 0.0) {
-                kind = 1;
-                T = T_HI;
-            } else {
                 kind = 2;
-                start_T(my_i, tg, stride, y, lo, hi);
-                T = exp(y);
+                x = 1.0 / T_HI;
+            } else {
+                kind = 3;
+                Gt = ratio * c_Gref[my_i];
+                x = start_invT(my_i, tg, stride, k_tab, slope);
             }
-            iT = df_from_double(1.0 / T);
+            iT = df_from_double(x);
             Pp = df_from_double(P * __longlong_as_double((long long)(1023 - E) << 52));
         }
         const unsigned on_all = __ballot_sync(0xffffffffu, kind != 0);
-        // ---- one evaluation per row (double-float); lane 3r + i keeps its G_i, D_i
+        // ---- one evaluation per row (double-float); lane 3r + i keeps its G_i
         dfl::df2 Gm = dfl::make(0.f, 0.f);
-        float Dm = 0.f;
-        for (int r = 0; r < nb; ++r) {
+        const auto evaluate = [&](int r) {
             const int l0 = NPOP * r;
             dfl::df2 iTr[NPOP], Ppr[NPOP], G[NPOP];
-            float D[NPOP];
 #pragma unroll
             for (int i = 0; i < NPOP; ++i) {
                 iTr[i] = dfl::make(__shfl_sync(0xffffffffu, iT.hi, l0 + i), __shfl_sync(0xffffffffu, iT.lo, l0 + i));
@@ -586,68 +818,61 @@ __global__ void __launch_bounds__(32 * EX_WARPS) exact_kernel(
             }
             const int Er = __shfl_sync(0xffffffffu, E, l0);
             const long long m = rows ? (long long)rows[base + r] : base + r;
-            eval_row(s_slot, iTr, (on_all >> l0) & 7u, Ppr, Er, emission + (size_t)m * NOUT, buf, lane, G, D);
-            if (my_r == r) {
-                Gm = my_i == 0 ? G[0] : (my_i == 1 ? G[1] : G[2]);
-                Dm = my_i == 0 ? D[0] : (my_i == 1 ? D[1] : D[2]);
+            eval_row(s_slot, s_exp, iTr, (on_all >> l0) & 7u, Ppr, Er, emission + (size_t)m * NOUT, buf, lane, G);
+            if (my_r == r) Gm = my_i == 0 ? G[0] : (my_i == 1 ? G[1] : G[2]);
+        };
+        unsigned todo = (1u << nb) - 1u;  // rows to evaluate: all of them, then those Newton moved
+        bool first = true;
+        while (todo) {
+#pragma unroll 1
+            for (unsigned left = todo; left; left &= left - 1u) evaluate(__ffs(left) - 1);
+            todo = 0u;
+            if (!first) break;
+            first = false;
+            // ---- Newton test of every population: converged when the step
+            // ln(G / Gt) d ln T / d ln G of ln T is below 1e-13 of ln T
+            bool redo = false;
+            if (kind == 3) {
+                const float f = __double2float_rn(df_to_double(Gm) - Gt) / __double2float_rn(Gt);
+                const float step = f * slope;
+                redo = !(fabsf(step) <= 1e-13f * fabsf(logf(iT.hi)));
+            }
+            unsigned redo_mask = __ballot_sync(0xffffffffu, redo);
+            while (redo_mask) {  // rare: Newton continues for one population over the whole warp
+                const int L = __ffs(redo_mask) - 1;
+                redo_mask &= redo_mask - 1;
+                const int ii = L % NPOP;
+                const int k = __shfl_sync(0xffffffffu, k_tab, L);
+                const double tgi = log(__shfl_sync(0xffffffffu, Gt, L));
+                // from the table's points around the start (one to either side, for
+                // a target that rounding put beyond its interval's end)
+                double lo = -log(__ldg(&g_invT_tab[ii][max(k - stride, 0)].x)),
+                       hi = -log(__ldg(&g_invT_tab[ii][min(k + 2 * stride, NTAB - 1)].x));
+                dfl::df2 x = dfl::make(__shfl_sync(0xffffffffu, iT.hi, L), __shfl_sync(0xffffffffu, iT.lo, L));
+                double y = -log(df_to_double(x));
+                for (int it = 0; it < 100; ++it) {
+                    double G, D;
+                    pop_G_warp(s_slot, s_exp, ii, x, lane, G, D);
+                    const double f = log(G) - tgi;
+                    const double step = f * G / D;
+                    if (fabs(step) <= 1e-13 * fabs(y)) break;
+                    if (f < 0.0) lo = y; else hi = y;
+                    double y_new = y - step;
+                    if (!(y_new > lo && y_new < hi)) y_new = 0.5 * (lo + hi);
+                    y = y_new;
+                    x = df_from_double(exp(-y));
+                }
+                if (lane == L) iT = x;
+                todo |= 1u << (L / NPOP);  // the row again, with the population's final temperature
             }
         }
-        // ---- Newton test of every population (FP64)
-        bool redo = false;
-        if (kind == 2) {
-            // converged when the Newton step is below 1e-13 of ln T (tested before the
-            // bracket: a start exact to the last bit gives a zero step, and y itself
-            // then sits on the updated bracket's end)
-            const double G = df_to_double(Gm);
-            const double f = log(G) - tg;
-            const double step = f * G / (double)Dm;
-            if (!(fabs(step) <= 1e-13 * fabs(y))) {
-                if (f < 0.0) lo = y; else hi = y;
-                double y_new = y - step;
-                if (!(y_new > lo && y_new < hi)) y_new = 0.5 * (lo + hi);
-                redo = true;
-                y = y_new;
-            }
+        if (temperature && mine) {
+            float T = 0.f;
+            if (kind == 1) T = (float)T_LO;
+            if (kind == 2) T = (float)T_HI;
+            if (kind == 3) T = dfl::recip(iT).hi;
+            temperature[(size_t)my_m * NPOP + my_i] = T;
         }
-        unsigned redo_mask = __ballot_sync(0xffffffffu, redo);
-        while (redo_mask) {  // rare: Newton continues for one population over the whole warp
-            const int L = __ffs(redo_mask) - 1;
-            redo_mask &= redo_mask - 1;
-            const int ri = L / NPOP, ii = L - NPOP * ri;
-            double yi = __shfl_sync(0xffffffffu, y, L), loi = __shfl_sync(0xffffffffu, lo, L),
-                   hii = __shfl_sync(0xffffffffu, hi, L);
-            const double tgi = __shfl_sync(0xffffffffu, tg, L);
-            double Ti = exp(yi), Gi = 0.0, Di = 0.0;
-            for (int it = 1; it < 100; ++it) {
-                Ti = exp(yi);
-                pop_G_warp(s_slot, ii, df_from_double(1.0 / Ti), lane, Gi, Di);
-                const double f = log(Gi) - tgi;
-                const double step = f * Gi / Di;
-                if (fabs(step) <= 1e-13 * fabs(yi)) break;
-                if (f < 0.0) loi = yi; else hii = yi;
-                double y_new = yi - step;
-                if (!(y_new > loi && y_new < hii)) y_new = 0.5 * (loi + hii);
-                yi = y_new;
-                if (it == 99) Ti = exp(yi);  // iteration limit: the last point
-            }
-            if (lane == L) {
-                T = Ti;
-                iT = df_from_double(1.0 / Ti);
-            }
-            // the row again, with the population's final temperature
-            const int l0 = NPOP * ri;
-            dfl::df2 iTr[NPOP], Ppr[NPOP], G[NPOP];
-            float D[NPOP];
-#pragma unroll
-            for (int i = 0; i < NPOP; ++i) {
-                iTr[i] = dfl::make(__shfl_sync(0xffffffffu, iT.hi, l0 + i), __shfl_sync(0xffffffffu, iT.lo, l0 + i));
-                Ppr[i] = dfl::make(__shfl_sync(0xffffffffu, Pp.hi, l0 + i), __shfl_sync(0xffffffffu, Pp.lo, l0 + i));
-            }
-            const int Er = __shfl_sync(0xffffffffu, E, l0);
-            const long long m = rows ? (long long)rows[base + ri] : base + ri;
-            eval_row(s_slot, iTr, (on_all >> l0) & 7u, Ppr, Er, emission + (size_t)m * NOUT, buf, lane, G, D);
-        }
-        if (temperature && mine) temperature[(size_t)my_m * NPOP + my_i] = (float)T;
     }
 }
 
@@ -723,17 +948,35 @@ std::vector<int> band_starts(const double* lam, int n)
     return start;
 }
 
-std::vector<double> share_table(const double* lam, int n)
+// shares w_i(lambda_j) = (lambda_j/0.55)^delta_i / sum_k (lambda_j/0.55)^delta_k:
+// first their fixed-point pairs for block_powers, w 2^58 = hi 2^29 + lo, |lo| <=
+// 2^28, 32 bytes per wavelength, then the shares themselves [3][n]; 8 doubles per
+// wavelength in all, so that a second table behind the first stays aligned
+constexpr int SHARES = 8;
+void fill_shares(const double* lam, int n, double* out)
 {
-    std::vector<double> w((size_t)NPOP * n);
+    double* w = out + 4 * (size_t)n;
     for (int j = 0; j < n; ++j) {
         double r[NPOP], sum = 0.0;
         for (int i = 0; i < NPOP; ++i) {
             r[i] = std::pow(lam[j] / 0.55, DELTA[i]);
             sum += r[i];
         }
-        for (int i = 0; i < NPOP; ++i) w[(size_t)i * n + j] = r[i] / sum;
+        int q[8] = {};
+        for (int i = 0; i < NPOP; ++i) {
+            const double v = r[i] / sum, h = std::floor(v * 536870912.0 + 0.5);
+            w[(size_t)i * n + j] = v;
+            q[2 * i] = (int)h;
+            q[2 * i + 1] = (int)std::floor((v * 536870912.0 - h) * 536870912.0 + 0.5);
+        }
+        std::memcpy(out + 4 * (size_t)j, q, sizeof q);
     }
+}
+
+std::vector<double> share_table(const double* lam, int n)
+{
+    std::vector<double> w((size_t)SHARES * n);
+    fill_shares(lam, n, w.data());
     return w;
 }
 
@@ -751,7 +994,7 @@ int launch_exact_emission(const double* absorbed, int n_in, const double* w_dev,
                           const unsigned* rows, long long nrows, double* emission, float* temperature,
                           cudaStream_t s, const double* absorbed2, int n2, const double* w2_dev)
 {
-    ECK(upload_model(s));
+    ECK(upload_model());
     // one warp per batch of rows, every row list alike (all cells, or the
     // surrogate's fallback rows).  SKIRT_EXACT_TABLE_STRIDE (a power of two up to 64)
     // starts the Newton solves from a coarser table: the same results through
@@ -762,10 +1005,15 @@ int launch_exact_emission(const double* absorbed, int n_in, const double* w_dev,
         if (v >= 1 && v <= 64 && (v & (v - 1)) == 0) stride = v;
     }
     if (nrows > 0) {
-        long long blocks = (nrows + EX_WARPS * EX_BATCH - 1) / (EX_WARPS * EX_BATCH);
+        // full batches once there are enough rows for them to fill the warps the
+        // device holds (152 SMs x 24); below that as many warps as rows allow, each
+        // with fewer rows in series (2000 rows: 115 us by tens, one by one below)
+        const long long warps = 152LL * 24;
+        const int batch = (int)std::min<long long>(EX_BATCH, (nrows + warps - 1) / warps);
+        long long blocks = (nrows + EX_WARPS * batch - 1) / (EX_WARPS * batch);
         if (blocks > 152LL * 32) blocks = 152LL * 32;
         exact_kernel<<<(int)blocks, 32 * EX_WARPS, 0, s>>>(absorbed, n_in, w_dev, absorbed2, n2, w2_dev, mass, rows,
-                                                           nrows, emission, temperature, stride);
+                                                           nrows, emission, temperature, stride, batch);
     }
     ECK(cudaGetLastError());
     return SKIRT_OK;
@@ -937,7 +1185,7 @@ extern "C" int skirt_dust_emission_pair(const double* absorbed_a, long long ncel
     ECK(cudaMallocAsync((void**)&d_w, sizeof(double) * w.size(), s));
     ECK(cudaMemcpyAsync(d_w, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice, s));
     int rc = launch_exact_emission(absorbed_a, n_a, d_w, mass, nullptr, ncell, emission, temperature, s, absorbed_b,
-                                   absorbed_b ? n_b : 0, absorbed_b ? d_w + (size_t)NPOP * n_a : nullptr);
+                                   absorbed_b ? n_b : 0, absorbed_b ? d_w + (size_t)SHARES * n_a : nullptr);
     cudaFreeAsync(d_w, s);
     ECK(cudaStreamSynchronize(s));
     return rc;
@@ -953,30 +1201,17 @@ extern "C" int skirt_dust_emission_pair(const double* absorbed_a, long long ncel
 // call time: a process whose framework allocator has already reserved the
 // device memory it may use, or a loop with a fixed memory budget decided up
 // front.  skirt_dust_emission_exact_static does the same exact solve with that
-// table in the fixed array below instead (3 x 4096 doubles = 96 KiB, held by
+// table in the fixed array below instead (8 x 4096 doubles = 256 KiB, held by
 // every device that loads the library until the process exits).
 // ---------------------------------------------------------------------------
 namespace {
 
 constexpr int STATIC_MAX_NIN = 4096;
-static __device__ __align__(256) double g_static_shares[NPOP * STATIC_MAX_NIN];
+static __device__ __align__(256) double g_static_shares[SHARES * STATIC_MAX_NIN];
 
 std::mutex g_static_mutex;
 double* g_static_ptr[64] = {};  // device address of g_static_shares, per device ordinal
-double g_static_host[NPOP * STATIC_MAX_NIN];  // host copy of the table (guarded by g_static_mutex)
-
-// shares w_i(lambda_j) = (lambda_j/0.55)^delta_i / sum_k (lambda_j/0.55)^delta_k into out[i*n + j]
-void fill_shares(const double* lam, int n, double* out)
-{
-    for (int j = 0; j < n; ++j) {
-        double r[NPOP], sum = 0.0;
-        for (int i = 0; i < NPOP; ++i) {
-            r[i] = std::pow(lam[j] / 0.55, DELTA[i]);
-            sum += r[i];
-        }
-        for (int i = 0; i < NPOP; ++i) out[(size_t)i * n + j] = r[i] / sum;
-    }
-}
+double g_static_host[SHARES * STATIC_MAX_NIN];  // host copy of the table (guarded by g_static_mutex)
 
 }  // namespace
 
@@ -1015,7 +1250,7 @@ extern "C" int skirt_dust_emission_exact_static(const double* absorbed, long lon
         // (CUDA does not promise that an asynchronous copy from pageable memory has
         // read its source when the call returns).
         fill_shares(lambda_in, n_in, g_static_host);
-        ECK(cudaMemcpyAsync(shares, g_static_host, sizeof(double) * NPOP * n_in, cudaMemcpyHostToDevice, s));
+        ECK(cudaMemcpyAsync(shares, g_static_host, sizeof(double) * SHARES * n_in, cudaMemcpyHostToDevice, s));
         ECK(cudaStreamSynchronize(s));
     }
     int rc = launch_exact_emission(absorbed, n_in, shares, mass, nullptr, ncell, emission, temperature, s);
