@@ -110,6 +110,7 @@ void fill_instrument(const skirt_instrument& s, InstrDev& d, long long img_off)
     const double e2[3] = {k[1] * e1[2] - k[2] * e1[1], k[2] * e1[0] - k[0] * e1[2], k[0] * e1[1] - k[1] * e1[0]};
     for (int a = 0; a < 3; ++a) {
         d.kobs[a] = k[a];
+        d.ikobs[a] = k[a] != 0.0 ? 1.0 / k[a] : 0.0;
         d.e1[a] = e1[a];
         d.e2[a] = e2[a];
         d.kobs_f[a] = (float)k[a];
@@ -169,6 +170,7 @@ int grid_init(skirt_grid_s* g, int nx, int ny, int nz, long long ncell, const do
     {
         // face planes lo + k d (k < n) and the upper bound, split into (hi, lo) FP32 pairs
         std::vector<float2> f;
+        std::vector<double> f64;
         const int nn[3] = {nx, ny, nz};
         for (int a = 0; a < 3; ++a) {
             const double lo = bbox[2 * a], hi = bbox[2 * a + 1], d = (hi - lo) / nn[a];
@@ -176,11 +178,16 @@ int grid_init(skirt_grid_s* g, int nx, int ny, int nz, long long ncell, const do
                 const double v = k < nn[a] ? lo + (double)k * d : hi;
                 const float h = (float)v;
                 f.push_back(make_float2(h, (float)(v - (double)h)));
+                f64.push_back(std::fma((double)k, d, lo));
             }
         }
         if ((e = cudaMalloc(&g->faces, sizeof(float2) * f.size())) != cudaSuccess)
             return fail(SKIRT_ERR_OOM, "faces: %s", cudaGetErrorString(e));
         if ((e = cudaMemcpy(g->faces, f.data(), sizeof(float2) * f.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
+            return fail(SKIRT_ERR_CUDA, "faces: %s", cudaGetErrorString(e));
+        if ((e = cudaMalloc(&g->faces64, sizeof(double) * f64.size())) != cudaSuccess)
+            return fail(SKIRT_ERR_OOM, "faces: %s", cudaGetErrorString(e));
+        if ((e = cudaMemcpy(g->faces64, f64.data(), sizeof(double) * f64.size(), cudaMemcpyHostToDevice)) != cudaSuccess)
             return fail(SKIRT_ERR_CUDA, "faces: %s", cudaGetErrorString(e));
     }
     if ((e = cudaEventCreate(&g->ev0)) != cudaSuccess || (e = cudaEventCreate(&g->ev1)) != cudaSuccess)
@@ -280,6 +287,7 @@ extern "C" int skirt_grid_destroy(skirt_grid_t g)
     if (g->kr64) cudaFree(g->kr64);
     if (g->kr_fast) cudaFree(g->kr_fast);
     if (g->faces) cudaFree(g->faces);
+    if (g->faces64) cudaFree(g->faces64);
     if (g->oct_nodes) cudaFree(g->oct_nodes);
     if (g->oct_leaf) cudaFree(g->oct_leaf);
     g->scratch.release();
@@ -528,6 +536,7 @@ extern "C" int skirt_trace(skirt_grid_t g, const skirt_source* src, const skirt_
     A.g_f = (const float*)(dp + L.g_f);
     A.L0_f = (const float*)(dp + L.L0_f);
     A.faces = g->faces;
+    A.faces64 = g->faces64;
     for (int a = 0; a < 3; ++a) {
         const float hi = (float)src->pos[a];
         A.src_df[a] = make_float2(hi, (float)(src->pos[a] - (double)hi));
@@ -615,8 +624,6 @@ extern "C" int skirt_trace(skirt_grid_t g, const skirt_source* src, const skirt_
         const unsigned long long fair = P.total / (8ull * (unsigned long long)pgrid * (unsigned long long)block);
         if ((unsigned long long)A.chunk > fair) A.chunk = fair > 0 ? (int)fair : 1;
     }
-    if (opts->precision == SKIRT_PREC_FP64 && trace_smem_bytes(A.ninstr, block) > 48 * 1024)
-        return fail(SKIRT_ERR_INVALID_ARG, "block too large for the shared-memory budget");
 
     // ---- the device work of one call (recorded into a graph when asked)
     auto enqueue = [&](cudaStream_t s, bool events) -> int {

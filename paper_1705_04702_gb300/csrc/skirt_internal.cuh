@@ -42,6 +42,7 @@ __device__ __forceinline__ float u01f(uint32_t x)
 // Per-instrument constants (host-computed in FP64, FP32 copies for the mixed form).
 struct InstrDev {
     double kobs[3], e1[3], e2[3];
+    double ikobs[3];    // 1 / kobs, zero for zero components
     double half_fov, inv_dpx, flux_norm;
     float kobs_f[3], e1_f[3], e2_f[3];
     float ikobs_f[3];   // 1 / kobs_f, zero for zero components
@@ -90,6 +91,7 @@ struct TraceArgs {
     const float* g_f;
     const float* L0_f;
     const float2* faces;                   // face planes as (hi, lo) FP32 pairs: x [nx+1], y [ny+1], z [nz+1]
+    const double* faces64;                 // face planes in FP64, the same order
     float2 src_df[3];                      // source position as (hi, lo) FP32 pairs
     float src_dir_f[3];
     float lo_f[3], d_f[3], id_f[3], hi_f[3];  // lower corner, cell size, its reciprocal, upper corner in FP32
@@ -246,6 +248,7 @@ struct skirt_grid_s {
     double* kr64 = nullptr;
     int fast = 0;              // the traversal order's fastest axis
     float2* faces = nullptr;  // exact face planes as (hi, lo) FP32 pairs, x then y then z
+    double* faces64 = nullptr;  // face planes as the FP64 form evaluates them, fma(k, d, lo)
     skirt::DevBuf scratch;  // per-call tables, accumulators, work queue
     skirt::DevBuf stage;    // device images of host outputs
     skirt::DevBuf cdf;      // dust source: [nlambda][ncell] running sums within tiles

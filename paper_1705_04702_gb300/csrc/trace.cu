@@ -1,11 +1,5 @@
-// Photon-packet life cycle on the GPU, plain FP64 form: one packet per
-// thread, written as a per-thread state machine so that every iteration of
-// the main loop does one cell crossing for every lane that is inside a
-// traversal, whatever kind of traversal it is (absorption deposit,
-// forced-interaction search, or peel-off line of sight).  Lanes that just
-// finished a traversal handle their event (launch, scattering, peel-off
-// tally) and rejoin the stepping loop.  Every quantity is FP64.  The mixed
-// form lives in trace_mixed.cu.
+// Photon-packet life cycle on the GPU, plain FP64 form: every quantity FP64.
+// The mixed form lives in trace_mixed.cu.
 //
 // Method (arXiv:1705.04702): Sect. 3.2 (stellar emission phase: packets per
 // wavelength, Monte Carlo launch / interaction sampling, peel-off to every
@@ -17,8 +11,24 @@
 // (octree dust grid: a cell crossing steps from a leaf to the leaf across its
 // exit face, through the precomputed face neighbour and a descent by the
 // lattice cell of the entry point).
+//
+// What bounds it is the FP64 pipe (85% active in a long run): a warp instruction
+// holds it for some 20 cycles of the SM, whatever its active lanes.  So the lanes
+// of a warp step together, peel-offs in some rounds and deposits and searches in
+// others (a deposit crossing costs three times a peel-off's FP64 instructions),
+// and handle their events together when few of them are stepping; and FP64 does
+// only what has to be FP64.  Distances and optical depths are compared as integers
+// (none is negative), face planes come from a table, the search starts from the
+// saved start of the deposit traversal it repeats, and the deposits of a path take
+// e^{-tau} once per round of crossings and subtract what each cell takes from it
+// in between.  A peel-off crossing is 5 or 6 FP64 instructions, a deposit crossing
+// 17 in thin cells.  3e5 packets of 3 wavelengths on a 97^3 disk take 39 ms (132
+// with one state machine per lane, every crossing 12 FP64 instructions and two
+// exponentials more per deposit, at 5 of 32 lanes).
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <type_traits>
 
 #include "skirt_internal.cuh"
 #include "trace_device.cuh"
@@ -26,92 +36,102 @@
 namespace skirt {
 namespace {
 
-// Arithmetic policy of the plain form (R = double throughout).
-template <typename R> struct P;
+// Lanes of one kind stepping below which a warp handles its idle lanes' events, and
+// crossings between warp votes (and between evaluations of e^{-tau}).  The case
+// named above with 8 / 24: 39 ms; 16 / 16: 48, 8 / 16: 43, 8 / 32: 43, 12 / 16: 46.
+constexpr int FP64_STEP_MIN = 8;
+constexpr int FP64_ROUND = 24;
+constexpr int FP64_MAXB = 512;     // threads per block (upper bound)
 
-template <> struct P<double> {
-    static __device__ __forceinline__ double kr(const TraceArgs& a, int m) { return __ldg(a.kr64 + m); }
-    static __device__ __forceinline__ double logr(double x) { return log(x); }
-    static __device__ __forceinline__ double sqrtr(double x) { return sqrt(x); }
-    static __device__ __forceinline__ double floorr(double x) { return floor(x); }
-    static __device__ __forceinline__ void sincospi2(double u, double* s, double* c) { sincospi(2.0 * u, s, c); }
-    static __device__ __forceinline__ double u(uint32_t x) { return (double)u01f(x); }
-    // e^{-tau_prev} (1 - e^{-dtau}) for the deposit
-    static __device__ __forceinline__ double dep_factor(double tau_prev, double dtau) {
-        return exp(-tau_prev) * (-expm1(-dtau));
-    }
-    static __device__ __forceinline__ double kobs(const InstrDev& I, int a) { return I.kobs[a]; }
-    static __device__ __forceinline__ double e1(const InstrDev& I, int a) { return I.e1[a]; }
-    static __device__ __forceinline__ double e2(const InstrDev& I, int a) { return I.e2[a]; }
-    static __device__ __forceinline__ double half_fov(const InstrDev& I) { return I.half_fov; }
-    static __device__ __forceinline__ double inv_dpx(const InstrDev& I) { return I.inv_dpx; }
-    static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
+// Per-thread state used only at events, in shared memory: arrays of blockDim.x.
+enum {
+    D_L_EMIT, D_L_ABS, D_L_ESC, D_L_RES,   // ledger of the current wavelength
+    D_L0, D_P_ESC, D_P_ABS, D_P_RES, D_P_PEEL, D_OM, D_PEEL_W, D_ALB, D_LABS,
+    D_B_T0, D_B_T1, D_B_T2,                // start of the deposit traversal: distances to its first faces
+    D_NUM
 };
+enum {
+    I_C_DEP, I_C_LOC, I_C_PEEL, I_C_SCAT,  // added to the 64-bit counters below 2^32
+    I_LAM, I_NSCAT, I_PEEL_I, I_PK, I_EV, I_RY, I_RZ, I_LEFT, I_QLO, I_QHI,
+    I_B_0, I_B_1, I_B_2, I_B_M,            // start of the deposit traversal: cell (lattice corner) and index (node)
+    I_NUM
+};
+constexpr int PEEL_SCATTER = 16;  // added to the instrument's index after a scattering (at most 16 instruments)
 
-// Distance along the ray from o (inverse direction component iv) to the
-// face plane lo + k d.  One fused multiply-add for the plane, so that every
-// grid kind evaluates the same plane to the same value.
-template <typename R>
-__device__ __forceinline__ R face_dist(R lo, int k, R d, R o, R iv)
+__device__ __forceinline__ long long bits(double v) { return __double_as_longlong(v); }
+// v, or 0 where its sign bit is set
+__device__ __forceinline__ double clip0(double v) { return __double2hiint(v) < 0 ? 0.0 : v; }
+
+// 1 - e^{-x} for x >= 0: below 1/16 the Taylor series x (1 - x/2 + ... + x^8/9!),
+// whose first omitted term is below 4e-18 of the result
+__device__ __forceinline__ double one_minus_exp_neg(double x)
 {
-    return (fma((R)k, d, lo) - o) * iv;
+    if (bits(x) < 0x3FB0000000000000ll) {
+        double p = fma(x, 1.0 / 362880.0, -1.0 / 40320.0);
+        p = fma(x, p, 1.0 / 5040.0);
+        p = fma(x, p, -1.0 / 720.0);
+        p = fma(x, p, 1.0 / 120.0);
+        p = fma(x, p, -1.0 / 24.0);
+        p = fma(x, p, 1.0 / 6.0);
+        p = fma(x, p, -0.5);
+        return fma(x * x, p, x);
+    }
+    return -expm1(-x);
 }
 
-template <typename R, bool OCT>
-__global__ void __launch_bounds__(512) trace_kernel(const TraceArgs A)
+template <bool OCT>
+__global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int t = threadIdx.x, nt = blockDim.x;
     InstrDev* sins = reinterpret_cast<InstrDev*>(smem_raw);
+    double* cd = reinterpret_cast<double*>(smem_raw + sizeof(InstrDev) * A.ninstr);
+    int* ci = reinterpret_cast<int*>(cd + (size_t)D_NUM * nt);
+    const auto D = [&](int k) -> double& { return cd[k * nt + t]; };
+    const auto I = [&](int k) -> int& { return ci[k * nt + t]; };
     for (int i = threadIdx.x; i < A.ninstr; i += blockDim.x) sins[i] = A.ins[i];
+    D(D_L_EMIT) = D(D_L_ABS) = D(D_L_ESC) = D(D_L_RES) = 0.0;
+    I(I_C_DEP) = I(I_C_LOC) = I(I_C_PEEL) = I(I_C_SCAT) = 0;
+    I(I_LAM) = -1;
+    I(I_LEFT) = I(I_QLO) = I(I_QHI) = 0;
     __syncthreads();
 
     const int NL = A.nlambda;
     const int nx = A.nx, ny = A.ny, nz = A.nz;
-    const R lo0 = (R)A.lo[0], lo1 = (R)A.lo[1], lo2 = (R)A.lo[2];
-    const R d0 = (R)A.d[0], d1 = (R)A.d[1], d2 = (R)A.d[2];
-    const R INF = P<R>::inf();
+    const double INF = __longlong_as_double(0x7ff0000000000000ll);
+    const double* __restrict__ faces = A.faces64;  // x [nx+1], y [ny+1], z [nz+1]
 
-    // ---- traversal state
+    // ---- traversal state: origin (x0, x1, x2), direction in its reciprocals
     int mode = M_NONE;
     int c0 = 0, c1 = 0, c2 = 0;
     int s0 = 0, s1 = 0, s2 = 0;
-    R o0 = 0, o1 = 0, o2 = 0;   // traversal origin
-    R v0 = 0, v1 = 0, v2 = 0;   // traversal direction
-    R iv0 = 0, iv1 = 0, iv2 = 0; // its inverse
-    R tn0 = 0, tn1 = 0, tn2 = 0; // distance to the next face on each axis
-    R tcur = 0;
-    double tau = 0.0;           // optical depth accumulated along this traversal
-    double tau_t = 0.0;         // interaction optical depth (locate)
-    double labs = 0.0;          // L (1 - albedo) (deposit)
-    R s_found = 0, last_dusty_end = 0;
+    double iv0 = 0, iv1 = 0, iv2 = 0;
+    double tn0 = 0, tn1 = 0, tn2 = 0;  // distance to the next face on each axis
+    double tcur = 0;
+    double tau = 0.0;                  // optical depth along this traversal
+    double par = 0.0;                  // deposit: L (1 - albedo) e^{-tau}; search: interaction optical depth
+    double s_found = 0, last_dusty_end = 0;
     bool found = false;
-    // octree: current leaf (node, level, leaf index, kr); c0..c2 hold its
-    // lattice corner
+    unsigned nsteps = 0;
+    int cur_m = 0;                     // the current cell (octree: leaf) and its extinction coefficient
+    double kr_cur = 0;
+    // octree: the current leaf's node and level (c0..c2: its lattice corner), the
+    // direction of the traversal
     const int OL = A.oct_levels;
-    int onode = 0, olev = 0, oleaf = 0, osteps = 0;
-    float okr = 0.f;
+    int onode = 0, olev = 0;
+    double v0 = 0, v1 = 0, v2 = 0;
 
     // ---- packet state
     int stage = ST_NEW;
-    int lam = -1;
-    unsigned long long q = 0, q_end = 0;
-    bool started = false;
-    uint32_t pk = 0;
-    double L = 0.0, L0 = 0.0, tau_path = 0.0;
-    R x0 = 0, x1 = 0, x2 = 0;   // position
-    R k0 = 0, k1 = 0, k2 = 0;   // direction
-    uint32_t ev = 0;
-    int nscat = 0;
-    R krs = 0, gg = 0;
-    double alb = 0.0;
-    int peel_i = 0, peel_kind = 0, after_peel = 0;
-    double peel_w = 0.0;
-    double p_esc = 0.0, p_abs = 0.0, p_res = 0.0, p_peel = 0.0;
-
-    // ---- thread-level ledger for the current wavelength, and work counters
-    int led_lam = -1;
-    double l_emit = 0.0, l_abs = 0.0, l_esc = 0.0, l_res = 0.0;
-    unsigned long long c_scat = 0, c_dep = 0, c_loc = 0, c_peel = 0;
+    bool alive = true, started = false;
+    int lam = 0;
+    double L = 0.0;
+    double x0 = 0, x1 = 0, x2 = 0;     // position
+    double k0 = 0, k1 = 0, k2 = 0;     // direction
+    double krs = 0, gg = 0;
+    bool unit = false;                 // krs is 1
+    bool have_pc = false;              // pc0..pc2 (octree: pc_node) is the position's cell
+    int pc0 = 0, pc1 = 0, pc2 = 0, pc_node = 0;
 
     // octree: the leaf holding lattice cell (j0, j1, j2), found by descending
     // from `node` (a node of level `lev`, or a leaf)
@@ -125,401 +145,484 @@ __global__ void __launch_bounds__(512) trace_kernel(const TraceArgs A)
         }
         onode = node;
         olev = oct_leaf_level(r);
-        oleaf = oct_leaf_index(r);
-        okr = __ldg(&A.oct_nodes[node].kr);
+        cur_m = oct_leaf_index(r);
+        kr_cur = (double)__ldg(&A.oct_nodes[node].kr);
         const int mask = ~((1 << (OL - olev)) - 1);
         c0 = j0 & mask;
         c1 = j1 & mask;
         c2 = j2 & mask;
     };
 
-    auto begin = [&](int m, R ox, R oy, R oz, R vx, R vy, R vz) {
+    // distances to the faces through which the current cell (of e lattice cells
+    // per axis) can be left
+    auto set_faces = [&](int e) {
+        const double* fy = faces + (nx + 1);
+        const double* fz = fy + (ny + 1);
+        tn0 = s0 ? clip0((__ldg(faces + c0 + (s0 > 0 ? e : 0)) - x0) * iv0) : INF;
+        tn1 = s1 ? clip0((__ldg(fy + c1 + (s1 > 0 ? e : 0)) - x1) * iv1) : INF;
+        tn2 = s2 ? clip0((__ldg(fz + c2 + (s2 > 0 ? e : 0)) - x2) * iv2) : INF;
+    };
+
+    // starts a traversal of kind m along (vx, vy, vz), whose reciprocals (zero
+    // for zero components) are (i0, i1, i2), from the packet's position
+    auto begin = [&](int m, double vx, double vy, double vz, double i0, double i1, double i2) {
         mode = m;
-        o0 = ox; o1 = oy; o2 = oz;
-        v0 = vx; v1 = vy; v2 = vz;
-        c0 = cell_index<R>(ox, lo0, d0, nx);
-        c1 = cell_index<R>(oy, lo1, d1, ny);
-        c2 = cell_index<R>(oz, lo2, d2, nz);
+        if (!have_pc) {
+            pc0 = cell_index<double>(x0, A.lo[0], A.d[0], nx);
+            pc1 = cell_index<double>(x1, A.lo[1], A.d[1], ny);
+            pc2 = cell_index<double>(x2, A.lo[2], A.d[2], nz);
+            pc_node = 0;
+            have_pc = true;
+        }
+        s0 = vx > 0.0 ? 1 : (vx < 0.0 ? -1 : 0);
+        s1 = vy > 0.0 ? 1 : (vy < 0.0 ? -1 : 0);
+        s2 = vz > 0.0 ? 1 : (vz < 0.0 ? -1 : 0);
+        iv0 = i0; iv1 = i1; iv2 = i2;
         if (OCT) {
-            oct_enter(0, 0, c0, c1, c2);
-            osteps = 0;
+            oct_enter(pc_node, 0, pc0, pc1, pc2);
+            pc0 = c0; pc1 = c1; pc2 = c2;
+            pc_node = onode;
+            v0 = vx; v1 = vy; v2 = vz;
+            set_faces(1 << (OL - olev));
+        } else {
+            c0 = pc0; c1 = pc1; c2 = pc2;
+            cur_m = (c2 * ny + c1) * nx + c0;
+            kr_cur = __ldg(A.kr64 + cur_m);
+            set_faces(1);
         }
-        s0 = vx > (R)0 ? 1 : (vx < (R)0 ? -1 : 0);
-        s1 = vy > (R)0 ? 1 : (vy < (R)0 ? -1 : 0);
-        s2 = vz > (R)0 ? 1 : (vz < (R)0 ? -1 : 0);
-        iv0 = s0 ? (R)1 / vx : (R)0;
-        iv1 = s1 ? (R)1 / vy : (R)0;
-        iv2 = s2 ? (R)1 / vz : (R)0;
-        if (!OCT) {
-            tn0 = s0 ? face_dist<R>(lo0, c0 + (s0 > 0), d0, ox, iv0) : INF;
-            tn1 = s1 ? face_dist<R>(lo1, c1 + (s1 > 0), d1, oy, iv1) : INF;
-            tn2 = s2 ? face_dist<R>(lo2, c2 + (s2 > 0), d2, oz, iv2) : INF;
-        }
-        tcur = (R)0;
+        tcur = 0.0;
         tau = 0.0;
+        nsteps = 0;
+    };
+
+    // one cell crossing (PEEL: of a peel-off; otherwise of a deposit or a search)
+    auto step = [&](auto kind) {
+        constexpr bool PEEL = decltype(kind)::value;
+        const long long b0 = bits(tn0), b1 = bits(tn1), b2 = bits(tn2);
+        const int axis = b0 <= b1 ? (b0 <= b2 ? 0 : 2) : (b1 <= b2 ? 1 : 2);
+        const double tnext = axis == 0 ? tn0 : (axis == 1 ? tn1 : tn2);
+        const int sa = axis == 0 ? s0 : (axis == 1 ? s1 : s2);
+        const int ca = axis == 0 ? c0 : (axis == 1 ? c1 : c2);
+        const int na = axis == 0 ? nx : (axis == 1 ? ny : nz);
+        // what the crossing leads to, requested before the crossing's work
+        int nb = 0, mn = 0;
+        bool out;
+        double kr_next = 0.0;
+        if (OCT) {
+            nb = __ldg(&A.oct_nodes[onode].nb[2 * axis + (sa > 0)]);
+            out = nb < 0;  // the exit face lies on the root box
+        } else {
+            out = (unsigned)(ca + sa) >= (unsigned)na;
+            mn = cur_m + sa * (axis == 0 ? 1 : (axis == 1 ? nx : nx * ny));
+            if (!out) kr_next = __ldg(A.kr64 + mn);
+        }
+        const double ds = clip0(tnext - tcur);
+        double krl = kr_cur;
+        if (!unit) krl *= krs;
+        const double dtau = krl * ds;
+        const double tau_n = tau + dtau;
+        ++nsteps;
+        if (PEEL) {
+        } else if (mode == M_DEPOSIT) {
+            if (bits(dtau) > 0) {
+                const double dep = par * one_minus_exp_neg(dtau);
+                if (bits(dep) > 0)
+                    atomicAdd(A.absorbed + ((size_t)cur_m * A.abs_cs + (size_t)lam * A.abs_ls), dep);
+                par -= dep;
+            }
+        } else if (bits(krl) > 0) {
+            if (bits(tau_n) >= bits(par)) {
+                s_found = tcur + (par - tau) / krl;
+                found = true;
+                mode = M_NONE;
+                return;  // the current cell stays
+            }
+            last_dusty_end = tnext;
+        }
+        tau = tau_n;
+        if (out) {
+            mode = M_NONE;
+            return;
+        }
+        tcur = tnext;
+        if (OCT) {
+            if (nsteps > (unsigned)A.oct_step_cap) {
+                atomicOr(A.err, (unsigned)ERRBIT_PATH);
+                mode = M_NONE;
+                return;
+            }
+            // lattice cell of the entry point into the next leaf: across the exit
+            // face along `axis`; along the other axes the cell of the crossing
+            // point, kept within the current leaf's cross-section
+            const int osz = 1 << (OL - olev);
+            int j[3];
+            const int cc[3] = {c0, c1, c2};
+            const double oo[3] = {x0, x1, x2}, vv[3] = {v0, v1, v2};
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                if (b == axis) {
+                    j[b] = sa > 0 ? cc[b] + osz : cc[b] - 1;
+                } else {
+                    const double f = floor((oo[b] + tnext * vv[b] - A.lo[b]) / A.d[b]);
+                    j[b] = f < (double)cc[b] ? cc[b] : (f > (double)(cc[b] + osz - 1) ? cc[b] + osz - 1 : (int)f);
+                }
+            }
+            // a neighbour that is not a leaf has the current level
+            oct_enter(nb, olev, j[0], j[1], j[2]);
+            set_faces(1 << (OL - olev));
+        } else {
+            cur_m = mn;
+            kr_cur = kr_next;
+            const int cn = ca + sa;
+            const int off = axis == 0 ? 0 : (axis == 1 ? nx + 1 : nx + 1 + ny + 1);
+            const double xa = axis == 0 ? x0 : (axis == 1 ? x1 : x2);
+            const double iva = axis == 0 ? iv0 : (axis == 1 ? iv1 : iv2);
+            const double tnew = clip0((__ldg(faces + off + cn + (sa > 0)) - xa) * iva);
+            c0 = axis == 0 ? cn : c0;
+            c1 = axis == 1 ? cn : c1;
+            c2 = axis == 2 ? cn : c2;
+            tn0 = axis == 0 ? tnew : tn0;
+            tn1 = axis == 1 ? tnew : tn1;
+            tn2 = axis == 2 ? tnew : tn2;
+        }
     };
 
     auto flush_ledger = [&]() {
-        if (led_lam >= 0) {
-            double* lg = A.ledger + 4 * (size_t)led_lam;
-            atomicAdd(lg + 0, l_emit);
-            atomicAdd(lg + 1, l_abs);
-            atomicAdd(lg + 2, l_esc);
-            atomicAdd(lg + 3, l_res);
+        const int ll = I(I_LAM);
+        if (ll >= 0) {
+            double* lg = A.ledger + 4 * (size_t)ll;
+            atomicAdd(lg + 0, D(D_L_EMIT));
+            atomicAdd(lg + 1, D(D_L_ABS));
+            atomicAdd(lg + 2, D(D_L_ESC));
+            atomicAdd(lg + 3, D(D_L_RES));
         }
-        l_emit = l_abs = l_esc = l_res = 0.0;
+        D(D_L_EMIT) = D(D_L_ABS) = D(D_L_ESC) = D(D_L_RES) = 0.0;
+    };
+
+    auto flush_counters = [&]() {
+        atomicAdd(A.counters + 0, (unsigned long long)(unsigned)I(I_C_SCAT));
+        atomicAdd(A.counters + 1, (unsigned long long)(unsigned)I(I_C_DEP));
+        atomicAdd(A.counters + 2, (unsigned long long)(unsigned)I(I_C_LOC));
+        atomicAdd(A.counters + 3, (unsigned long long)(unsigned)I(I_C_PEEL));
+        I(I_C_DEP) = I(I_C_LOC) = I(I_C_PEEL) = I(I_C_SCAT) = 0;
     };
 
     auto draw = [&](uint32_t event, uint32_t block) -> uint4 {
-        return philox10(make_uint4(pk, (uint32_t)lam, event, (A.phase << 24) | block), A.key0, A.key1);
+        return philox10(make_uint4((unsigned)I(I_PK), (uint32_t)lam, event, (A.phase << 24) | block), A.key0, A.key1);
+    };
+
+    // Event handling: one pass over the stages in the order a packet meets them,
+    // from the end of a traversal to the start of the next.  A lane goes round
+    // again only where no traversal came of a pass (a peel-off of zero weight).
+    auto events = [&]() {
+        int need;
+        do {
+            need = M_NONE;
+            if (stage == ST_PEEL_DONE) {
+                I(I_C_PEEL) += (int)nsteps;
+                const int pk = I(I_PEEL_I), pi = pk & (PEEL_SCATTER - 1);
+                const InstrDev& S = sins[pi];
+                const double w = D(D_PEEL_W);
+                if (w > 0.0) {
+                    const double flux = w * exp(-tau) * S.flux_norm;
+                    D(D_P_PEEL) += flux;
+                    const double a = x0 * S.e1[0] + x1 * S.e1[1] + x2 * S.e1[2];
+                    const double b = x0 * S.e2[0] + x1 * S.e2[1] + x2 * S.e2[2];
+                    const double fa = floor((a + S.half_fov) * S.inv_dpx);
+                    const double fb = floor((b + S.half_fov) * S.inv_dpx);
+                    if (fa >= 0.0 && fa < (double)S.npx && fb >= 0.0 && fb < (double)S.npx) {
+                        const long long pix = (long long)fb * S.npx + (long long)fa;
+                        atomicAdd(A.images + S.img_off + pix * NL + lam, flux);
+                    } else {
+                        atomicAdd(A.oof + (size_t)pi * NL + lam, flux);
+                    }
+                }
+                I(I_PEEL_I) = pk + 1;
+                stage = pi + 1 < A.ninstr ? ST_PEEL : (pk & PEEL_SCATTER ? ST_AFTER_SCATTER : ST_START_DEP);
+            } else if (stage == ST_DEPOSIT_DONE) {
+                I(I_C_DEP) += (int)nsteps;
+                const double om = -expm1(-tau);  // what the path takes
+                D(D_P_ESC) += L * exp(-tau);
+                D(D_P_ABS) += D(D_LABS) * om;
+                if (!(tau > 0.0)) {
+                    if (!(tau == 0.0)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
+                    L = 0.0;
+                    I(I_NSCAT) = I(I_EV) - 1;
+                    stage = ST_END_PACKET;
+                } else {
+                    // forced scattering: tau_int from the exponential truncated at tau_path
+                    const uint4 r = draw((unsigned)I(I_EV), 0u);
+                    I(I_RY) = (int)r.y;
+                    I(I_RZ) = (int)r.z;
+                    D(D_OM) = om;
+                    par = -log1p(-(double)u01f(r.x) * om);
+                    // the search: position and direction of the deposit traversal just
+                    // ended, from its start
+                    mode = M_LOCATE;
+                    tn0 = D(D_B_T0); tn1 = D(D_B_T1); tn2 = D(D_B_T2);
+                    c0 = I(I_B_0); c1 = I(I_B_1); c2 = I(I_B_2);
+                    if (OCT) {
+                        oct_enter(I(I_B_M), 0, c0, c1, c2);
+                    } else {
+                        cur_m = I(I_B_M);
+                        kr_cur = __ldg(A.kr64 + cur_m);
+                    }
+                    tcur = 0.0;
+                    tau = 0.0;
+                    nsteps = 0;
+                    found = false;
+                    last_dusty_end = 0.0;
+                    stage = ST_LOCATE_DONE;
+                    break;
+                }
+            } else if (stage == ST_LOCATE_DONE) {
+                I(I_C_LOC) += (int)nsteps;
+                const double s = found ? s_found : last_dusty_end;
+                x0 += s * k0;
+                x1 += s * k1;
+                x2 += s * k2;
+                have_pc = found;
+                if (found) {
+                    pc0 = c0; pc1 = c1; pc2 = c2;
+                    pc_node = onode;
+                }
+                L = L * D(D_ALB) * D(D_OM);
+                I(I_NSCAT) = I(I_EV);
+                if (L > 0.0 && A.peel && A.ninstr > 0) {
+                    I(I_PEEL_I) = PEEL_SCATTER;
+                    stage = ST_PEEL;
+                } else {
+                    stage = ST_AFTER_SCATTER;
+                }
+            }
+
+            if (stage == ST_AFTER_SCATTER) {
+                if (L <= A.w_min * D(D_L0)) {
+                    D(D_P_RES) += L;
+                    stage = ST_END_PACKET;
+                } else if (I(I_EV) >= A.max_events) {
+                    atomicOr(A.err, (unsigned)ERRBIT_EVENT_CAP);
+                    D(D_P_RES) += L;
+                    stage = ST_END_PACKET;
+                } else {
+                    // Henyey-Greenstein scattering: mu by inverse CDF, azimuth uniform
+                    const double mu = hg_mu<double>(gg, (double)u01f((unsigned)I(I_RY)));
+                    double sp, cp;
+                    sincospi(2.0 * (double)u01f((unsigned)I(I_RZ)), &sp, &cp);
+                    hg_rotate<double>(k0, k1, k2, mu, sp, cp);
+                    stage = ST_START_DEP;
+                }
+            }
+
+            if (stage == ST_END_PACKET) {
+                I(I_C_SCAT) += I(I_NSCAT);
+                if ((unsigned)(I(I_C_SCAT) | I(I_C_DEP) | I(I_C_LOC) | I(I_C_PEEL)) >> 30) flush_counters();
+                const double pe = D(D_P_ESC), pa = D(D_P_ABS), pr = D(D_P_RES), pp = D(D_P_PEEL);
+                D(D_L_ABS) += pa;
+                D(D_L_ESC) += pe;
+                D(D_L_RES) += pr;
+                if (!isfinite(pe + pa + pr + pp)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
+                const uint32_t li = (uint32_t)I(I_PK) - (uint32_t)__ldg(A.pk_first + lam);  // index within this call
+                if (li < (uint32_t)A.nrec) {
+                    double* rec = A.records + ((size_t)lam * A.nrec + li) * SKIRT_REC_FIELDS;
+                    rec[0] = (double)I(I_NSCAT);
+                    rec[1] = pe;
+                    rec[2] = pa;
+                    rec[3] = pr;
+                    rec[4] = pp;
+                    rec[5] = x0;
+                    rec[6] = x1;
+                    rec[7] = x2;
+                }
+                stage = ST_NEW;
+            }
+
+            if (stage == ST_NEW) {
+                if (I(I_LEFT) == 0) {
+                    unsigned long long q;
+                    if (!A.persistent) {
+                        q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+                        if (started || q >= A.q_count) { alive = false; break; }
+                        started = true;
+                        q += A.q_base;
+                        I(I_LEFT) = 1;
+                    } else {
+                        // warp-aggregated refill from the global work queue
+                        const unsigned mask = __activemask();
+                        const int lane = threadIdx.x & 31;
+                        const int leader = __ffs(mask) - 1;
+                        const unsigned rank = __popc(mask & ((1u << lane) - 1u));
+                        unsigned long long base = 0;
+                        if (lane == leader)
+                            base = atomicAdd(A.queue, (unsigned long long)__popc(mask) * (unsigned long long)A.chunk);
+                        base = __shfl_sync(mask, base, leader);
+                        q = base + (unsigned long long)rank * A.chunk;
+                        if (q >= A.total) { alive = false; break; }
+                        I(I_LEFT) = (int)(A.total - q < (unsigned long long)A.chunk ? A.total - q : A.chunk);
+                    }
+                    I(I_QLO) = (int)(unsigned)q;
+                    I(I_QHI) = (int)(unsigned)(q >> 32);
+                }
+                I(I_LEFT) -= 1;
+                const unsigned long long qq = ((unsigned long long)(unsigned)I(I_QHI) << 32) | (unsigned)I(I_QLO);
+                I(I_QLO) = (int)(unsigned)(qq + 1);
+                I(I_QHI) = (int)(unsigned)((qq + 1) >> 32);
+                int ll = I(I_LAM);
+                if (ll < 0 || qq < __ldg(A.offsets + ll) || qq >= __ldg(A.offsets + ll + 1)) {
+                    int a = 0, b = NL - 1;  // last wavelength whose offset <= qq
+                    while (a < b) {
+                        const int mid = (a + b + 1) >> 1;
+                        if (__ldg(A.offsets + mid) <= qq) a = mid; else b = mid - 1;
+                    }
+                    flush_ledger();
+                    ll = a;
+                    I(I_LAM) = ll;
+                    D(D_ALB) = __ldg(A.albedo + ll);
+                    D(D_L0) = __ldg(A.L0 + ll);
+                }
+                lam = ll;
+                krs = __ldg(A.kscale + lam);
+                unit = bits(krs) == 0x3FF0000000000000ll;
+                gg = __ldg(A.g + lam);
+                I(I_PK) = (int)(uint32_t)(qq - __ldg(A.offsets + lam) + __ldg(A.pk_first + lam));
+                L = D(D_L0);
+                D(D_P_ESC) = D(D_P_ABS) = D(D_P_RES) = D(D_P_PEEL) = 0.0;
+                I(I_EV) = 0;
+                I(I_NSCAT) = 0;
+                D(D_L_EMIT) += L;
+                have_pc = false;
+
+                // ---- launch (Sect. 3.2): position from the source, isotropic direction
+                bool isotropic = true;
+                if (A.src_kind == SKIRT_SRC_BEAM) {
+                    x0 = A.src_pos[0]; x1 = A.src_pos[1]; x2 = A.src_pos[2];
+                    k0 = A.src_dir[0]; k1 = A.src_dir[1]; k2 = A.src_dir[2];
+                    isotropic = false;
+                } else if (A.src_kind == SKIRT_SRC_DISK) {
+                    for (uint32_t tries = 0;; ++tries) {
+                        const uint4 r = draw(0u, tries == 0 ? 0u : tries + 1u);
+                        const double u0 = u01f(r.x), u1 = u01f(r.y), u2 = u01f(r.z), u3 = u01f(r.w);
+                        const double Rr = -A.h_R * (log(u0) + log(u1));
+                        const double z = (u2 < 0.5) ? A.h_z * log(2.0 * u2) : -A.h_z * log(2.0 * (1.0 - u2));
+                        double sp, cp;
+                        sincospi(2.0 * u3, &sp, &cp);
+                        x0 = A.src_pos[0] + Rr * cp;
+                        x1 = A.src_pos[1] + Rr * sp;
+                        x2 = A.src_pos[2] + z;
+                        const bool inside = x0 >= A.lo[0] && x0 <= A.hi[0] && x1 >= A.lo[1] && x1 <= A.hi[1] &&
+                                            x2 >= A.lo[2] && x2 <= A.hi[2];
+                        if (inside) break;
+                        if (tries + 1 >= 64) {
+                            atomicOr(A.err, (unsigned)ERRBIT_SOURCE);
+                            x0 = A.src_pos[0]; x1 = A.src_pos[1]; x2 = A.src_pos[2];
+                            break;
+                        }
+                    }
+                } else if (A.src_kind == SKIRT_SRC_DUST) {
+                    const uint4 r = draw(0u, 0u);
+                    const long long a = dust_cell(A, lam, (double)u01f(r.x));
+                    if (OCT) {
+                        // uniform point in the leaf's box
+                        const int4 lf = __ldg(&A.oct_leaf[a]);
+                        const double side = (double)(1 << (OL - lf.w));
+                        x0 = A.lo[0] + ((double)lf.x + (double)u01f(r.y) * side) * A.d[0];
+                        x1 = A.lo[1] + ((double)lf.y + (double)u01f(r.z) * side) * A.d[1];
+                        x2 = A.lo[2] + ((double)lf.z + (double)u01f(r.w) * side) * A.d[2];
+                    } else {
+                        const int ix = (int)(a % nx), iy = (int)((a / nx) % ny), iz = (int)(a / ((long long)nx * ny));
+                        x0 = A.lo[0] + ((double)ix + (double)u01f(r.y)) * A.d[0];
+                        x1 = A.lo[1] + ((double)iy + (double)u01f(r.z)) * A.d[1];
+                        x2 = A.lo[2] + ((double)iz + (double)u01f(r.w)) * A.d[2];
+                    }
+                } else {
+                    x0 = A.src_pos[0]; x1 = A.src_pos[1]; x2 = A.src_pos[2];
+                }
+                stage = ST_START_DEP;
+                if (isotropic) {
+                    const uint4 r = draw(0u, 1u);
+                    const double mu = 2.0 * (double)u01f(r.x) - 1.0;
+                    const double st = sqrt(fmax(1.0 - mu * mu, 0.0));
+                    double sp, cp;
+                    sincospi(2.0 * (double)u01f(r.y), &sp, &cp);
+                    k0 = st * cp; k1 = st * sp; k2 = mu;
+                    if (A.peel && A.ninstr > 0) {
+                        I(I_PEEL_I) = 0;
+                        stage = ST_PEEL;
+                    }
+                }
+            }
+
+            double w0 = k0, w1 = k1, w2 = k2, i0 = 0.0, i1 = 0.0, i2 = 0.0;  // the traversal to start
+            if (stage == ST_PEEL) {
+                const int pk = I(I_PEEL_I);
+                const InstrDev& S = sins[pk & (PEEL_SCATTER - 1)];
+                double w = L;  // isotropic emission: phase factor 1
+                if (pk & PEEL_SCATTER) {
+                    const double mu = k0 * S.kobs[0] + k1 * S.kobs[1] + k2 * S.kobs[2];
+                    w = L * hg_phase<double>(gg, mu);
+                }
+                D(D_PEEL_W) = w;
+                stage = ST_PEEL_DONE;
+                nsteps = 0;
+                if (w > 0.0) {
+                    need = M_PEEL;
+                    w0 = S.kobs[0]; w1 = S.kobs[1]; w2 = S.kobs[2];
+                    i0 = S.ikobs[0]; i1 = S.ikobs[1]; i2 = S.ikobs[2];
+                }
+            } else if (stage == ST_START_DEP) {
+                I(I_EV) += 1;
+                par = L * (1.0 - D(D_ALB));
+                D(D_LABS) = par;
+                need = M_DEPOSIT;
+                i0 = k0 != 0.0 ? 1.0 / k0 : 0.0;
+                i1 = k1 != 0.0 ? 1.0 / k1 : 0.0;
+                i2 = k2 != 0.0 ? 1.0 / k2 : 0.0;
+                stage = ST_DEPOSIT_DONE;
+            }
+            if (need != M_NONE) {
+                begin(need, w0, w1, w2, i0, i1, i2);
+                if (need == M_DEPOSIT) {
+                    D(D_B_T0) = tn0; D(D_B_T1) = tn1; D(D_B_T2) = tn2;
+                    I(I_B_0) = c0; I(I_B_1) = c1; I(I_B_2) = c2;
+                    I(I_B_M) = OCT ? onode : cur_m;
+                }
+            }
+        } while (need == M_NONE);
+    };
+
+    // FP64_ROUND crossings of the lanes in one kind of traversal
+    auto round = [&](auto kind) {
+        constexpr bool PEEL = decltype(kind)::value;
+#pragma unroll 1
+        for (int r = 0; r < FP64_ROUND; ++r) {
+            if (PEEL ? mode == M_PEEL : (mode == M_DEPOSIT || mode == M_LOCATE)) step(kind);
+            __syncwarp();
+        }
     };
 
     for (;;) {
-        if (mode != M_NONE) {
-            // ---------------- one cell crossing ----------------
-            int osz = 1;
-            if (OCT) {
-                // exit distances from the current leaf's box
-                osz = 1 << (OL - olev);
-                tn0 = s0 ? face_dist<R>(lo0, c0 + (s0 > 0 ? osz : 0), d0, o0, iv0) : INF;
-                tn1 = s1 ? face_dist<R>(lo1, c1 + (s1 > 0 ? osz : 0), d1, o1, iv1) : INF;
-                tn2 = s2 ? face_dist<R>(lo2, c2 + (s2 > 0 ? osz : 0), d2, o2, iv2) : INF;
-            }
-            const int axis = (tn0 <= tn1) ? ((tn0 <= tn2) ? 0 : 2) : ((tn1 <= tn2) ? 1 : 2);
-            const R tnext = axis == 0 ? tn0 : (axis == 1 ? tn1 : tn2);
-            R ds = tnext - tcur;
-            if (ds < (R)0) ds = (R)0;
-            const int m = OCT ? oleaf : (c2 * ny + c1) * nx + c0;
-            const R krl = (OCT ? (R)okr : P<R>::kr(A, m)) * krs;
-            const R dtau_r = krl * ds;
-            const double dtau = (double)dtau_r;
-            bool done = false;
-            if (mode == M_DEPOSIT) {
-                ++c_dep;
-                if (dtau_r > (R)0) {
-                    const double dep = labs * P<R>::dep_factor(tau, dtau_r);
-                    if (dep > 0.0) {
-                        atomicAdd(A.absorbed + ((size_t)m * A.abs_cs + (size_t)lam * A.abs_ls), dep);
-                        p_abs += dep;
-                    }
-                }
-                tau += dtau;
-            } else if (mode == M_LOCATE) {
-                ++c_loc;
-                if (krl > (R)0 && tau + dtau >= tau_t) {
-                    s_found = tcur + (R)(tau_t - tau) / krl;
-                    found = true;
-                    done = true;
-                } else {
-                    tau += dtau;
-                    if (krl > (R)0) last_dusty_end = tnext;
-                }
+        const unsigned pm = __ballot_sync(0xffffffffu, mode == M_PEEL);
+        const unsigned dm = __ballot_sync(0xffffffffu, mode == M_DEPOSIT || mode == M_LOCATE);
+        const unsigned wm = __ballot_sync(0xffffffffu, mode == M_NONE && alive);
+        if (!(pm | dm | wm)) break;
+        const int np = __popc(pm), nd = __popc(dm);
+        if (max(np, nd) >= FP64_STEP_MIN || !wm) {
+            if (np >= nd) {
+                round(std::true_type{});
             } else {
-                ++c_peel;
-                tau += dtau;
-            }
-            if (!done && OCT) {
-                tcur = tnext;
-                const int sa = axis == 0 ? s0 : (axis == 1 ? s1 : s2);
-                const int nb = __ldg(&A.oct_nodes[onode].nb[2 * axis + (sa > 0)]);
-                if (nb < 0) {
-                    done = true;  // the exit face lies on the root box
-                } else if (++osteps > A.oct_step_cap) {
-                    atomicOr(A.err, (unsigned)ERRBIT_PATH);
-                    done = true;
-                } else {
-                    // lattice cell of the entry point into the next leaf: across
-                    // the exit face along `axis`; along the other axes the
-                    // cell of the crossing point, kept within the current
-                    // leaf's cross-section
-                    int j[3];
-                    const int cc[3] = {c0, c1, c2};
-                    const R oo[3] = {o0, o1, o2}, vv[3] = {v0, v1, v2}, ll[3] = {lo0, lo1, lo2},
-                            dd[3] = {d0, d1, d2};
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) {
-                        if (b == axis) {
-                            j[b] = sa > 0 ? cc[b] + osz : cc[b] - 1;
-                        } else {
-                            const R f = P<R>::floorr((oo[b] + tnext * vv[b] - ll[b]) / dd[b]);
-                            const int jb = f < (R)cc[b] ? cc[b] : (f > (R)(cc[b] + osz - 1) ? cc[b] + osz - 1 : (int)f);
-                            j[b] = jb;
-                        }
-                    }
-                    // a neighbour that is not a leaf has the current level
-                    oct_enter(nb, olev, j[0], j[1], j[2]);
-                }
-            } else if (!done) {
-                tcur = tnext;
-                if (axis == 0) {
-                    c0 += s0;
-                    if ((unsigned)c0 >= (unsigned)nx) done = true;
-                    else tn0 = face_dist<R>(lo0, c0 + (s0 > 0), d0, o0, iv0);
-                } else if (axis == 1) {
-                    c1 += s1;
-                    if ((unsigned)c1 >= (unsigned)ny) done = true;
-                    else tn1 = face_dist<R>(lo1, c1 + (s1 > 0), d1, o1, iv1);
-                } else {
-                    c2 += s2;
-                    if ((unsigned)c2 >= (unsigned)nz) done = true;
-                    else tn2 = face_dist<R>(lo2, c2 + (s2 > 0), d2, o2, iv2);
-                }
-            }
-            if (done) mode = M_NONE;
-            continue;
-        }
-
-        // ---------------- event handling ----------------
-        if (stage == ST_NEW) {
-            if (q >= q_end) {
-                if (!A.persistent) {
-                    if (started) break;
-                    started = true;
-                    q = A.q_base + (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-                    q_end = (q < A.q_base + A.q_count) ? q + 1 : q;
-                    if (q >= q_end) break;
-                } else {
-                    // warp-aggregated refill from the global work queue
-                    const unsigned mask = __activemask();
-                    const int lane = threadIdx.x & 31;
-                    const int leader = __ffs(mask) - 1;
-                    const unsigned rank = __popc(mask & ((1u << lane) - 1u));
-                    unsigned long long base = 0;
-                    if (lane == leader)
-                        base = atomicAdd(A.queue, (unsigned long long)__popc(mask) * (unsigned long long)A.chunk);
-                    base = __shfl_sync(mask, base, leader);
-                    q = base + (unsigned long long)rank * A.chunk;
-                    if (q >= A.total) break;
-                    q_end = q + A.chunk;
-                    if (q_end > A.total) q_end = A.total;
-                }
-            }
-            const unsigned long long qq = q++;
-            if (lam < 0 || qq < __ldg(A.offsets + lam) || qq >= __ldg(A.offsets + lam + 1)) {
-                int a = 0, b = NL - 1;  // last wavelength whose offset <= qq
-                while (a < b) {
-                    const int mid = (a + b + 1) >> 1;
-                    if (__ldg(A.offsets + mid) <= qq) a = mid; else b = mid - 1;
-                }
-                lam = a;
-                krs = (R)__ldg(A.kscale + lam);
-                alb = __ldg(A.albedo + lam);
-                gg = (R)__ldg(A.g + lam);
-                L0 = __ldg(A.L0 + lam);
-                if (led_lam != lam) {
-                    flush_ledger();
-                    led_lam = lam;
-                }
-            }
-            pk = (uint32_t)(qq - __ldg(A.offsets + lam) + __ldg(A.pk_first + lam));
-            L = L0;
-            p_esc = p_abs = p_res = p_peel = 0.0;
-            ev = 0;
-            nscat = 0;
-            l_emit += L0;
-
-            // ---- launch (Sect. 3.2): position from the source, isotropic direction
-            bool isotropic = true;
-            if (A.src_kind == SKIRT_SRC_BEAM) {
-                x0 = (R)A.src_pos[0]; x1 = (R)A.src_pos[1]; x2 = (R)A.src_pos[2];
-                k0 = (R)A.src_dir[0]; k1 = (R)A.src_dir[1]; k2 = (R)A.src_dir[2];
-                isotropic = false;
-            } else if (A.src_kind == SKIRT_SRC_DISK) {
-                const R hR = (R)A.h_R, hz = (R)A.h_z;
-                for (uint32_t tries = 0;; ++tries) {
-                    const uint4 r = draw(0u, tries == 0 ? 0u : tries + 1u);
-                    const R u0 = P<R>::u(r.x), u1 = P<R>::u(r.y), u2 = P<R>::u(r.z), u3 = P<R>::u(r.w);
-                    const R Rr = -hR * (P<R>::logr(u0) + P<R>::logr(u1));
-                    const R z = (u2 < (R)0.5) ? hz * P<R>::logr((R)2 * u2) : -hz * P<R>::logr((R)2 * ((R)1 - u2));
-                    R sp, cp;
-                    P<R>::sincospi2(u3, &sp, &cp);
-                    x0 = (R)A.src_pos[0] + Rr * cp;
-                    x1 = (R)A.src_pos[1] + Rr * sp;
-                    x2 = (R)A.src_pos[2] + z;
-                    const bool inside = x0 >= lo0 && x0 <= (R)A.hi[0] && x1 >= lo1 && x1 <= (R)A.hi[1] &&
-                                        x2 >= lo2 && x2 <= (R)A.hi[2];
-                    if (inside) break;
-                    if (tries + 1 >= 64) {
-                        atomicOr(A.err, (unsigned)ERRBIT_SOURCE);
-                        x0 = (R)A.src_pos[0]; x1 = (R)A.src_pos[1]; x2 = (R)A.src_pos[2];
-                        break;
-                    }
-                }
-            } else if (A.src_kind == SKIRT_SRC_DUST) {
-                const uint4 r = draw(0u, 0u);
-                const long long a = dust_cell(A, lam, (double)u01f(r.x));
-                if (OCT) {
-                    // uniform point in the leaf's box
-                    const int4 lf = __ldg(&A.oct_leaf[a]);
-                    const R side = (R)(1 << (OL - lf.w));
-                    x0 = lo0 + ((R)lf.x + P<R>::u(r.y) * side) * d0;
-                    x1 = lo1 + ((R)lf.y + P<R>::u(r.z) * side) * d1;
-                    x2 = lo2 + ((R)lf.z + P<R>::u(r.w) * side) * d2;
-                } else {
-                    const int ix = (int)(a % nx), iy = (int)((a / nx) % ny), iz = (int)(a / ((long long)nx * ny));
-                    x0 = lo0 + ((R)ix + P<R>::u(r.y)) * d0;
-                    x1 = lo1 + ((R)iy + P<R>::u(r.z)) * d1;
-                    x2 = lo2 + ((R)iz + P<R>::u(r.w)) * d2;
-                }
-            } else {
-                x0 = (R)A.src_pos[0]; x1 = (R)A.src_pos[1]; x2 = (R)A.src_pos[2];
-            }
-            if (isotropic) {
-                const uint4 r = draw(0u, 1u);
-                const R mu = (R)2 * P<R>::u(r.x) - (R)1;
-                const R st = P<R>::sqrtr(fmax((R)1 - mu * mu, (R)0));
-                R sp, cp;
-                P<R>::sincospi2(P<R>::u(r.y), &sp, &cp);
-                k0 = st * cp; k1 = st * sp; k2 = mu;
-            }
-            if (isotropic && A.peel && A.ninstr > 0) {
-                // emission peel-off: isotropic emission, phase factor 1
-                peel_kind = 0;
-                peel_i = 0;
-                peel_w = L;
-                after_peel = ST_START_DEP;
-                stage = ST_PEEL_DONE;
-                if (peel_w > 0.0) {
-                    const InstrDev& I = sins[0];
-                    begin(M_PEEL, x0, x1, x2, P<R>::kobs(I, 0), P<R>::kobs(I, 1), P<R>::kobs(I, 2));
-                } else {
-                    tau = 0.0;
-                }
-            } else {
-                stage = ST_START_DEP;
+                // e^{-tau} afresh, so that the subtractions of at most a round's deposits
+                // stand between it and a deposit
+                if (mode == M_DEPOSIT && bits(tau) > 0) par = D(D_LABS) * exp(-tau);
+                __syncwarp();
+                round(std::false_type{});
             }
             continue;
         }
-
-        if (stage == ST_START_DEP) {
-            ++ev;
-            labs = L * (1.0 - alb);
-            begin(M_DEPOSIT, x0, x1, x2, k0, k1, k2);
-            stage = ST_DEPOSIT_DONE;
-            continue;
-        }
-
-        if (stage == ST_DEPOSIT_DONE) {
-            tau_path = tau;
-            p_esc += L * exp(-tau_path);
-            if (!(tau_path > 0.0)) {
-                if (!(tau_path == 0.0)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
-                L = 0.0;
-                nscat = (int)ev - 1;
-                stage = ST_END_PACKET;
-                continue;
-            }
-            // forced scattering: tau_int from the exponential truncated at tau_path
-            const uint4 r = draw(ev, 0u);
-            const double u0 = (double)u01f(r.x);
-            tau_t = -log1p(-u0 * (-expm1(-tau_path)));
-            begin(M_LOCATE, x0, x1, x2, k0, k1, k2);
-            last_dusty_end = (R)0;
-            found = false;
-            stage = ST_LOCATE_DONE;
-            continue;
-        }
-
-        if (stage == ST_LOCATE_DONE) {
-            const R s = found ? s_found : last_dusty_end;
-            x0 += s * k0;
-            x1 += s * k1;
-            x2 += s * k2;
-            L = L * alb * (-expm1(-tau_path));
-            nscat = (int)ev;
-            if (L > 0.0 && A.peel && A.ninstr > 0) {
-                peel_kind = 1;
-                peel_i = 0;
-                const InstrDev& I = sins[0];
-                const R mu = k0 * P<R>::kobs(I, 0) + k1 * P<R>::kobs(I, 1) + k2 * P<R>::kobs(I, 2);
-                peel_w = L * (double)hg_phase<R>(gg, mu);
-                after_peel = ST_AFTER_SCATTER;
-                stage = ST_PEEL_DONE;
-                begin(M_PEEL, x0, x1, x2, P<R>::kobs(I, 0), P<R>::kobs(I, 1), P<R>::kobs(I, 2));
-            } else {
-                stage = ST_AFTER_SCATTER;
-            }
-            continue;
-        }
-
-        if (stage == ST_PEEL_DONE) {
-            const InstrDev& I = sins[peel_i];
-            if (peel_w > 0.0) {
-                const double flux = peel_w * exp(-tau) * I.flux_norm;
-                p_peel += flux;
-                const R a = x0 * P<R>::e1(I, 0) + x1 * P<R>::e1(I, 1) + x2 * P<R>::e1(I, 2);
-                const R b = x0 * P<R>::e2(I, 0) + x1 * P<R>::e2(I, 1) + x2 * P<R>::e2(I, 2);
-                const R fa = P<R>::floorr((a + P<R>::half_fov(I)) * P<R>::inv_dpx(I));
-                const R fb = P<R>::floorr((b + P<R>::half_fov(I)) * P<R>::inv_dpx(I));
-                if (fa >= (R)0 && fa < (R)I.npx && fb >= (R)0 && fb < (R)I.npx) {
-                    const long long pix = (long long)fb * I.npx + (long long)fa;
-                    atomicAdd(A.images + I.img_off + pix * NL + lam, flux);
-                } else {
-                    atomicAdd(A.oof + (size_t)peel_i * NL + lam, flux);
-                }
-            }
-            ++peel_i;
-            if (peel_i < A.ninstr) {
-                const InstrDev& J = sins[peel_i];
-                if (peel_kind == 0) {
-                    peel_w = L;
-                } else {
-                    const R mu = k0 * P<R>::kobs(J, 0) + k1 * P<R>::kobs(J, 1) + k2 * P<R>::kobs(J, 2);
-                    peel_w = L * (double)hg_phase<R>(gg, mu);
-                }
-                if (peel_w > 0.0) begin(M_PEEL, x0, x1, x2, P<R>::kobs(J, 0), P<R>::kobs(J, 1), P<R>::kobs(J, 2));
-            } else {
-                stage = after_peel;
-            }
-            continue;
-        }
-
-        if (stage == ST_AFTER_SCATTER) {
-            if (L <= A.w_min * L0) {
-                p_res += L;
-                stage = ST_END_PACKET;
-            } else if ((int)ev >= A.max_events) {
-                atomicOr(A.err, (unsigned)ERRBIT_EVENT_CAP);
-                p_res += L;
-                stage = ST_END_PACKET;
-            } else {
-                // Henyey-Greenstein scattering: mu by inverse CDF, azimuth uniform
-                const uint4 r = draw(ev, 0u);
-                const R mu = hg_mu<R>(gg, P<R>::u(r.y));
-                R sp, cp;
-                P<R>::sincospi2(P<R>::u(r.z), &sp, &cp);
-                hg_rotate<R>(k0, k1, k2, mu, sp, cp);
-                stage = ST_START_DEP;
-            }
-            continue;
-        }
-
-        // ST_END_PACKET
-        c_scat += (unsigned long long)nscat;
-        l_abs += p_abs;
-        l_esc += p_esc;
-        l_res += p_res;
-        if (!isfinite(p_esc + p_abs + p_res + p_peel)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
-        const uint32_t li = pk - (uint32_t)__ldg(A.pk_first + lam);  // index within this call
-        if (li < (uint32_t)A.nrec) {
-            double* rec = A.records + ((size_t)lam * A.nrec + li) * SKIRT_REC_FIELDS;
-            rec[0] = (double)nscat;
-            rec[1] = p_esc;
-            rec[2] = p_abs;
-            rec[3] = p_res;
-            rec[4] = p_peel;
-            rec[5] = (double)x0;
-            rec[6] = (double)x1;
-            rec[7] = (double)x2;
-        }
-        stage = ST_NEW;
+        if (mode == M_NONE && alive) events();
     }
 
     flush_ledger();
-    atomicAdd(A.counters + 0, c_scat);
-    atomicAdd(A.counters + 1, c_dep);
-    atomicAdd(A.counters + 2, c_loc);
-    atomicAdd(A.counters + 3, c_peel);
+    flush_counters();
 }
 
 // SED = sum over the pixels of every image plus the out-of-frame peel-offs.
@@ -559,32 +662,40 @@ __global__ void f32_to_f64_kernel(const float* __restrict__ in, double* __restri
 
 }  // namespace
 
-// The FP64 form keeps only the instruments in shared memory.  Its lanes run
-// independent state machines with no point where the warp is known to be
-// converged, so its peel-off tallies are plain reductions.
 size_t trace_smem_bytes(int ninstr, int block)
 {
-    (void)block;
-    return sizeof(InstrDev) * (size_t)ninstr;
+    return sizeof(InstrDev) * (size_t)ninstr + (sizeof(double) * D_NUM + sizeof(int) * I_NUM) * (size_t)block;
+}
+
+static cudaError_t set_smem_limit()
+{
+    const int bytes = (int)trace_smem_bytes(16, FP64_MAXB);
+    cudaError_t e = cudaFuncSetAttribute(trace_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(trace_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 cudaError_t launch_trace(const TraceArgs& a, int precision, int block, int grid, cudaStream_t s)
 {
     if (precision == SKIRT_PREC_MIXED) return launch_trace_mixed(a, block, grid, s);
+    cudaError_t e = set_smem_limit();
+    if (e != cudaSuccess) return e;
     const size_t smem = trace_smem_bytes(a.ninstr, block);
     if (a.oct_levels > 0)
-        trace_kernel<double, true><<<grid, block, smem, s>>>(a);
+        trace_kernel<true><<<grid, block, smem, s>>>(a);
     else
-        trace_kernel<double, false><<<grid, block, smem, s>>>(a);
+        trace_kernel<false><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t trace_occupancy(int precision, int block, int* blocks_per_sm, bool octree)
 {
     if (precision == SKIRT_PREC_MIXED) return trace_mixed_occupancy(block, blocks_per_sm, octree);
+    cudaError_t e = set_smem_limit();
+    if (e != cudaSuccess) return e;
     const size_t smem = trace_smem_bytes(16, block);
-    return octree ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_kernel<double, true>, block, smem)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_kernel<double, false>, block, smem);
+    return octree ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_kernel<true>, block, smem)
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_kernel<false>, block, smem);
 }
 
 CellOrder cell_order(int nx, int ny, int nz, int fast)
