@@ -636,12 +636,11 @@ extern "C" int skirt_mlp_train_opts_default(skirt_mlp_train_opts* o)
 namespace {
 
 // Per-call scratch of a training step: the per-CTA partial gradients and
-// losses, the loss accumulator and the reduction's block counter.
+// losses, and the loss accumulator.
 struct Work {
     float* part = nullptr;
     float* part_loss = nullptr;
     float* loss = nullptr;
-    unsigned* done = nullptr;
     cudaError_t alloc(int rows, cudaStream_t s)
     {
         const int ncta = (rows + train_rows_per_cta() - 1) / train_rows_per_cta();
@@ -649,9 +648,7 @@ struct Work {
         if ((e = cudaMallocAsync((void**)&part, sizeof(float) * (size_t)ncta * NPARAM, s))) return e;
         if ((e = cudaMallocAsync((void**)&part_loss, sizeof(float) * (size_t)ncta, s))) return e;
         if ((e = cudaMallocAsync((void**)&loss, sizeof(float), s))) return e;
-        if ((e = cudaMallocAsync((void**)&done, sizeof(unsigned), s))) return e;
-        if ((e = cudaMemsetAsync(loss, 0, sizeof(float), s))) return e;
-        return cudaMemsetAsync(done, 0, sizeof(unsigned), s);
+        return cudaMemsetAsync(loss, 0, sizeof(float), s);
     }
     void release(cudaStream_t s)
     {
@@ -659,10 +656,11 @@ struct Work {
             if (*p) cudaFreeAsync(*p, s);
             *p = nullptr;
         }
-        if (done) cudaFreeAsync(done, s);
-        done = nullptr;
     }
 };
+
+// steps per replayed graph
+constexpr int TRAIN_UNROLL = 8;
 
 // Everything a training call acquires, released on every return path (the
 // stream-ordered frees go on the caller's stream, after the private stream's
@@ -680,7 +678,8 @@ struct TrainScope {
     cudaStream_t cs = nullptr;
     cudaEvent_t ready = nullptr;
     cudaGraph_t graph = nullptr;
-    cudaGraphExec_t gexec = nullptr;
+    cudaGraphExec_t gexec = nullptr;   // TRAIN_UNROLL steps
+    cudaGraphExec_t gexec1 = nullptr;  // one step
     explicit TrainScope(cudaStream_t st) : s(st) {}
     ~TrainScope()
     {
@@ -689,6 +688,7 @@ struct TrainScope {
             cudaStreamSynchronize(cs);
         }
         if (gexec) cudaGraphExecDestroy(gexec);
+        if (gexec1) cudaGraphExecDestroy(gexec1);
         if (graph) cudaGraphDestroy(graph);
         if (cs) cudaStreamDestroy(cs);
         if (ready) cudaEventDestroy(ready);
@@ -722,7 +722,7 @@ extern "C" int skirt_mlp_grad(skirt_mlp_t net, const float* x_std, const float* 
     MCK(cudaMemcpyAsync(d_t, target, sizeof(float) * (size_t)n * NO, cudaMemcpyDefault, s));
     if (int r = repack(net, s)) return r;
     MCK(launch_train_step(net->Wb, net->P, nullptr, d_t, nullptr, nullptr, nullptr, 0, n, d_x, n, w.part, w.part_loss,
-                          net->G, 0, nullptr, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, nullptr, w.loss, w.done, s));
+                          net->G, 0, nullptr, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, nullptr, w.loss, 0, 0, s));
     if (grad) MCK(cudaMemcpyAsync(grad, net->G, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, s));
     float l = 0.f;
     MCK(cudaMemcpyAsync(&l, w.loss, sizeof(float), cudaMemcpyDeviceToHost, s));
@@ -818,36 +818,41 @@ extern "C" int skirt_mlp_train(skirt_mlp_t net, const float* features, const dou
 
     // the BF16 weights the first step reads
     if (int r = repack(net, s)) return r;
-    // one training step (the fused tensor-core tile kernel, then the ordered
-    // gradient sum with the Adam step and the step counter) as a CUDA graph,
-    // captured on a private stream and replayed for every step
+    // training steps (the fused tensor-core tile kernel, then the ordered gradient
+    // sum with the Adam step and the step counter) as CUDA graphs of TRAIN_UNROLL
+    // steps and of one, captured on a private stream and replayed: the device
+    // counter tells a step which rows it takes.  Within a graph a kernel starts
+    // while its predecessor ends (programmatic dependent launch).
     cudaStream_t& cs = sc.cs;
     MCK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaEvent_t& ready = sc.ready;
     MCK(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming));
     MCK(cudaEventRecord(ready, s));
     MCK(cudaStreamWaitEvent(cs, ready, 0));
-    cudaGraph_t& graph = sc.graph;
-    cudaGraphExec_t& gexec = sc.gexec;
+    const auto capture = [&](int count, cudaGraphExec_t& gexec) -> int {
+        cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+        if (e != cudaSuccess) return set_error(SKIRT_ERR_CUDA, "training graph: %s", cudaGetErrorString(e));
+        for (int k = 0; k < count && e == cudaSuccess; ++k)
+            e = launch_train_step(net->Wb, net->P, features, target, net->stats, d_ab, d_t, steps, n, nullptr, B,
+                                  w.part, w.part_loss, net->G, 1, net->P, net->Mo, net->Vo, d_sched, opts->beta1,
+                                  opts->beta2, opts->eps, net->Wb, w.loss, k, k == count - 1 ? count : 0, cs);
+        const cudaError_t ec = cudaStreamEndCapture(cs, &sc.graph);
+        if (e == cudaSuccess) e = ec;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&gexec, sc.graph, 0);
+        if (sc.graph) cudaGraphDestroy(sc.graph);
+        sc.graph = nullptr;
+        return e == cudaSuccess ? SKIRT_OK : set_error(SKIRT_ERR_CUDA, "training graph: %s", cudaGetErrorString(e));
+    };
+    const long long unrolled = steps / TRAIN_UNROLL * TRAIN_UNROLL;
+    if (unrolled > 0)
+        if (int r = capture(TRAIN_UNROLL, sc.gexec)) return r;
+    if (unrolled < steps)
+        if (int r = capture(1, sc.gexec1)) return r;
     int rc = SKIRT_OK;
-    cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        e = launch_train_step(net->Wb, net->P, features, target, net->stats, d_ab, d_t, steps, n, nullptr, B, w.part,
-                              w.part_loss, net->G, 1, net->P, net->Mo, net->Vo, d_sched, opts->beta1, opts->beta2,
-                              opts->eps, net->Wb, w.loss, w.done, cs);
-        if (e != cudaSuccess) {
-            cudaGraph_t broken = nullptr;
-            cudaStreamEndCapture(cs, &broken);
-            if (broken) cudaGraphDestroy(broken);
-            return set_error(SKIRT_ERR_CUDA, "training step launch: %s", cudaGetErrorString(e));
-        }
-        e = cudaStreamEndCapture(cs, &graph);
-    }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&gexec, graph, 0);
-    if (e != cudaSuccess) rc = set_error(SKIRT_ERR_CUDA, "training graph: %s", cudaGetErrorString(e));
     for (int ep = 0; ep < opts->epochs && rc == SKIRT_OK; ++ep) {
-        e = cudaMemsetAsync(w.loss, 0, sizeof(float), cs);
-        for (long long k = 0; k < steps && e == cudaSuccess; ++k) e = cudaGraphLaunch(gexec, cs);
+        cudaError_t e = cudaMemsetAsync(w.loss, 0, sizeof(float), cs);
+        for (long long k = 0; k < unrolled && e == cudaSuccess; k += TRAIN_UNROLL) e = cudaGraphLaunch(sc.gexec, cs);
+        for (long long k = unrolled; k < steps && e == cudaSuccess; ++k) e = cudaGraphLaunch(sc.gexec1, cs);
         if (e == cudaSuccess && loss_history) {
             float l = 0.f;
             e = cudaMemcpyAsync(&l, w.loss, sizeof(float), cudaMemcpyDeviceToHost, cs);

@@ -43,7 +43,7 @@ constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + NH * NIN, OFF_W2 = OFF_B1 + NH, OFF_
               OFF_W3 = OFF_B2 + NH, OFF_B3 = OFF_W3 + NO * NH;
 
 constexpr int TR = 32;      // rows per CTA
-constexpr int TWARPS = 8;   // warps per CTA
+constexpr int TWARPS = 16;  // warps per CTA
 // shared-memory row strides (elements), each row padded by 8 BF16 (16 bytes)
 // so that the eight rows an ldmatrix touches start in different bank groups
 constexpr int P1 = NIN + 8;   // 40
@@ -62,11 +62,32 @@ constexpr size_t S_G1 = S_D1 + 2 * TR * P2;                           // fp32 [3
 constexpr size_t S_G2 = S_G1 + 4 * TR * NH;                           // fp32 [32][128]: SiLU'(Z2), then dZ2
 constexpr size_t S_Z3 = S_G2 + 4 * TR * NH;                           // fp32 [32][104]: logits, then dZ3
 constexpr size_t S_LOSS = S_Z3 + 4 * TR * NOP;                        // fp32 [32]
-constexpr size_t S_TOTAL = S_LOSS + 4 * TR;
+constexpr size_t S_T = S_LOSS + 4 * TR;                               // fp32 [32][100]: targets
+constexpr size_t S_B = S_T + 4 * TR * NO;                             // fp32 b1 [128], b2 [128], b3 [100]
+constexpr size_t S_IDX = S_B + 4 * (NH + NH + NO);                    // int64 [32]: the rows in the data
+constexpr size_t S_TOTAL = S_IDX + 8 * TR;
 static_assert(S_TOTAL <= 227 * 1024, "shared memory of one CTA");
-static_assert(S_X % 16 == 0 && S_A1 % 16 == 0 && S_D3 % 16 == 0 && S_G1 % 16 == 0, "16-byte aligned tiles");
+static_assert(S_X % 16 == 0 && S_A1 % 16 == 0 && S_D3 % 16 == 0 && S_G1 % 16 == 0 && S_T % 16 == 0 && S_IDX % 8 == 0,
+              "16-byte aligned tiles");
 
 __device__ __forceinline__ unsigned su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Programmatic dependent launch: a kernel may start once every block of its
+// predecessor has called launch_dependents, and waits for its results in
+// wait_predecessor.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p)
 {
@@ -145,17 +166,17 @@ __device__ __forceinline__ void fwd_tile(float (&c)[4], const uint32_t (&a)[KT][
 }
 
 // dst[o][i] (o < mrows, row stride outK) = sum over the 32 rows r of D[r][o] Act[r][i]
-// for the output rows of m-tile mt and all ntiles n-tiles of i: A = D^T, B = Act,
-// both through ldmatrix.trans of the row-major tiles
+// for the output rows of m-tile mt and the n-tiles nt0 .. nt1 - 1 of i: A = D^T,
+// B = Act, both through ldmatrix.trans of the row-major tiles
 template <int SD, int SA>
-__device__ __forceinline__ void wgrad(const uint16_t* D, const uint16_t* Act, int ntiles, int mt, int outK, int mrows,
+__device__ __forceinline__ void wgrad(const uint16_t* D, const uint16_t* Act, int nt0, int nt1, int mt, int outK, int mrows,
                                       float* dst, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
     uint32_t a0[4], a1[4];
     frag_at<SD>(a0, D, 16 * mt, 0, lane);
     frag_at<SD>(a1, D, 16 * mt, 16, lane);
-    for (int np = 0; np < ntiles; np += 2) {
+    for (int np = nt0; np < nt1; np += 2) {
         float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
         uint32_t b[4];
         frag_b2t<SA>(b, Act, 0, 8 * np, lane);
@@ -187,7 +208,8 @@ struct TileArgs {
     const float* target;      // [n_data][100] row shapes
     const float* stats;       // mean[32], 1/std[32]
     const unsigned long long* ab;
-    const long long* t_dev;
+    const long long* t_dev;   // the step of the first launch of this graph
+    int ahead;                // this launch's steps after it
     long long steps, n_data;
     const float* x_std;       // direct rows [nrows][32]
     int nrows;                // rows in this batch
@@ -217,52 +239,73 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
     const int row0 = blockIdx.x * TR;
     const int nvalid = min(TR, A.nrows - row0);
 
-    // ---- stage the weights (16-byte chunks into padded rows), zero the pads
+    float* T = reinterpret_cast<float*>(sm + S_T);
+    float* SB = reinterpret_cast<float*>(sm + S_B);
+    long long* idx = reinterpret_cast<long long*>(sm + S_IDX);
+    // ---- what does not depend on the previous step, done while it ends: the rows'
+    // places in the data (32 threads: the permutation's 64-bit modulus is slow)
+    if (tid < TR) {
+        long long at = -1;
+        if (tid < nvalid) {
+            at = row0 + tid;
+            if (A.feat) {
+                const long long st = *A.t_dev + A.ahead;
+                const unsigned long long pa = A.ab[2 * (st / A.steps)], pb = A.ab[2 * (st / A.steps) + 1];
+                const unsigned long long q = (unsigned long long)((st % A.steps) * (long long)A.nrows + at);
+                at = (long long)((pa * q + pb) % (unsigned long long)A.n_data);
+            }
+        }
+        idx[tid] = at;
+    }
+    // zero what no copy fills: W3's rows 104 .. 111, and dZ3's columns 100 .. 111,
+    // which take part in the W3 products
+    for (int i = tid; i < (NOK - NOP) * (NH / 8); i += blockDim.x)
+        *reinterpret_cast<uint4*>(W3 + (NOP + i / (NH / 8)) * P2 + 8 * (i % (NH / 8))) = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i < TR * (NOK - NO); i += blockDim.x) D3[(i / (NOK - NO)) * P3 + NO + i % (NOK - NO)] = 0;
+    __syncthreads();
+    // the target shapes in T, the standardised features (bf16) in X
+    for (int i = tid; i < TR * (NO / 4); i += blockDim.x) {
+        const int r = i / (NO / 4), c = i % (NO / 4);
+        if (idx[r] >= 0) cp_async16(T + r * NO + 4 * c, A.target + idx[r] * NO + 4 * c);
+    }
+    cp_commit();
+    for (int i = tid; i < TR * NIN; i += blockDim.x) {
+        const int r = i / NIN, c = i % NIN;
+        const long long s = idx[r];
+        float v = 0.f;
+        if (s >= 0) v = A.feat ? (A.feat[s * NIN + c] - A.stats[c]) * A.stats[NIN + c] : A.x_std[s * NIN + c];
+        X[r * P1 + c] = bf16_bits(v);
+    }
+    // the dependents are let go only now, so that they start after the previous
+    // step's results are complete (the gradient sum reads its moments right away)
+    wait_predecessor();
+    launch_dependents();
+    // ---- the weights by asynchronous copies of 16 bytes into padded rows, each
+    // layer's in a group of its own, so that a layer starts when its weights are in
     {
         const uint4* src = reinterpret_cast<const uint4*>(A.Wb);
         for (int i = tid; i < NH * (NIN / 8); i += blockDim.x)
-            *reinterpret_cast<uint4*>(W1 + (i / (NIN / 8)) * P1 + 8 * (i % (NIN / 8))) = src[i];
+            cp_async16(W1 + (i / (NIN / 8)) * P1 + 8 * (i % (NIN / 8)), src + i);
+        cp_commit();
         src += NH * (NIN / 8);
         for (int i = tid; i < NH * (NH / 8); i += blockDim.x)
-            *reinterpret_cast<uint4*>(W2 + (i / (NH / 8)) * P2 + 8 * (i % (NH / 8))) = src[i];
+            cp_async16(W2 + (i / (NH / 8)) * P2 + 8 * (i % (NH / 8)), src + i);
+        cp_commit();
         src += NH * (NH / 8);
-        for (int i = tid; i < NOK * (NH / 8); i += blockDim.x) {
-            const int r = i / (NH / 8);
-            *reinterpret_cast<uint4*>(W3 + r * P2 + 8 * (i % (NH / 8))) =
-                r < NOP ? src[i] : make_uint4(0u, 0u, 0u, 0u);
-        }
-        // dZ3 columns 100..111 take part in the W3 products as zeros
-        for (int i = tid; i < TR * (NOK - NO); i += blockDim.x) D3[(i / (NOK - NO)) * P3 + NO + i % (NOK - NO)] = 0;
+        for (int i = tid; i < NOP * (NH / 8); i += blockDim.x)
+            cp_async16(W3 + (i / (NH / 8)) * P2 + 8 * (i % (NH / 8)), src + i);
+        cp_commit();
+        for (int i = tid; i < NH + NH + NO; i += blockDim.x)
+            SB[i] = i < NH ? A.P[OFF_B1 + i] : (i < 2 * NH ? A.P[OFF_B2 + i - NH] : A.P[OFF_B3 + i - 2 * NH]);
     }
-    // ---- the rows: standardised features (bf16) in X
-    unsigned long long pa = 0, pb = 0;
-    long long first = 0;
-    if (A.feat) {
-        const long long st = *A.t_dev;
-        pa = A.ab[2 * (st / A.steps)];
-        pb = A.ab[2 * (st / A.steps) + 1];
-        first = (st % A.steps) * (long long)A.nrows;
-    }
-    auto data_row = [&](int r) -> long long {
-        const long long q = first + row0 + r;
-        return A.feat ? (long long)((pa * (unsigned long long)q + pb) % (unsigned long long)A.n_data) : (long long)(row0 + r);
-    };
-    for (int i = tid; i < TR * NIN; i += blockDim.x) {
-        const int r = i / NIN, c = i % NIN;
-        float v = 0.f;
-        if (r < nvalid) {
-            const long long s = data_row(r);
-            v = A.feat ? (A.feat[s * NIN + c] - A.stats[c]) * A.stats[NIN + c] : A.x_std[s * NIN + c];
-        }
-        X[r * P1 + c] = bf16_bits(v);
-    }
+    cp_wait<2>();
     __syncthreads();
 
     const int rt = warp & 1;          // row tile of this warp in the forward and backward products
-    const int q4 = warp >> 1;         // its group of four n-tiles
-    const float* b1v = A.P + OFF_B1;
-    const float* b2v = A.P + OFF_B2;
-    const float* b3v = A.P + OFF_B3;
+    const int q8 = warp >> 1;         // its pair of n-tiles
+    const float* b1v = SB;
+    const float* b2v = SB + NH;
+    const float* b3v = SB + 2 * NH;
 
     // ---- layer 1: Z1 = X W1^T + b1; A1 = SiLU(Z1) (bf16), G1 = SiLU'(Z1)
     {
@@ -270,8 +313,8 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
         frag_a<P1>(a[0], X, 16 * rt, 0, lane);
         frag_a<P1>(a[1], X, 16 * rt, 16, lane);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int nt = 4 * q4 + j;
+        for (int j = 0; j < 2; ++j) {
+            const int nt = 2 * q8 + j;
             const int c = 8 * nt + 2 * t;
             float acc[4] = {b1v[c], b1v[c + 1], b1v[c], b1v[c + 1]};
             fwd_tile<2, P1, P1>(acc, a, W1, nt, g, t);
@@ -286,6 +329,7 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
             }
         }
     }
+    cp_wait<1>();
     __syncthreads();
     // ---- layer 2
     {
@@ -293,8 +337,8 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) frag_a<P2>(a[kk], A1, 16 * rt, 16 * kk, lane);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int nt = 4 * q4 + j;
+        for (int j = 0; j < 2; ++j) {
+            const int nt = 2 * q8 + j;
             const int c = 8 * nt + 2 * t;
             float acc[4] = {b2v[c], b2v[c + 1], b2v[c], b2v[c + 1]};
             fwd_tile<8, P2, P2>(acc, a, W2, nt, g, t);
@@ -309,15 +353,16 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
             }
         }
     }
+    cp_wait<0>();
     __syncthreads();
-    // ---- layer 3: logits Z3 (n-tiles q4, q4 + 4, q4 + 8, q4 + 12 < 13)
+    // ---- layer 3: logits Z3 (n-tiles q8, q8 + 8 < 13)
     {
         uint32_t a[8][4];
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) frag_a<P2>(a[kk], A2, 16 * rt, 16 * kk, lane);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int nt = q4 + 4 * j;
+        for (int j = 0; j < 2; ++j) {
+            const int nt = q8 + 8 * j;
             if (nt < NOP / 8) {
                 const int c = 8 * nt + 2 * t;
                 const float bb0 = c < NO ? b3v[c] : 0.f, bb1 = c + 1 < NO ? b3v[c + 1] : 0.f;
@@ -348,8 +393,7 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
         for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         const float ls = logf(s);
         const bool live = r < nvalid;
-        const long long srow = live ? data_row(r) : 0;
-        const float* tr = A.target + srow * NO;
+        const float* tr = T + r * NO;
         float l = 0.f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -375,9 +419,8 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
         uint32_t a[7][4];
 #pragma unroll
         for (int kk = 0; kk < 7; ++kk) frag_a<P3>(a[kk], D3, 16 * rt, 16 * kk, lane);
-#pragma unroll
-        for (int jp = 0; jp < 2; ++jp) {
-            const int nt = 4 * q4 + 2 * jp;  // n-tiles nt, nt + 1
+        {
+            const int nt = 2 * q8;  // n-tiles nt, nt + 1
             float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int kk = 0; kk < 7; ++kk) {
@@ -407,9 +450,8 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
         uint32_t a[8][4];
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) frag_a<P2>(a[kk], D2, 16 * rt, 16 * kk, lane);
-#pragma unroll
-        for (int jp = 0; jp < 2; ++jp) {
-            const int nt = 4 * q4 + 2 * jp;
+        {
+            const int nt = 2 * q8;
             float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
@@ -454,64 +496,86 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
         for (int r = 0; r < TR; ++r) l += r < nvalid ? LS[r] : 0.f;
         A.part_loss[blockIdx.x] = l;
     }
-    // ---- weight gradients dW = dZ^T Act over the 32 rows (2 k-tiles):
-    // warp w takes m-tile w of dW2 and dW1 and, for w < 7, of dW3
-    wgrad<P2, P2>(D2, A1, NH / 8, warp, NH, NH, part + OFF_W2, lane);
-    if (warp < 7) wgrad<P3, P2>(D3, A2, NH / 8, warp, NH, NO, part + OFF_W3, lane);
-    wgrad<P2, P1>(D1, X, NIN / 8, warp, NIN, NH, part + OFF_W1, lane);
+    // ---- weight gradients dW = dZ^T Act over the 32 rows (2 k-tiles): warp w takes
+    // half of the n-tiles of m-tile w mod 8 of dW2 and dW1 and, below 7, of dW3
+    const int mt = warp & 7, hf = warp >> 3;
+    wgrad<P2, P2>(D2, A1, hf * (NH / 16), (hf + 1) * (NH / 16), mt, NH, NH, part + OFF_W2, lane);
+    if (mt < 7) wgrad<P3, P2>(D3, A2, hf * (NH / 16), (hf + 1) * (NH / 16), mt, NH, NO, part + OFF_W3, lane);
+    wgrad<P2, P1>(D1, X, hf * (NIN / 16), (hf + 1) * (NIN / 16), mt, NIN, NH, part + OFF_W1, lane);
 }
 
 // g = sum over the CTAs of their partial gradients (in CTA order); with
 // adam: the Adam step of the FP32 parameters and their BF16 copies for the
-// next step, the loss, and (last block) the step counter
-__global__ void train_reduce_kernel(const float* __restrict__ part, const float* __restrict__ part_loss, int ncta,
-                                    float* __restrict__ G, int adam, float* __restrict__ P, float* __restrict__ Mo,
-                                    float* __restrict__ Vo, const float* __restrict__ sched, long long* t_dev, float b1,
-                                    float b2, float eps, uint16_t* __restrict__ Wb, float* loss_acc,
-                                    unsigned* done)
+// next step.  The last block instead sums the loss (partials in CTA order) and,
+// at the end of a graph, moves the step counter on by the graph's steps (every
+// other block of the graph has read it by then).
+constexpr int RED_T = 128;   // threads per block
+__global__ void __launch_bounds__(RED_T) train_reduce_kernel(
+    const float* __restrict__ part, const float* __restrict__ part_loss, int ncta, float* __restrict__ G, int adam,
+    float* __restrict__ P, float* __restrict__ Mo, float* __restrict__ Vo, const float* __restrict__ sched,
+    long long* t_dev, int ahead, int advance, float b1, float b2, float eps, uint16_t* __restrict__ Wb,
+    float* loss_acc)
 {
-    long long st = 0;
-    float lr = 0.f, c1 = 1.f, c2 = 1.f;
+    launch_dependents();
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ float sl[RED_T];
+        float l = 0.f;
+        wait_predecessor();
+        for (int c0 = 0; c0 < ncta; c0 += RED_T) {
+            const int n = min(RED_T, ncta - c0);
+            if (threadIdx.x < n) sl[threadIdx.x] = part_loss[c0 + threadIdx.x];
+            __syncthreads();
+            if (threadIdx.x == 0)
+                for (int c = 0; c < n; ++c) l += sl[c];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            *loss_acc += l;
+            if (advance) *t_dev += advance;
+        }
+        return;
+    }
+    const int i = blockIdx.x * RED_T + threadIdx.x;
+    if (i >= NPARAM) return;
+    float mi = 0.f, vi = 0.f, p = 0.f, lr = 0.f, c1 = 1.f, c2 = 1.f;
     if (adam) {
-        st = *t_dev;
+        // the previous step's results, complete before this kernel could start
+        const long long st = *t_dev + ahead;
         lr = sched[3 * st];
         c1 = sched[3 * st + 1];
         c2 = sched[3 * st + 2];
+        mi = Mo[i];
+        vi = Vo[i];
+        p = P[i];
     }
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NPARAM; i += gridDim.x * blockDim.x) {
-        float gi = 0.f;
-        for (int c = 0; c < ncta; ++c) gi += part[(size_t)c * NPARAM + i];
-        G[i] = gi;
-        if (adam) {
-            const float mi = b1 * Mo[i] + (1.f - b1) * gi;
-            const float vi = b2 * Vo[i] + (1.f - b2) * gi * gi;
-            Mo[i] = mi;
-            Vo[i] = vi;
-            const float p = P[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-            P[i] = p;
-            // the bf16 copy of a weight (biases stay fp32): W1, W2, W3 contiguous
-            int w = -1;
-            if (i < OFF_B1) w = i;
-            else if (i >= OFF_W2 && i < OFF_B2) w = NH * NIN + (i - OFF_W2);
-            else if (i >= OFF_W3 && i < OFF_B3) w = NH * NIN + NH * NH + (i - OFF_W3);
-            if (w >= 0) Wb[w] = bf16_bits(p);
-        }
+    wait_predecessor();
+    float gi = 0.f;
+    // 32 partials in flight at a time, added in order
+    const float* src = part + i;
+    int c = 0;
+    for (; c + 32 <= ncta; c += 32) {
+        float v[32];
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+            asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v[k]) : "l"(src + (size_t)(c + k) * NPARAM));
+#pragma unroll
+        for (int k = 0; k < 32; ++k) gi += v[k];
     }
-    // the last block: loss of the step (partials in CTA order) and the step counter
-    __shared__ bool last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last && threadIdx.x == 0) {
-        __threadfence();
-        float l = 0.f;
-        for (int c = 0; c < ncta; ++c) l += part_loss[c];
-        *loss_acc += l;
-        if (adam) *t_dev = st + 1;
-        *done = 0;
+    for (; c < ncta; ++c) gi += __ldcs(src + (size_t)c * NPARAM);
+    G[i] = gi;
+    if (adam) {
+        mi = fmaf(1.f - b1, gi, b1 * mi);
+        vi = fmaf((1.f - b2) * gi, gi, b2 * vi);
+        Mo[i] = mi;
+        Vo[i] = vi;
+        p = p - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        P[i] = p;
+        // the bf16 copy of a weight (biases stay fp32): W1, W2, W3 contiguous
+        int w = -1;
+        if (i < OFF_B1) w = i;
+        else if (i >= OFF_W2 && i < OFF_B2) w = NH * NIN + (i - OFF_W2);
+        else if (i >= OFF_W3 && i < OFF_B3) w = NH * NIN + NH * NH + (i - OFF_W3);
+        if (w >= 0) Wb[w] = bf16_bits(p);
     }
 }
 
@@ -522,20 +586,17 @@ int train_rows_per_cta() { return TR; }
 
 // One step (or one gradient): nrows rows, either gathered from feat/target
 // with the permutation schedule (feat != nullptr) or taken from x_std/target.
+// ahead: this step's place in the captured graph; advance: the graph's steps on
+// its last one (0 elsewhere).
 cudaError_t launch_train_step(const uint16_t* Wb, const float* P, const float* feat, const float* target,
                               const float* stats, const unsigned long long* ab, long long* t_dev,
                               long long steps, long long n_data, const float* x_std, int nrows, float* part,
                               float* part_loss, float* G, int adam, float* Pw, float* Mo, float* Vo,
                               const float* sched, float b1, float b2, float eps, uint16_t* Wb_out, float* loss_acc,
-                              unsigned* done, cudaStream_t s)
+                              int ahead, int advance, cudaStream_t s)
 {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(train_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)S_TOTAL);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    cudaError_t se = cudaFuncSetAttribute(train_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S_TOTAL);
+    if (se != cudaSuccess) return se;
     TileArgs A;
     A.Wb = Wb;
     A.P = P;
@@ -544,6 +605,7 @@ cudaError_t launch_train_step(const uint16_t* Wb, const float* P, const float* f
     A.stats = stats;
     A.ab = ab;
     A.t_dev = t_dev;
+    A.ahead = ahead;
     A.steps = steps;
     A.n_data = n_data;
     A.x_std = x_std;
@@ -552,12 +614,23 @@ cudaError_t launch_train_step(const uint16_t* Wb, const float* P, const float* f
     A.part = part;
     A.part_loss = part_loss;
     const int ncta = (nrows + TR - 1) / TR;
-    train_tile_kernel<<<ncta, 32 * TWARPS, S_TOTAL, s>>>(A);
-    cudaError_t e = cudaGetLastError();
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ncta);
+    cfg.blockDim = dim3(32 * TWARPS);
+    cfg.dynamicSmemBytes = S_TOTAL;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, train_tile_kernel, A);
     if (e != cudaSuccess) return e;
-    train_reduce_kernel<<<(NPARAM + 255) / 256, 256, 0, s>>>(part, part_loss, ncta, G, adam, Pw, Mo, Vo, sched, t_dev, b1,
-                                                             b2, eps, Wb_out, loss_acc, done);
-    return cudaGetLastError();
+    cfg.gridDim = dim3((NPARAM + RED_T - 1) / RED_T + 1);
+    cfg.blockDim = dim3(RED_T);
+    cfg.dynamicSmemBytes = 0;
+    return cudaLaunchKernelEx(&cfg, train_reduce_kernel, (const float*)part, (const float*)part_loss, ncta, G, adam, Pw,
+                              Mo, Vo, sched, t_dev, ahead, advance, b1, b2, eps, Wb_out, loss_acc);
 }
 
 }  // namespace skirt

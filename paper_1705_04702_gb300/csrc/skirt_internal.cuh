@@ -222,7 +222,7 @@ cudaError_t launch_train_step(const uint16_t* Wb, const float* P, const float* f
                               long long steps, long long n_data, const float* x_std, int nrows, float* part,
                               float* part_loss, float* G, int adam, float* Pw, float* Mo, float* Vo,
                               const float* sched, float b1, float b2, float eps, uint16_t* Wb_out, float* loss_acc,
-                              unsigned* done, cudaStream_t s);
+                              int ahead, int advance, cudaStream_t s);
 
 // error reporting shared by the translation units (api.cu)
 int set_error(int code, const char* fmt, ...);
