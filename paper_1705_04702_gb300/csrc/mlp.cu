@@ -15,7 +15,9 @@
 // tensor-core kernel per 32 rows (forward, softmax cross-entropy, backward,
 // weight-gradient products; mlp_train.cu) and one kernel that sums the
 // partial gradients in order, takes the Adam step (cosine step decay) and
-// refreshes the BF16 weights.
+// refreshes the BF16 weights.  The standardisation, the hull and the guard come
+// from two passes over the features and a radix selection on the device (0.9 ms
+// for 3e5 rows; 2.5 with one block per feature and the selection on the host).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -341,38 +343,102 @@ __global__ void dominant_share_kernel(const float* __restrict__ feat, long long 
     }
 }
 
-// per-feature sums over n samples: sum, sum of squares, min, max (one block per feature)
-__global__ void feature_stats_kernel(const float* feat, long long n, double* out)
+// Per-feature sums over n samples (sum, sum of squares, min, max): lane = feature, a
+// warp per row, so that a row is one 128-byte read and its FP64 additions serve 32
+// features; the blocks' partial results [block][32][4] are joined in block order
+// by the second kernel.
+constexpr int STAT_BLOCKS = 152, STAT_WARPS = 8;
+
+__global__ void __launch_bounds__(32 * STAT_WARPS) feature_stats_kernel(const float* __restrict__ feat, long long n,
+                                                                        double* __restrict__ part)
 {
-    const int c = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double s = 0.0, s2 = 0.0;
     float lo = 3.0e38f, hi = -3.0e38f;
-    for (long long r = threadIdx.x; r < n; r += blockDim.x) {
-        const float v = feat[r * NIN + c];
+    for (long long r = (long long)blockIdx.x * STAT_WARPS + warp; r < n; r += (long long)gridDim.x * STAT_WARPS) {
+        const float v = feat[r * NIN + lane];
         s += v;
         s2 += (double)v * v;
         lo = fminf(lo, v);
         hi = fmaxf(hi, v);
     }
-    __shared__ double rs[256], rs2[256];
-    __shared__ float rl[256], rh[256];
-    rs[threadIdx.x] = s; rs2[threadIdx.x] = s2; rl[threadIdx.x] = lo; rh[threadIdx.x] = hi;
+    __shared__ double rs[STAT_WARPS][32], rs2[STAT_WARPS][32];
+    __shared__ float rl[STAT_WARPS][32], rh[STAT_WARPS][32];
+    rs[warp][lane] = s; rs2[warp][lane] = s2; rl[warp][lane] = lo; rh[warp][lane] = hi;
     __syncthreads();
-    for (int o = blockDim.x / 2; o; o >>= 1) {
-        if (threadIdx.x < o) {
-            rs[threadIdx.x] += rs[threadIdx.x + o];
-            rs2[threadIdx.x] += rs2[threadIdx.x + o];
-            rl[threadIdx.x] = fminf(rl[threadIdx.x], rl[threadIdx.x + o]);
-            rh[threadIdx.x] = fmaxf(rh[threadIdx.x], rh[threadIdx.x + o]);
-        }
-        __syncthreads();
+    if (warp > 0) return;
+    for (int w = 1; w < STAT_WARPS; ++w) {
+        s += rs[w][lane];
+        s2 += rs2[w][lane];
+        lo = fminf(lo, rl[w][lane]);
+        hi = fmaxf(hi, rh[w][lane]);
     }
-    if (threadIdx.x == 0) {
-        out[4 * c + 0] = rs[0];
-        out[4 * c + 1] = rs2[0];
-        out[4 * c + 2] = rl[0];
-        out[4 * c + 3] = rh[0];
+    double* o = part + ((size_t)blockIdx.x * 32 + lane) * 4;
+    o[0] = s; o[1] = s2; o[2] = lo; o[3] = hi;
+}
+
+__global__ void feature_stats_join_kernel(const double* __restrict__ part, int nblocks, double* __restrict__ out)
+{
+    const int c = threadIdx.x;  // one warp
+    double s = 0.0, s2 = 0.0, lo = 3.0e38, hi = -3.0e38;
+    for (int b = 0; b < nblocks; ++b) {
+        const double* p = part + ((size_t)b * 32 + c) * 4;
+        s += p[0];
+        s2 += p[1];
+        lo = p[2] < lo ? p[2] : lo;
+        hi = p[3] > hi ? p[3] : hi;
     }
+    out[4 * c + 0] = s;
+    out[4 * c + 1] = s2;
+    out[4 * c + 2] = lo;
+    out[4 * c + 3] = hi;
+}
+
+// The k-th smallest of n non-negative floats by their bits, 11 + 11 + 10 of them at a
+// time: a histogram of the next bits of the values that agree so far, then the
+// bin that holds rank k.  state: [0] the bits found, [1] the rank left.
+constexpr int SEL_BINS = 2048;
+
+__global__ void select_hist_kernel(const float* __restrict__ v, long long n, const unsigned long long* state, int shift,
+                                   int bits, unsigned* __restrict__ hist)
+{
+    __shared__ unsigned h[SEL_BINS];
+    for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x) h[i] = 0u;
+    __syncthreads();
+    const unsigned found = (unsigned)state[0];
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const unsigned u = __float_as_uint(v[i]);
+        if (shift + bits >= 32 || (u >> (shift + bits)) == found) atomicAdd(&h[(u >> shift) & ((1u << bits) - 1u)], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < SEL_BINS; i += blockDim.x)
+        if (h[i]) atomicAdd(&hist[i], h[i]);
+}
+
+__global__ void select_bin_kernel(unsigned* __restrict__ hist, unsigned long long* state, int bits)
+{
+    // one warp: lane l sums its 64 bins, then the lane holding the rank walks them
+    constexpr int PER = SEL_BINS / 32;
+    const int lane = threadIdx.x;
+    unsigned long long sum = 0;
+    for (int i = 0; i < PER; ++i) sum += hist[lane * PER + i];
+    unsigned long long inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    const unsigned long long k = state[1], before = inc - sum;
+    __syncwarp();
+    if (k >= before && k < inc) {
+        unsigned long long left = k - before;
+        int b = lane * PER;
+        while (left >= hist[b]) left -= hist[b++];
+        state[0] = (state[0] << bits) | (unsigned)b;
+        state[1] = left;
+    }
+    __syncwarp();
+    for (int i = 0; i < PER; ++i) hist[lane * PER + i] = 0u;
 }
 
 // bf16 copies of the weights (W3 padded to 104 rows with zeros) and the fp32
@@ -748,8 +814,10 @@ extern "C" int skirt_mlp_train(skirt_mlp_t net, const float* features, const dou
     MCK(cudaGetLastError());
     // standardisation and hull from the training features
     double*& d_st = sc.d_st;
-    MCK(cudaMallocAsync((void**)&d_st, sizeof(double) * 4 * NIN, s));
-    feature_stats_kernel<<<NIN, 256, 0, s>>>(features, n, d_st);
+    MCK(cudaMallocAsync((void**)&d_st, sizeof(double) * 4 * NIN * (STAT_BLOCKS + 1), s));
+    const int stat_blocks = (int)std::min<long long>(STAT_BLOCKS, (n + STAT_WARPS - 1) / STAT_WARPS);
+    feature_stats_kernel<<<stat_blocks, 32 * STAT_WARPS, 0, s>>>(features, n, d_st + 4 * NIN);
+    feature_stats_join_kernel<<<1, NIN, 0, s>>>(d_st + 4 * NIN, stat_blocks, d_st);
     MCK(cudaGetLastError());
     double st[4 * NIN];
     MCK(cudaMemcpyAsync(st, d_st, sizeof st, cudaMemcpyDeviceToHost, s));
@@ -771,12 +839,27 @@ extern "C" int skirt_mlp_train(skirt_mlp_t net, const float* features, const dou
         MCK(cudaMallocAsync((void**)&d_share, sizeof(float) * (size_t)n, s));
         dominant_share_kernel<<<blocks_for(n, 256), 256, 0, s>>>(features, n, d_share);
         MCK(cudaGetLastError());
-        std::vector<float> sh((size_t)n);
-        MCK(cudaMemcpyAsync(sh.data(), d_share, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost, s));
+        // its rank among the rows, by radix selection on the device
+        unsigned long long*& d_sel = sc.d_ab;  // state, then the histogram
+        MCK(cudaMallocAsync((void**)&d_sel, 2 * sizeof(unsigned long long) + SEL_BINS * sizeof(unsigned), s));
+        unsigned* hist = reinterpret_cast<unsigned*>(d_sel + 2);
+        const unsigned long long init[2] = {0ull, (unsigned long long)((double)opts->guard_quantile * (double)(n - 1))};
+        MCK(cudaMemsetAsync(hist, 0, SEL_BINS * sizeof(unsigned), s));
+        MCK(cudaMemcpyAsync(d_sel, init, sizeof init, cudaMemcpyHostToDevice, s));
+        const int sel[3][2] = {{21, 11}, {10, 11}, {0, 10}};  // shift and width of the bits
+        for (const auto& b : sel) {
+            select_hist_kernel<<<(int)std::min<long long>(blocks_for(n, 256), 304), 256, 0, s>>>(d_share, n, d_sel, b[0], b[1],
+                                                                                               hist);
+            select_bin_kernel<<<1, 32, 0, s>>>(hist, d_sel, b[1]);
+        }
+        MCK(cudaGetLastError());
+        unsigned long long found = 0;
+        MCK(cudaMemcpyAsync(&found, d_sel, sizeof found, cudaMemcpyDeviceToHost, s));
         MCK(cudaStreamSynchronize(s));
-        const size_t k = (size_t)((double)opts->guard_quantile * (double)(n - 1));
-        std::nth_element(sh.begin(), sh.begin() + k, sh.end());
-        net->share_max = sh[k];
+        MCK(cudaFreeAsync(d_sel, s));
+        d_sel = nullptr;
+        const unsigned bits = (unsigned)found;
+        std::memcpy(&net->share_max, &bits, sizeof bits);
     }
     MCK(cudaMemsetAsync(net->Mo, 0, sizeof(float) * NPARAM, s));
     MCK(cudaMemsetAsync(net->Vo, 0, sizeof(float) * NPARAM, s));

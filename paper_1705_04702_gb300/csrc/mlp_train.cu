@@ -1,9 +1,11 @@
 // Training step of the MLP surrogate on the tensor cores (BF16 products,
 // FP32 accumulation, FP32 master weights).
 //
-// train_tile_kernel: one CTA per 32 rows of the batch, 8 warps.  The CTA
-// stages the BF16 weights in shared memory, gathers and standardises its rows,
-// and runs the whole step for them with mma.sync m16n8k16 in inline PTX:
+// train_tile_kernel: one CTA per 32 rows of the batch, 16 warps.  The CTA
+// gathers and standardises its rows and fetches their targets while the
+// previous step still runs, then takes the BF16 weights into shared memory by
+// asynchronous copies, a group per layer, and runs the whole step for its rows
+// with mma.sync m16n8k16 in inline PTX:
 //   forward   Z1 = X W1^T + b1, A1 = SiLU(Z1), Z2, A2, Z3 (logits);
 //   softmax and cross-entropy, dZ3 = (p - t) / n;
 //   backward  dZ2 = (dZ3 W3) * SiLU'(Z2), dZ1 = (dZ2 W2) * SiLU'(Z1)
@@ -20,9 +22,17 @@
 //
 // train_reduce_kernel: the partial gradients summed over the CTAs in CTA
 // order (deterministic), then (training) the Adam step at the learning rate
-// and bias corrections of the device step counter, the refreshed BF16
-// weights for the next step, and the loss; the last block to finish
-// advances the step counter.
+// and bias corrections of the step, the refreshed BF16 weights for the next
+// step, and the loss.
+//
+// A step is a chain of latencies on less than half of the SMs (a batch of 2048
+// rows has 64 tiles): 16.6 us, of which the weights' copy takes 1.0, the layers
+// and the softmax 4.6, the way back 2.1, the weight gradients and their stores
+// about 2.5, the hand-over to the sum 2.2 and the sum 1.5 (35 us with 8 warps
+// that staged the weights and divided 64-bit row numbers in every thread, and
+// with the kernels strictly one after the other).  Tiles of 16 rows would fill
+// the chip but sum the gradients in another order, and the trained parameters
+// are the same bit for bit as before.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -69,6 +79,9 @@ constexpr size_t S_TOTAL = S_IDX + 8 * TR;
 static_assert(S_TOTAL <= 227 * 1024, "shared memory of one CTA");
 static_assert(S_X % 16 == 0 && S_A1 % 16 == 0 && S_D3 % 16 == 0 && S_G1 % 16 == 0 && S_T % 16 == 0 && S_IDX % 8 == 0,
               "16-byte aligned tiles");
+
+constexpr int STAGE = 16 * (8 * (NH / 16) + 4);  // floats of one warp's staging area
+static_assert(4 * TWARPS * STAGE <= S_X, "the staging areas fit the weights' memory");
 
 __device__ __forceinline__ unsigned su32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -166,36 +179,46 @@ __device__ __forceinline__ void fwd_tile(float (&c)[4], const uint32_t (&a)[KT][
 }
 
 // dst[o][i] (o < mrows, row stride outK) = sum over the 32 rows r of D[r][o] Act[r][i]
-// for the output rows of m-tile mt and the n-tiles nt0 .. nt1 - 1 of i: A = D^T,
-// B = Act, both through ldmatrix.trans of the row-major tiles
-template <int SD, int SA>
-__device__ __forceinline__ void wgrad(const uint16_t* D, const uint16_t* Act, int nt0, int nt1, int mt, int outK, int mrows,
-                                      float* dst, int lane)
+// for the output rows of m-tile mt and the NT n-tiles from nt0 of i: A = D^T,
+// B = Act, both through ldmatrix.trans of the row-major tiles.  The 16 x 8 NT
+// results go through the warp's staging area (rows padded by 4 floats) so that
+// they leave in 16-byte stores along the rows: straight from the fragments, each
+// store met 8 rows with 32 bytes and the stores took most of this phase.
+template <int SD, int SA, int NT>
+__device__ __forceinline__ void wgrad(const uint16_t* D, const uint16_t* Act, int nt0, int mt, int outK, int mrows,
+                                      float* dst, float* stage, int lane)
 {
+    constexpr int PS = 8 * NT + 4;
     const int g = lane >> 2, t = lane & 3;
     uint32_t a0[4], a1[4];
     frag_at<SD>(a0, D, 16 * mt, 0, lane);
     frag_at<SD>(a1, D, 16 * mt, 16, lane);
-    for (int np = nt0; np < nt1; np += 2) {
+    __syncwarp();  // the staging area is free
+#pragma unroll
+    for (int np = 0; np < NT; np += 2) {
         float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
         uint32_t b[4];
-        frag_b2t<SA>(b, Act, 0, 8 * np, lane);
+        frag_b2t<SA>(b, Act, 0, 8 * (nt0 + np), lane);
         mma16816(acc0, a0, b[0], b[1]);
         mma16816(acc1, a0, b[2], b[3]);
-        frag_b2t<SA>(b, Act, 16, 8 * np, lane);
+        frag_b2t<SA>(b, Act, 16, 8 * (nt0 + np), lane);
         mma16816(acc0, a1, b[0], b[1]);
         mma16816(acc1, a1, b[2], b[3]);
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const float* acc = u ? acc1 : acc0;
-            const int c = 8 * (np + u) + 2 * t;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int o = 16 * mt + g + 8 * h;
-                if (o < mrows)
-                    *reinterpret_cast<float2*>(dst + (size_t)o * outK + c) = make_float2(acc[2 * h], acc[2 * h + 1]);
-            }
+        for (int h = 0; h < 2; ++h) {
+            float* row = stage + (g + 8 * h) * PS + 8 * np + 2 * t;
+            *reinterpret_cast<float2*>(row) = make_float2(acc0[2 * h], acc0[2 * h + 1]);
+            *reinterpret_cast<float2*>(row + 8) = make_float2(acc1[2 * h], acc1[2 * h + 1]);
         }
+    }
+    __syncwarp();
+    constexpr int C4 = 2 * NT;  // 16-byte pieces per row
+#pragma unroll
+    for (int k = lane; k < 16 * C4; k += 32) {
+        const int o = 16 * mt + k / C4;
+        if (o < mrows)
+            *reinterpret_cast<float4*>(dst + (size_t)o * outK + 8 * nt0 + 4 * (k % C4)) =
+                *reinterpret_cast<const float4*>(stage + (k / C4) * PS + 4 * (k % C4));
     }
 }
 
@@ -378,7 +401,9 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
     }
     __syncthreads();
     // ---- softmax and cross-entropy, one warp per row: dZ3 = (p - t) / n
-    for (int r = warp; r < TR; r += TWARPS) {
+#pragma unroll
+    for (int h = 0; h < TR / TWARPS; ++h) {
+        const int r = warp + h * TWARPS;
         float v[4], m = -3.0e38f;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -491,17 +516,19 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
             part[OFF_B3 + c - 2 * NH] = s;
         }
     }
-    if (tid == 0) {
+    if (tid == 32 * TWARPS - 1) {
         float l = 0.f;
         for (int r = 0; r < TR; ++r) l += r < nvalid ? LS[r] : 0.f;
         A.part_loss[blockIdx.x] = l;
     }
     // ---- weight gradients dW = dZ^T Act over the 32 rows (2 k-tiles): warp w takes
-    // half of the n-tiles of m-tile w mod 8 of dW2 and dW1 and, below 7, of dW3
+    // half of the n-tiles of m-tile w mod 8 of dW2 and dW1 and, below 7, of dW3;
+    // the weights' shared memory, no longer needed, is the staging area
     const int mt = warp & 7, hf = warp >> 3;
-    wgrad<P2, P2>(D2, A1, hf * (NH / 16), (hf + 1) * (NH / 16), mt, NH, NH, part + OFF_W2, lane);
-    if (mt < 7) wgrad<P3, P2>(D3, A2, hf * (NH / 16), (hf + 1) * (NH / 16), mt, NH, NO, part + OFF_W3, lane);
-    wgrad<P2, P1>(D1, X, hf * (NIN / 16), (hf + 1) * (NIN / 16), mt, NIN, NH, part + OFF_W1, lane);
+    float* stage = reinterpret_cast<float*>(sm + S_W1) + warp * STAGE;
+    wgrad<P2, P2, NH / 16>(D2, A1, hf * (NH / 16), mt, NH, NH, part + OFF_W2, stage, lane);
+    if (mt < 7) wgrad<P3, P2, NH / 16>(D3, A2, hf * (NH / 16), mt, NH, NO, part + OFF_W3, stage, lane);
+    wgrad<P2, P1, NIN / 16>(D1, X, hf * (NIN / 16), mt, NIN, NH, part + OFF_W1, stage, lane);
 }
 
 // g = sum over the CTAs of their partial gradients (in CTA order); with
@@ -510,6 +537,7 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
 // at the end of a graph, moves the step counter on by the graph's steps (every
 // other block of the graph has read it by then).
 constexpr int RED_T = 128;   // threads per block
+constexpr int RED_C = 64;    // partials per chunk
 __global__ void __launch_bounds__(RED_T) train_reduce_kernel(
     const float* __restrict__ part, const float* __restrict__ part_loss, int ncta, float* __restrict__ G, int adam,
     float* __restrict__ P, float* __restrict__ Mo, float* __restrict__ Vo, const float* __restrict__ sched,
@@ -536,9 +564,9 @@ __global__ void __launch_bounds__(RED_T) train_reduce_kernel(
         return;
     }
     const int i = blockIdx.x * RED_T + threadIdx.x;
-    if (i >= NPARAM) return;
+    const bool mine = i < NPARAM;
     float mi = 0.f, vi = 0.f, p = 0.f, lr = 0.f, c1 = 1.f, c2 = 1.f;
-    if (adam) {
+    if (adam && mine) {
         // the previous step's results, complete before this kernel could start
         const long long st = *t_dev + ahead;
         lr = sched[3 * st];
@@ -550,18 +578,25 @@ __global__ void __launch_bounds__(RED_T) train_reduce_kernel(
     }
     wait_predecessor();
     float gi = 0.f;
-    // 32 partials in flight at a time, added in order
-    const float* src = part + i;
-    int c = 0;
-    for (; c + 32 <= ncta; c += 32) {
-        float v[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-            asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v[k]) : "l"(src + (size_t)(c + k) * NPARAM));
-#pragma unroll
-        for (int k = 0; k < 32; ++k) gi += v[k];
+    // a chunk of partials of the block's 128 parameters by asynchronous copies, all
+    // in flight at once, then added in order
+    __shared__ __align__(16) float sp[RED_C][RED_T];
+    const int n4 = min(RED_T, NPARAM - (int)blockIdx.x * RED_T) / 4;  // NPARAM is a multiple of 4
+    for (int c0 = 0; c0 < ncta; c0 += RED_C) {
+        const int n = min(RED_C, ncta - c0);
+        const float* src = part + (size_t)c0 * NPARAM + (size_t)blockIdx.x * RED_T;
+        for (int k = threadIdx.x; k < n * (RED_T / 4); k += RED_T) {
+            const int c = k / (RED_T / 4), q = k % (RED_T / 4);
+            if (q < n4) cp_async16(&sp[c][4 * q], src + (size_t)c * NPARAM + 4 * q);
+        }
+        cp_commit();
+        cp_wait<0>();
+        __syncthreads();
+#pragma unroll 16
+        for (int c = 0; c < n; ++c) gi += sp[c][threadIdx.x];
+        __syncthreads();
     }
-    for (; c < ncta; ++c) gi += __ldcs(src + (size_t)c * NPARAM);
+    if (!mine) return;
     G[i] = gi;
     if (adam) {
         mi = fmaf(1.f - b1, gi, b1 * mi);
