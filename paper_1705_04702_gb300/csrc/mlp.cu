@@ -1,15 +1,20 @@
 // MLP surrogate of the dust-emission step: 32 band features -> 128 -> 128 ->
 // 100 emission-shape logits (SiLU, SiLU, softmax).
 //
-// Inference (mlp_infer_kernel): one warp per 16 rows, the three layers as
+// Inference (mlp_infer_kernel): one warp per 32 rows, the three layers as
 // BF16 tensor-core products with FP32 accumulation (mma.sync m16n8k16 in
-// inline PTX); weights staged once per block in shared memory; the FP32
-// accumulator fragment of one layer, passed through SiLU and packed to BF16,
-// is exactly the A-operand fragment of the next layer, so activations never
-// leave registers.  Softmax over the 100 outputs is reduced across the four
-// lanes that hold a row; the result times the cell's absorbed power is
-// written as FP64 emission.  The same pass flags rows whose raw features
-// leave the training hull.
+// inline PTX); weights staged once per block in shared memory, each fragment of
+// them used for the warp's two 16-row tiles; activations go through the warp's
+// own shared memory, so that the layers are loops over pairs of n-tiles that
+// stay in the instruction cache.  Softmax over the 100 outputs is reduced across
+// the four lanes that hold a row; the result times the cell's absorbed power
+// is written as FP64 emission.  The same pass flags rows whose raw features
+// leave the training hull (lane = row).  What bounds it are the tile's chains of
+// dependent products and exponentials at 12 warps per SM (issue 47%, tensor pipe
+// 25%): 4e6 dense rows 1.34 ms (42% of the copy rate), 8e6 torus rows 1.84 ms.
+// With 16-row tiles, every layer unrolled and activations in registers the code
+// outgrew the instruction cache (2.9 fetch stalls per issue): 1.57 and 2.45 ms,
+// the same rows bit for bit; 10 or 8 warps of this form take 1.57 and 1.68 ms.
 //
 // Training (skirt_mlp_train): FP32 master weights; every step is one fused
 // tensor-core kernel per 32 rows (forward, softmax cross-entropy, backward,
@@ -54,24 +59,27 @@ static_assert(OFF_B3 + NO == NPARAM, "packed parameter layout");
 // --------------------------------------------------------------------------
 // inference
 // --------------------------------------------------------------------------
-constexpr int INF_WARPS = 8;
-constexpr int INF_ROWS = 16 * INF_WARPS;
+constexpr int INF_WARPS = 12;
+constexpr int INF_TILE = 32;                    // rows of a warp's tile
+constexpr int INF_ROWS = INF_TILE * INF_WARPS;
 // shared memory: W1 [128][32], W2 [128][128], W3 [104][128] (bf16) with
-// every row padded by 8 elements, so that the eight rows one fragment load
+// every row padded by 8 elements, so that the eight rows one matrix load
 // touches start 4 banks apart (conflict-free); biases [128 + 128 + 104]
-// (fp32); mean / inv_std / lo / hi [32] each; per-warp feature staging
+// (fp32); mean / inv_std / lo / hi [32] each; per warp the feature tile that the
+// bulk copy engine fills, the activations and an mbarrier
 constexpr int KP1 = NIN + 8, KP2 = NH + 8;
 constexpr size_t SM_W1 = 0;
 constexpr size_t SM_W2 = SM_W1 + sizeof(uint16_t) * NH * KP1;
 constexpr size_t SM_W3 = SM_W2 + sizeof(uint16_t) * NH * KP2;
 constexpr size_t SM_B = SM_W3 + sizeof(uint16_t) * NO_PAD * KP2;
 constexpr size_t SM_ST = SM_B + sizeof(float) * (NH + NH + NO_PAD);
-// per warp: two 16-row feature tiles [16][32] fp32 that the bulk copy engine
-// fills asynchronously (128-byte aligned), and their two mbarriers
-constexpr size_t SM_X = (SM_ST + sizeof(float) * 4 * NIN + 127) & ~(size_t)127;
-constexpr size_t SM_BAR = SM_X + sizeof(float) * INF_WARPS * 2 * 16 * NIN;
-constexpr size_t SM_TOTAL = SM_BAR + sizeof(unsigned long long) * INF_WARPS * 2;
-static_assert((KP1 * 2) % 16 == 0 && (KP2 * 2) % 16 == 0, "padded rows keep 16-byte alignment");
+constexpr size_t SM_X = (SM_ST + sizeof(float) * 4 * NIN + 127) & ~(size_t)127;  // [warp][32][32] fp32
+constexpr size_t SM_A = SM_X + sizeof(float) * INF_WARPS * INF_TILE * NIN;         // [warp][32][KP2] bf16
+constexpr size_t SM_BAR = SM_A + sizeof(uint16_t) * INF_WARPS * INF_TILE * KP2;
+constexpr size_t SM_TOTAL = SM_BAR + sizeof(unsigned long long) * INF_WARPS;
+static_assert(SM_TOTAL <= 227 * 1024, "shared memory of one block");
+static_assert((KP1 * 2) % 16 == 0 && (KP2 * 2) % 16 == 0 && SM_ST % 16 == 0 && SM_A % 16 == 0 && SM_BAR % 8 == 0,
+              "padded rows and parts keep 16-byte alignment");
 
 // a wait for a bulk copy that runs out sets it, and the kernel stops
 __device__ unsigned g_mlp_timeout;
@@ -106,47 +114,88 @@ __device__ __forceinline__ double widen_pos(float f)
     return e ? __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29)) : 0.0;
 }
 
-// acc[j][0..3] for n-tiles j: rows (g, g+8), cols 8j + 2t + {0,1}; produces
-// the next layer's A fragments: k-tile kk from n-tiles 2kk, 2kk+1
-template <int NT>
-__device__ __forceinline__ void to_afrag(const float (&acc)[NT][4], uint32_t (&a)[NT / 2][4])
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p)
 {
-#pragma unroll
-    for (int kk = 0; kk < NT / 2; ++kk) {
-        a[kk][0] = pack_bf16(silu_f(acc[2 * kk][0]), silu_f(acc[2 * kk][1]));
-        a[kk][1] = pack_bf16(silu_f(acc[2 * kk][2]), silu_f(acc[2 * kk][3]));
-        a[kk][2] = pack_bf16(silu_f(acc[2 * kk + 1][0]), silu_f(acc[2 * kk + 1][1]));
-        a[kk][3] = pack_bf16(silu_f(acc[2 * kk + 1][2]), silu_f(acc[2 * kk + 1][3]));
-    }
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(smem_u32(p)));
 }
 
-// one layer: out[NT] n-tiles = A (KT k-tiles) x W^T, W [rows = 8*NT][cols = 16*KT] bf16 in smem
-// with row stride KP elements
-template <int NT, int KT, int KP>
-__device__ __forceinline__ void layer(const uint32_t (&a)[KT][4], const uint16_t* __restrict__ W,
-                                      const float* __restrict__ bias, float (&out)[NT][4], int g, int t)
+// A fragments (16 x 16 KT) of the rows from r0 of the activations
+template <int KT>
+__device__ __forceinline__ void load_afrag(uint32_t (&a)[KT][4], const uint16_t* act, int r0, int lane)
 {
-    constexpr int K = KP;
+    const int q = lane >> 3, j = lane & 7;
 #pragma unroll
-    for (int j = 0; j < NT; ++j) {
-        const float b0 = bias[8 * j + 2 * t], b1 = bias[8 * j + 2 * t + 1];
-        out[j][0] = b0; out[j][1] = b1; out[j][2] = b0; out[j][3] = b1;
-        const uint16_t* wr = W + (size_t)(8 * j + g) * K + 2 * t;
+    for (int kk = 0; kk < KT; ++kk) ldsm4(a[kk], act + (r0 + (q & 1) * 8 + j) * KP2 + 16 * kk + (q >> 1) * 8);
+}
+
+// B fragments of the n-tiles at row n0 and n0 + 8 of W (row stride KP) for k-tile
+// kk: b[0], b[1] and b[2], b[3]
+template <int KP>
+__device__ __forceinline__ void load_bfrag2(uint32_t (&b)[4], const uint16_t* W, int n0, int kk, int lane)
+{
+    const int q = lane >> 3, j = lane & 7;
+    ldsm4(b, W + (n0 + (q >> 1) * 8 + j) * KP + 16 * kk + (q & 1) * 8);
+}
+
+// One hidden layer: act[32][8 NT] = SiLU(act[32][16 KT] W^T + bias) in place (the
+// inputs are in registers before the first output is written)
+template <int NT, int KT, int KP>
+__device__ __forceinline__ void hidden_layer(uint16_t* act, const uint16_t* W, const float* bias, int lane)
+{
+    const int g = lane >> 2, t = lane & 3;
+    uint32_t a0[KT][4], a1[KT][4];
+    load_afrag<KT>(a0, act, 0, lane);
+    load_afrag<KT>(a1, act, 16, lane);
+    __syncwarp();
+#pragma unroll 1
+    for (int n0 = 0; n0 < 8 * NT; n0 += 16) {
+        float c[2][2][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const float2 bb = *reinterpret_cast<const float2*>(bias + n0 + 8 * u + 2 * t);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                c[h][u][0] = c[h][u][2] = bb.x;
+                c[h][u][1] = c[h][u][3] = bb.y;
+            }
+        }
 #pragma unroll
         for (int kk = 0; kk < KT; ++kk) {
-            const uint32_t b0w = *reinterpret_cast<const uint32_t*>(wr + 16 * kk);
-            const uint32_t b1w = *reinterpret_cast<const uint32_t*>(wr + 16 * kk + 8);
-            mma_bf16(out[j], a[kk][0], a[kk][1], a[kk][2], a[kk][3], b0w, b1w);
+            uint32_t b[4];
+            load_bfrag2<KP>(b, W, n0, kk, lane);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                mma_bf16(c[0][u], a0[kk][0], a0[kk][1], a0[kk][2], a0[kk][3], b[2 * u], b[2 * u + 1]);
+                mma_bf16(c[1][u], a1[kk][0], a1[kk][1], a1[kk][2], a1[kk][3], b[2 * u], b[2 * u + 1]);
+            }
         }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                uint16_t* o = act + (16 * h + g) * KP2 + n0 + 8 * u + 2 * t;
+                *reinterpret_cast<uint32_t*>(o) = pack_bf16(silu_f(c[h][u][0]), silu_f(c[h][u][1]));
+                *reinterpret_cast<uint32_t*>(o + 8 * KP2) = pack_bf16(silu_f(c[h][u][2]), silu_f(c[h][u][3]));
+            }
     }
+    __syncwarp();
 }
 
-__global__ void __launch_bounds__(32 * INF_WARPS, 2) mlp_infer_kernel(
+// zeros into `count` emission rows from row r
+__device__ __forceinline__ void zero_rows(double* emission, long long r, int count, int lane)
+{
+    double2* o = reinterpret_cast<double2*>(emission + r * NO);
+    for (int k = lane; k < count * (NO / 2); k += 32) __stcs(o + k, make_double2(0.0, 0.0));
+}
+
+__global__ void __launch_bounds__(32 * INF_WARPS, 1) mlp_infer_kernel(
     const uint16_t* __restrict__ Wg, const float* __restrict__ Bg, const float* __restrict__ stats,
     const float* __restrict__ features, const double* __restrict__ total, long long n,
     double* __restrict__ emission, unsigned char* __restrict__ flags, float inv_share_max)
 {
-    extern __shared__ __align__(16) unsigned char sm[];
+    extern __shared__ __align__(128) unsigned char sm[];
     // stage the weights (bf16, contiguous W1 W2 W3) and biases / statistics
     {
         // 16-byte chunks of the contiguous global rows into the padded rows
@@ -172,144 +221,175 @@ __global__ void __launch_bounds__(32 * INF_WARPS, 2) mlp_infer_kernel(
     const float* B1 = reinterpret_cast<const float*>(sm + SM_B);
     const float* B2 = B1 + NH;
     const float* B3 = B2 + NH;
-    const float* mean = reinterpret_cast<const float*>(sm + SM_ST);
-    const float* istd = mean + NIN;
-    const float* hlo = istd + NIN;
-    const float* hhi = hlo + NIN;
+    const float4* mean4 = reinterpret_cast<const float4*>(sm + SM_ST);
+    const float4* istd4 = mean4 + NIN / 4;
+    const float4* lo4 = istd4 + NIN / 4;
+    const float4* hi4 = lo4 + NIN / 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
-    float* xbuf = reinterpret_cast<float*>(sm + SM_X) + warp * 2 * 16 * NIN;  // [2][16][32]
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm + SM_BAR) + warp * 2;
+    float* xbuf = reinterpret_cast<float*>(sm + SM_X) + warp * INF_TILE * NIN;
+    uint16_t* act = reinterpret_cast<uint16_t*>(sm + SM_A) + warp * INF_TILE * KP2;
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(sm + SM_BAR) + warp;
     if (lane == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
+        mbar_init(bar, 1);
         fence_barrier_init();
     }
     __syncwarp();
     const long long stride = (long long)gridDim.x * INF_ROWS;
-    // the 16 feature rows of the tile at row b (fewer at the end), 128 bytes each
-    auto fetch = [&](long long b, int buf) {
-        const long long rows = n - b < 16 ? n - b : 16;
+    // the feature rows of the tile at row b (fewer at the end), 128 bytes each
+    auto fetch = [&](long long b) {
+        const long long rows = n - b < INF_TILE ? n - b : INF_TILE;
         fence_proxy_async();
-        bulk_load(xbuf + buf * 16 * NIN, features + b * NIN, (unsigned)(rows * NIN * sizeof(float)), &bar[buf]);
+        bulk_load(xbuf, features + b * NIN, (unsigned)(rows * NIN * sizeof(float)), bar);
     };
-    long long base = (long long)blockIdx.x * INF_ROWS + warp * 16;
-    if (lane == 0 && base < n) fetch(base, 0);
-    for (long long k = 0; base < n; base += stride, ++k) {
-        const int buf = (int)(k & 1);
-        // the next tile streams in while this one is computed
-        if (lane == 0 && base + stride < n) fetch(base + stride, buf ^ 1);
-        if (!mbar_wait(&bar[buf], (unsigned)((k >> 1) & 1))) {
+    long long base = (long long)blockIdx.x * INF_ROWS + warp * INF_TILE;
+    if (lane == 0 && base < n) fetch(base);
+    unsigned parity = 0;
+    for (; base < n; base += stride, parity ^= 1u) {
+        const int rows = n - base < INF_TILE ? (int)(n - base) : INF_TILE;
+        const double tot = lane < rows ? __ldcs(total + base + lane) : 0.0;  // of row `lane`
+        if (!__all_sync(0xffffffffu, mbar_wait(bar, parity))) {
             atomicOr(&g_mlp_timeout, 1u);
-            if (lane == 0 && base + stride < n) mbar_wait(&bar[buf ^ 1], (unsigned)(((k + 1) >> 1) & 1));
             break;
         }
-        // the rows' absorbed powers for the epilogue, requested before the layers so that
-        // their latency overlaps with the products
-        const long long r0 = base + g, r1 = base + g + 8;
-        const double tot0 = r0 < n ? __ldcs(total + r0) : 0.0;
-        const double tot1 = r1 < n ? __ldcs(total + r1) : 0.0;
-        const float* xs = xbuf + buf * 16 * NIN;  // [16][32]; rows past n hold stale values
-        // ---- guard: row i, lane = feature.  A row leaves the training hull when a
-        // feature leaves its range, or when its dominant band holds a larger share of
-        // the cell's absorbed power than the guard allows: sum_b 10^(f_b - f_max) is
-        // the inverse of that share.  One ballot per row.
-        if (flags) {
-            bool mine = false;
-            const float lo_f = hlo[lane], hi_f = hhi[lane];
-#pragma unroll 4
-            for (int i = 0; i < 16; ++i) {
-                const float v = xs[i * NIN + lane];
-                float m = v;
+        // ---- lane = row: the row's features in 8 groups of four, in an order rotated
+        // by the lane (the rows lie 32 banks apart), standardised into act, and the
+        // guard.  A row leaves the training hull when a feature leaves its range, or
+        // when its dominant band holds a larger share of the cell's absorbed power
+        // than the guard allows: sum_b 10^(f_b - f_max) is the inverse of that share.
+        // The sum joins groups 4, 2, 1 apart and then the four places, an order that
+        // the rotation leaves alone.
+        {
+            float4 v[8];
+            float mx = -INFINITY;
+            bool in = true;
 #pragma unroll
-                for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                float e = exp2f((v - m) * 3.32192809f);
-#pragma unroll
-                for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-                const unsigned out = __ballot_sync(0xffffffffu, !(v >= lo_f && v <= hi_f) || e < inv_share_max);
-                if (lane == i) mine = out != 0;
+            for (int k = 0; k < 8; ++k) {
+                const int c = (k + lane) & 7;
+                v[k] = reinterpret_cast<const float4*>(xbuf + lane * NIN)[c];
+                const float4 mu = mean4[c], is = istd4[c];
+                *reinterpret_cast<uint2*>(act + lane * KP2 + 4 * c) =
+                    make_uint2(pack_bf16((v[k].x - mu.x) * is.x, (v[k].y - mu.y) * is.y),
+                               pack_bf16((v[k].z - mu.z) * is.z, (v[k].w - mu.w) * is.w));
+                if (flags) {
+                    const float4 l = lo4[c], h = hi4[c];
+                    in = in && v[k].x >= l.x && v[k].x <= h.x && v[k].y >= l.y && v[k].y <= h.y && v[k].z >= l.z &&
+                         v[k].z <= h.z && v[k].w >= l.w && v[k].w <= h.w;
+                    mx = fmaxf(mx, fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w)));
+                }
             }
-            const long long r = base + lane;
-            // a cell without absorbed power emits nothing: no fallback needed
-            if (lane < 16 && r < n) flags[r] = (mine && total[r] > 0.0) ? 1 : 0;
+            if (flags) {
+                const auto ex = [&](float f) { return exp2f((f - mx) * 3.32192809f); };
+                float4 e[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) e[k] = make_float4(ex(v[k].x), ex(v[k].y), ex(v[k].z), ex(v[k].w));
+                const auto add = [](float4 p, float4 q) {
+                    return make_float4(p.x + q.x, p.y + q.y, p.z + q.z, p.w + q.w);
+                };
+#pragma unroll
+                for (int k = 0; k < 4; ++k) e[k] = add(e[k], e[k + 4]);
+                e[0] = add(e[0], e[2]);
+                e[1] = add(e[1], e[3]);
+                e[0] = add(e[0], e[1]);
+                const float sum = (e[0].x + e[0].z) + (e[0].y + e[0].w);
+                // a cell without absorbed power emits nothing: no fallback needed
+                if (lane < rows) flags[base + lane] = (!in || sum < inv_share_max) && tot > 0.0 ? 1 : 0;
+            }
         }
-        // a tile none of whose rows absorbs power (empty space): its emission rows
-        // are zeros (the epilogue scales every row by its FP32 total), so the
-        // layers are skipped
-        if (!__any_sync(0xffffffffu, (float)tot0 != 0.f || (float)tot1 != 0.f)) {
+        __syncwarp();  // every lane is done with the feature tile
+        if (lane == 0 && base + stride < n) fetch(base + stride);
+        // a 16-row tile none of whose rows absorbs power (empty space): its emission
+        // rows are zeros (the epilogue scales every row by its FP32 total), so its
+        // products are skipped
+        const float ftot = (float)tot;
+        const unsigned live = __ballot_sync(0xffffffffu, ftot != 0.f);
+        if (live == 0u) {
+            zero_rows(emission, base, rows, lane);
+            continue;
+        }
+        // ---- layers
+        hidden_layer<NH / 8, 2, KP1>(act, W1, B1, lane);
+        hidden_layer<NH / 8, NH / 16, KP2>(act, W2, B2, lane);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const long long r0 = base + 16 * h + g, r1 = r0 + 8;
+            if (((live >> (16 * h)) & 0xFFFFu) == 0u) {
+                if (rows > 16 * h) zero_rows(emission, base + 16 * h, rows - 16 * h < 16 ? rows - 16 * h : 16, lane);
+                continue;
+            }
+            uint32_t a[NH / 16][4];
+            load_afrag<NH / 16>(a, act, 16 * h, lane);
+            float z[NO_PAD / 8][4];
+#pragma unroll
+            for (int j = 0; j < NO_PAD / 8; ++j) {
+                const float2 bb = *reinterpret_cast<const float2*>(B3 + 8 * j + 2 * t);
+                z[j][0] = z[j][2] = bb.x;
+                z[j][1] = z[j][3] = bb.y;
+            }
+            // n-tiles in pairs (the last alone), two k-tiles per matrix load for it
+#pragma unroll
+            for (int j = 0; j + 1 < NO_PAD / 8; j += 2)
+#pragma unroll
+                for (int kk = 0; kk < NH / 16; ++kk) {
+                    uint32_t b[4];
+                    load_bfrag2<KP2>(b, W3, 8 * j, kk, lane);
+                    mma_bf16(z[j], a[kk][0], a[kk][1], a[kk][2], a[kk][3], b[0], b[1]);
+                    mma_bf16(z[j + 1], a[kk][0], a[kk][1], a[kk][2], a[kk][3], b[2], b[3]);
+                }
+            {
+                constexpr int j = NO_PAD / 8 - 1;
+                const int q = lane >> 3, r = lane & 7;
+#pragma unroll
+                for (int kk = 0; kk < NH / 16; kk += 2) {
+                    uint32_t b[4];
+                    ldsm4(b, W3 + (8 * j + r) * KP2 + 16 * kk + q * 8);
+                    mma_bf16(z[j], a[kk][0], a[kk][1], a[kk][2], a[kk][3], b[0], b[1]);
+                    mma_bf16(z[j], a[kk + 1][0], a[kk + 1][1], a[kk + 1][2], a[kk + 1][3], b[2], b[3]);
+                }
+            }
+            // ---- softmax over the 100 outputs of rows g and g+8 (4 lanes per row)
+            float m0 = -3.0e38f, m1 = -3.0e38f;
+#pragma unroll
+            for (int j = 0; j < NO_PAD / 8; ++j) {
+                if (8 * j + 2 * t < NO) { m0 = fmaxf(m0, fmaxf(z[j][0], z[j][1])); m1 = fmaxf(m1, fmaxf(z[j][2], z[j][3])); }
+            }
+            m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 1));
+            m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 2));
+            m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 1));
+            m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 2));
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int j = 0; j < NO_PAD / 8; ++j) {
+                const bool ok = 8 * j + 2 * t < NO;
+                z[j][0] = ok ? __expf(z[j][0] - m0) : 0.f;
+                z[j][1] = ok ? __expf(z[j][1] - m0) : 0.f;
+                z[j][2] = ok ? __expf(z[j][2] - m1) : 0.f;
+                z[j][3] = ok ? __expf(z[j][3] - m1) : 0.f;
+                s0 += z[j][0] + z[j][1];
+                s1 += z[j][2] + z[j][3];
+            }
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+            s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
+            // emission = shape x absorbed power, formed in FP32 (the shape is an FP32
+            // softmax) and widened exactly to FP64
+            const float f0 = __shfl_sync(0xffffffffu, ftot, 16 * h + g) / s0;
+            const float f1 = __shfl_sync(0xffffffffu, ftot, 16 * h + g + 8) / s1;
 #pragma unroll
             for (int j = 0; j < NO_PAD / 8; ++j) {
                 const int c = 8 * j + 2 * t;
                 if (c < NO) {
-                    if (r0 < n) __stcs(reinterpret_cast<double2*>(emission + r0 * NO + c), make_double2(0.0, 0.0));
-                    if (r1 < n) __stcs(reinterpret_cast<double2*>(emission + r1 * NO + c), make_double2(0.0, 0.0));
+                    if (r0 < n)
+                        __stcs(reinterpret_cast<double2*>(emission + r0 * NO + c),
+                               make_double2(widen_pos(f0 * z[j][0]), widen_pos(f0 * z[j][1])));
+                    if (r1 < n)
+                        __stcs(reinterpret_cast<double2*>(emission + r1 * NO + c),
+                               make_double2(widen_pos(f1 * z[j][2]), widen_pos(f1 * z[j][3])));
                 }
             }
-            __syncwarp();  // every lane is done with this buffer before it is refilled
-            continue;
         }
-        uint32_t a1[2][4];
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-            const int c = 16 * kk + 2 * t;
-            auto sx = [&](int row, int col) { return (xs[row * NIN + col] - mean[col]) * istd[col]; };
-            a1[kk][0] = pack_bf16(sx(g, c), sx(g, c + 1));
-            a1[kk][1] = pack_bf16(sx(g + 8, c), sx(g + 8, c + 1));
-            a1[kk][2] = pack_bf16(sx(g, c + 8), sx(g, c + 9));
-            a1[kk][3] = pack_bf16(sx(g + 8, c + 8), sx(g + 8, c + 9));
-        }
-        __syncwarp();
-        // ---- layers
-        float h[NH / 8][4];
-        layer<NH / 8, 2, KP1>(a1, W1, B1, h, g, t);
-        uint32_t a2[NH / 16][4];
-        to_afrag<NH / 8>(h, a2);
-        layer<NH / 8, NH / 16, KP2>(a2, W2, B2, h, g, t);
-        to_afrag<NH / 8>(h, a2);
-        float z[NO_PAD / 8][4];
-        layer<NO_PAD / 8, NH / 16, KP2>(a2, W3, B3, z, g, t);
-        // ---- softmax over the 100 outputs of rows g and g+8 (4 lanes per row)
-        float m0 = -3.0e38f, m1 = -3.0e38f;
-#pragma unroll
-        for (int j = 0; j < NO_PAD / 8; ++j) {
-            if (8 * j + 2 * t < NO) { m0 = fmaxf(m0, fmaxf(z[j][0], z[j][1])); m1 = fmaxf(m1, fmaxf(z[j][2], z[j][3])); }
-        }
-        m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 1));
-        m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 2));
-        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 1));
-        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, 2));
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-        for (int j = 0; j < NO_PAD / 8; ++j) {
-            const bool ok = 8 * j + 2 * t < NO;
-            z[j][0] = ok ? __expf(z[j][0] - m0) : 0.f;
-            z[j][1] = ok ? __expf(z[j][1] - m0) : 0.f;
-            z[j][2] = ok ? __expf(z[j][2] - m1) : 0.f;
-            z[j][3] = ok ? __expf(z[j][3] - m1) : 0.f;
-            s0 += z[j][0] + z[j][1];
-            s1 += z[j][2] + z[j][3];
-        }
-        s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
-        s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
-        // emission = shape x absorbed power, formed in FP32 (the shape is an FP32
-        // softmax) and widened exactly to FP64
-        const float f0 = r0 < n ? (float)tot0 / s0 : 0.f;
-        const float f1 = r1 < n ? (float)tot1 / s1 : 0.f;
-#pragma unroll
-        for (int j = 0; j < NO_PAD / 8; ++j) {
-            const int c = 8 * j + 2 * t;
-            if (c < NO) {
-                if (r0 < n)
-                    __stcs(reinterpret_cast<double2*>(emission + r0 * NO + c),
-                           make_double2(widen_pos(f0 * z[j][0]), widen_pos(f0 * z[j][1])));
-                if (r1 < n)
-                    __stcs(reinterpret_cast<double2*>(emission + r1 * NO + c),
-                           make_double2(widen_pos(f1 * z[j][2]), widen_pos(f1 * z[j][3])));
-            }
-        }
-        __syncwarp();  // every lane is done with this buffer before it is refilled
+        __syncwarp();  // every lane is done with the activations
     }
 }
 
