@@ -59,7 +59,7 @@ enum { ERRBIT_EVENT_CAP = 1, ERRBIT_SOURCE = 2, ERRBIT_NONFINITE = 4, ERRBIT_PAT
 // ~ref = level << 27 | leaf index (levels up to 15).  kr: the leaf's extinction coefficient.
 // nb[2a + (positive side)]: for a leaf, the node across that face along
 // axis a of the same level, or the leaf of a larger size that covers it
-// (-1 outside the root box).
+// (-1 outside the root box).  The mixed kernel loads a node at once: the array starts on a 32-byte boundary.
 struct __align__(16) OctNode {
     int ref;
     float kr;

@@ -15,7 +15,7 @@ enum {
     ST_DEPOSIT_DONE,
     ST_LOCATE_DONE,
     ST_PEEL_DONE,
-    ST_PEEL,  // mixed form: start the peel-off towards the current instrument
+    ST_PEEL,  // start the peel-off towards the current instrument
     ST_AFTER_SCATTER,
     ST_END_PACKET,
 };

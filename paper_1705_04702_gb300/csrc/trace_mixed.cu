@@ -45,7 +45,8 @@
 // start of the deposit traversal it repeats.  Against selecting every operand
 // by axis and setting traversals up inside each stage: 1e7 packets on the
 // 256^3 disk 172 ms (259), 8e6 packets of 200 wavelengths on the 128^3 torus
-// 117 ms (200), 3e6 packets on an octree of 8.3e5 leaves 58 ms (94), the same
+// 117 ms (200), 3e6 packets on an octree of 8.3e5 leaves 58 ms (94; 40 with
+// step_oct's later changes), the same
 // histories bit for bit.  A crossing is now ~99 warp instructions for the
 // lanes of a warp (27 of them the deposit's); events take a fifth of the
 // instructions, run by 4 to 5 lanes at a time.
@@ -138,13 +139,15 @@ __device__ __forceinline__ float df_diff(float2 f, float xh, float xl)
     return __fadd_rn(__fsub_rn(f.x, xh), __fsub_rn(f.y, xl));
 }
 
-// Integer <-> FP32 for 0 <= i < 2^23 by the 2^23 offset: one logical and one
-// FP32 instruction, where a conversion instruction would occupy a slow pipe
-// (measured on the octree kernel, whose crossings held three float-to-int
-// conversions: FP64/conversion pipe 64% active).
-__device__ __forceinline__ float i2f_small(int i) { return __int_as_float(0x4B000000 | i) - 8388608.f; }
-// floor(f) for 0 <= f < 2^23
-__device__ __forceinline__ int floor_small(float f) { return __float_as_int(__fadd_rd(f, 8388608.f)) & 0x7FFFFF; }
+// Integers 0 <= i < 2^23 and FP32 by the 2^23 offset: i + 2^23 has i in its
+// low 23 bits.  Logical and FP32 instructions, where a conversion instruction
+// would occupy a slow pipe (measured on the octree kernel, whose crossings
+// held three float-to-int conversions: FP64/conversion pipe 64% active).
+constexpr float TWO23 = 8388608.f;
+constexpr int TWO23_BITS = 0x4B000000;
+// floor(f) + 2^23 for 0 <= f < 2^23, as bits
+__device__ __forceinline__ int floor_bits(float f) { return __float_as_int(__fadd_rd(f, TWO23)); }
+__device__ __forceinline__ int floor_small(float f) { return floor_bits(f) & 0x7FFFFF; }
 
 // Distance along the ray to face plane k (FP32 index) of one axis.
 __device__ __forceinline__ float face_t(float k, float d, float lo, float x, float iv)
@@ -178,6 +181,25 @@ constexpr int PEEL_SCATTER = 16;  // at most 16 instruments
 
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
+// An octree node's 32 bytes, fetched by one load: the children or the leaf, its
+// density, and the nodes across its six faces.
+struct OctRec {
+    int ref;
+    float kr;
+    int nb[6];
+};
+__device__ __forceinline__ OctRec oct_load(const OctNode* p)
+{
+    OctRec r;
+    int k;
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r.ref), "=r"(k), "=r"(r.nb[0]), "=r"(r.nb[1]), "=r"(r.nb[2]), "=r"(r.nb[3]), "=r"(r.nb[4]),
+          "=r"(r.nb[5])
+        : "l"(p));
+    r.kr = __int_as_float(k);
+    return r;
+}
+
 // Grid kinds.  G_CART: Cartesian, face indices held as FP32 integers (every
 // dimension below 2^23, so that they stay exact); G_CART_BIG: Cartesian with a
 // longer axis, face indices as integers; G_OCT: octree (Sect. 7.9), where the
@@ -210,11 +232,12 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     int mode = M_NONE;
     // Cartesian: per axis the index of the next face (kf), its step (sf: +1, -1
     // or 0) and the cell-index stride of a crossing (st); octree: the leaf's
-    // lattice corner (c) and the step
+    // lattice corner (c, an integer in FP32) and minus the step (s)
     using KF = typename std::conditional<BIG, int, float>::type;
     KF kf0 = 0, kf1 = 0, kf2 = 0, sf0 = 0, sf1 = 0, sf2 = 0;
     int st0 = 0, st1 = 0, st2 = 0;
-    int c0 = 0, c1 = 0, c2 = 0, s0 = 0, s1 = 0, s2 = 0;
+    float c0 = 0.f, c1 = 0.f, c2 = 0.f;
+    int s0 = 0, s1 = 0, s2 = 0;
     float iv0 = 0.f, iv1 = 0.f, iv2 = 0.f, tn0 = 0.f, tn1 = 0.f, tn2 = 0.f, tcur = 0.f;
     float t_end = 0.f;               // Cartesian: no crossing before this distance leaves the grid
     float tau_h = 0.f, tau_l = 0.f;  // running optical depth of the traversal (double-float)
@@ -232,6 +255,11 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     const OctNode* __restrict__ nodes = A.oct_nodes;
     bool started = false;  // per-wavelength schedule: this thread's packet is taken
     int onode = 0, olev = 0, pc_node = 0;
+    // octree: the distance at which the ray leaves the current leaf, the axis of
+    // that face, the node across it, and the way from the leaf's corner to the
+    // entry point's lattice cell along that axis
+    float oex = 0.f, odel = 0.f;
+    int oax = 0, onb = 0;
     float v0 = 0.f, v1 = 0.f, v2 = 0.f;
     // ---- packet state (registers)
     int stage = ST_NEW;
@@ -250,24 +278,36 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         return c;
     };
 
-    // octree: enter the leaf holding lattice cell (j0, j1, j2), descending
-    // from `node` (a leaf, or a node of level `lev`)
-    auto oct_enter = [&](int node, int lev, int j0, int j1, int j2) {
-        int2 h = __ldg(reinterpret_cast<const int2*>(nodes + node));
-        while (h.x >= 0 && lev < OL) {
+    // octree: enter the leaf holding the lattice cell (j0, j1, j2) (given as
+    // 2^23 + j in FP32 bits), descending from `node` (a leaf, or a node of level
+    // `lev`), whose record is q; q becomes the leaf's
+    auto oct_enter = [&](OctRec& q, int node, int lev, int j0, int j1, int j2) {
+        while (q.ref >= 0 && lev < OL) {
             ++lev;
             const int b = OL - lev;
-            node = h.x + (((j0 >> b) & 1) | (((j1 >> b) & 1) << 1) | (((j2 >> b) & 1) << 2));
-            h = __ldg(reinterpret_cast<const int2*>(nodes + node));
+            node = q.ref + (((j0 >> b) & 1) | (((j1 >> b) & 1) << 1) | (((j2 >> b) & 1) << 2));
+            q = oct_load(nodes + node);
         }
         onode = node;
-        olev = oct_leaf_level(h.x);
-        cur_m = oct_leaf_index(h.x);
-        kr_cur = __int_as_float(h.y);
-        const int mask = ~((1 << (OL - olev)) - 1);
-        c0 = j0 & mask;
-        c1 = j1 & mask;
-        c2 = j2 & mask;
+        olev = oct_leaf_level(q.ref);
+        cur_m = oct_leaf_index(q.ref);
+        kr_cur = q.kr;
+        const int mask = (int)(~0u << (OL - olev));
+        c0 = __int_as_float(j0 & mask) - TWO23;
+        c1 = __int_as_float(j1 & mask) - TWO23;
+        c2 = __int_as_float(j2 & mask) - TWO23;
+    };
+
+    // octree: where the ray leaves the current leaf, from its face distances and
+    // its record (inside its parent, the node across a face is the sibling)
+    auto oct_exit = [&](const OctRec& q) {
+        oex = fminf(fminf(tn0, tn1), tn2);
+        oax = (tn0 == oex) ? 0 : ((tn1 == oex) ? 1 : 2);
+        const int ss = oax == 0 ? s0 : (oax == 1 ? s1 : s2);
+        const int lo = oax == 0 ? q.nb[0] : (oax == 1 ? q.nb[2] : q.nb[4]);
+        const int hi = oax == 0 ? q.nb[1] : (oax == 1 ? q.nb[3] : q.nb[5]);
+        onb = ss < 0 ? hi : lo;
+        odel = ss < 0 ? __int_as_float((127 + OL - olev) << 23) : -1.f;
     };
 
     // starts a traversal of kind m along (vx, vy, vz), whose reciprocals (zero
@@ -285,9 +325,11 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
             pc_node = 0;
             have_pc = true;
         }
+        OctRec q;
         if constexpr (OCT) {
-            oct_enter(pc_node, 0, pc0, pc1, pc2);
-            pc0 = c0; pc1 = c1; pc2 = c2;
+            q = oct_load(nodes + pc_node);
+            oct_enter(q, pc_node, 0, TWO23_BITS | pc0, TWO23_BITS | pc1, TWO23_BITS | pc2);
+            pc0 = floor_small(c0); pc1 = floor_small(c1); pc2 = floor_small(c2);
             pc_node = onode;
             v0 = vx; v1 = vy; v2 = vz;
         }
@@ -305,7 +347,10 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         tau_h = tau_l = 0.f;
         nsteps = 0;
         if constexpr (OCT) {
-            s0 = g0; s1 = g1; s2 = g2;
+            // minus the step: as a mask, all ones for a step up and zero or the low
+            // bit (clear in a power of two) otherwise
+            s0 = -g0; s1 = -g1; s2 = -g2;
+            oct_exit(q);
         } else {
             kf0 = (KF)n0; kf1 = (KF)n1; kf2 = (KF)n2;
             sf0 = (KF)g0; sf1 = (KF)g1; sf2 = (KF)g2;
@@ -328,7 +373,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
     auto keep_start = [&]() {
         C.b_t0[t] = tn0; C.b_t1[t] = tn1; C.b_t2[t] = tn2;
         if constexpr (OCT) {
-            C.b_k0[t] = c0; C.b_k1[t] = c1; C.b_k2[t] = c2;
+            C.b_k0[t] = __float_as_int(c0); C.b_k1[t] = __float_as_int(c1); C.b_k2[t] = __float_as_int(c2);
             C.b_m[t] = onode;
         } else {
             if constexpr (BIG) { C.b_k0[t] = kf0; C.b_k1[t] = kf1; C.b_k2[t] = kf2; }
@@ -344,12 +389,13 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         mode = M_LOCATE;
         tn0 = C.b_t0[t]; tn1 = C.b_t1[t]; tn2 = C.b_t2[t];
         if constexpr (OCT) {
-            c0 = C.b_k0[t]; c1 = C.b_k1[t]; c2 = C.b_k2[t];
+            c0 = __int_as_float(C.b_k0[t]); c1 = __int_as_float(C.b_k1[t]); c2 = __int_as_float(C.b_k2[t]);
             onode = C.b_m[t];
-            const int2 h = __ldg(reinterpret_cast<const int2*>(nodes + onode));
-            olev = oct_leaf_level(h.x);
-            cur_m = oct_leaf_index(h.x);
-            kr_cur = __int_as_float(h.y);
+            const OctRec q = oct_load(nodes + onode);
+            olev = oct_leaf_level(q.ref);
+            cur_m = oct_leaf_index(q.ref);
+            kr_cur = q.kr;
+            oct_exit(q);
         } else {
             if constexpr (BIG) { kf0 = C.b_k0[t]; kf1 = C.b_k1[t]; kf2 = C.b_k2[t]; }
             else { kf0 = __int_as_float(C.b_k0[t]); kf1 = __int_as_float(C.b_k1[t]); kf2 = __int_as_float(C.b_k2[t]); }
@@ -387,74 +433,66 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         df_accumulate(tau_h, tau_l, dtau);
     };
 
-    // one leaf crossing of an octree traversal: the face neighbour and its
-    // node are loaded before the crossing's work
+    // One leaf crossing of an octree traversal.  The node across the exit face
+    // is loaded before the crossing's work, all 32 bytes at once: its six
+    // neighbours arrive with its density, so the next crossing's node is known
+    // as soon as its exit face is.  (Loading the neighbour's index by itself
+    // costs a second dependent access: the L1 share holds fewer lines than the
+    // SM's lanes keep in use.)  The lattice corner stays in FP32, where the
+    // entry point's clamp and floor, the alignment to the leaf (a mask on the
+    // bits of c + 2^23) and the next faces need no conversion; the exit axis's
+    // own lattice coordinate is set under its predicate, not by a branch.
+    // 3e6 packets, 8.3e5 leaves: 57.2 -> 40.1 ms; 1e7 packets, 8.2e6 leaves
+    // (nodes 2.4 times the L2): 417 -> 330 ms, the same histories.
     auto step_oct = [&]() {
-        const float tmin = fminf(fminf(tn0, tn1), tn2);
-        const int axis = (tn0 == tmin) ? 0 : ((tn1 == tmin) ? 1 : 2);
-        const int ss = axis == 0 ? s0 : (axis == 1 ? s1 : s2);
-        // a face inside the parent leads to the sibling, whose index follows
-        // from the leaf's own (children blocks start at multiples of 8);
-        // only a face on the parent's boundary needs the stored neighbour
-        const bool inner = olev > 0 && ((onode >> axis) & 1) == (ss < 0 ? 1 : 0);
-        const int nb = inner ? onode ^ (1 << axis) : __ldg(&nodes[onode].nb[2 * axis + (ss > 0)]);
+        const float tmin = oex;
+        const int nb = onb;
         const bool out = nb < 0;
-        const int2 nbh = out ? make_int2(0, 0) : __ldg(reinterpret_cast<const int2*>(nodes + nb));
+        OctRec q = oct_load(nodes + max(nb, 0));
         const float ds = fmaxf(tmin - tcur, 0.f);
         const int m = cur_m;
         const float krl = kr_cur * krs;
         const float dtau = krl * ds;
         ++nsteps;
-        const int run = mode;
         cell_work(m, tmin, dtau, krl);
-        bool done = mode == M_NONE;
-        if (!done) {
-            tcur = tmin;
-            if (out) {
-                done = true;
-            } else if (nsteps > (unsigned)A.oct_step_cap) {
-                atomicOr(A.err, (unsigned)ERRBIT_PATH);
-                done = true;
+        const bool over = nsteps > (unsigned)A.oct_step_cap;
+        if (mode != M_NONE) {
+            if (out || over || tau_h > A.tau_cut) {
+                if (!out && over) atomicOr(A.err, (unsigned)ERRBIT_PATH);
+                mode = M_NONE;
             } else {
-                // lattice cell of the entry point: across the exit face along
-                // `axis`, elsewhere the crossing point's cell kept within the
-                // current leaf's cross-section
-                const int e = 1 << (OL - olev);
-                const float em = __int_as_float((127 + OL - olev) << 23) - 1.f;  // e - 1
-                const float f0 = i2f_small(c0), f1 = i2f_small(c1), f2 = i2f_small(c2);
+                tcur = tmin;
+                last = oax + 1;
+                // lattice cell of the entry point: across the exit face along its
+                // axis, elsewhere the crossing point's cell kept within the current
+                // leaf's cross-section
+                const float em = __int_as_float((127 + OL - olev) << 23) - 1.f;  // the leaf's extent - 1
                 const float p0 = (x0 + tmin * v0 - A.lo_f[0]) * A.id_f[0];
                 const float p1 = (x1 + tmin * v1 - A.lo_f[1]) * A.id_f[1];
                 const float p2 = (x2 + tmin * v2 - A.lo_f[2]) * A.id_f[2];
-                int j0 = floor_small(fminf(fmaxf(p0, f0), f0 + em));
-                int j1 = floor_small(fminf(fmaxf(p1, f1), f1 + em));
-                int j2 = floor_small(fminf(fmaxf(p2, f2), f2 + em));
-                const int ja = ss > 0 ? (axis == 0 ? c0 : (axis == 1 ? c1 : c2)) + e
-                                      : (axis == 0 ? c0 : (axis == 1 ? c1 : c2)) - 1;
-                j0 = axis == 0 ? ja : j0;
-                j1 = axis == 1 ? ja : j1;
-                j2 = axis == 2 ? ja : j2;
+                float f0 = fminf(fmaxf(p0, c0), c0 + em);
+                float f1 = fminf(fmaxf(p1, c1), c1 + em);
+                float f2 = fminf(fmaxf(p2, c2), c2 + em);
+                asm("{\n\t"
+                    ".reg .pred p0, p1, p2;\n\t"
+                    "setp.eq.s32 p0, %3, 0;\n\t"
+                    "setp.eq.s32 p1, %3, 1;\n\t"
+                    "setp.eq.s32 p2, %3, 2;\n\t"
+                    "@p0 add.rn.f32 %0, %4, %7;\n\t"
+                    "@p1 add.rn.f32 %1, %5, %7;\n\t"
+                    "@p2 add.rn.f32 %2, %6, %7;\n\t"
+                    "}"
+                    : "+f"(f0), "+f"(f1), "+f"(f2)
+                    : "r"(oax), "f"(c0), "f"(c1), "f"(c2), "f"(odel));
                 // a neighbour that is not a leaf has the current level
-                if (nbh.x < 0) {
-                    onode = nb;
-                    olev = oct_leaf_level(nbh.x);
-                    cur_m = oct_leaf_index(nbh.x);
-                    kr_cur = __int_as_float(nbh.y);
-                    const int mask = ~((1 << (OL - olev)) - 1);
-                    c0 = j0 & mask;
-                    c1 = j1 & mask;
-                    c2 = j2 & mask;
-                } else {
-                    oct_enter(nb, olev, j0, j1, j2);
-                }
-                const int en = 1 << (OL - olev);
-                tn0 = s0 ? face_t(i2f_small(c0 + (s0 > 0 ? en : 0)), A.d_f[0], A.lo_f[0], x0, iv0) : INF;
-                tn1 = s1 ? face_t(i2f_small(c1 + (s1 > 0 ? en : 0)), A.d_f[1], A.lo_f[1], x1, iv1) : INF;
-                tn2 = s2 ? face_t(i2f_small(c2 + (s2 > 0 ? en : 0)), A.d_f[2], A.lo_f[2], x2, iv2) : INF;
-                last = axis + 1;
+                oct_enter(q, nb, olev, floor_bits(f0), floor_bits(f1), floor_bits(f2));
+                const int en = (127 + OL - olev) << 23;  // the new leaf's extent: a power of two's bits
+                tn0 = s0 ? face_t(c0 + __int_as_float(en & s0), A.d_f[0], A.lo_f[0], x0, iv0) : INF;
+                tn1 = s1 ? face_t(c1 + __int_as_float(en & s1), A.d_f[1], A.lo_f[1], x1, iv1) : INF;
+                tn2 = s2 ? face_t(c2 + __int_as_float(en & s2), A.d_f[2], A.lo_f[2], x2, iv2) : INF;
+                oct_exit(q);
             }
         }
-        if (tau_h > A.tau_cut && run != M_LOCATE) done = true;
-        if (done) mode = M_NONE;
     };
 
     // one cell crossing of the current traversal (Cartesian)
