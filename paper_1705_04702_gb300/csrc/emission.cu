@@ -359,7 +359,12 @@ __device__ __forceinline__ double fixed58_to_double(unsigned long long sum, unsi
 constexpr int BR_WARPS = 4;    // warps per block
 constexpr int BR_STAGES = 2;   // stages of a warp's ring
 constexpr int BR_MAXW = 16;
-__device__ unsigned g_band_timeout;
+// The band starts as a call uploads them: NB + 1 starts, then a zero that a kernel
+// sets when a row copy did not arrive in time.
+constexpr int BAND_INTS = NB + 2;
+
+// a stage holds about 3 KB, or two rows of the widest table
+constexpr size_t BR_SMEM_MAX = 128 + (size_t)BR_WARPS * BR_STAGES * 2 * BR_MAXW * NB * sizeof(double);
 
 // features and total of one row from its band values; s: where the bands start
 template <int W>
@@ -417,7 +422,7 @@ __device__ __forceinline__ void band_row(const double* row, int first, int width
 
 template <int W>
 __global__ void __launch_bounds__(32 * BR_WARPS) band_rows_kernel(
-    const double* __restrict__ A, long long ncell, int n_in, int rows, const int* __restrict__ start,
+    const double* __restrict__ A, long long ncell, int n_in, int rows, const int* __restrict__ start, int* timeout,
     const float* __restrict__ mass, float tiny, float* __restrict__ features, double* __restrict__ total)
 {
     extern __shared__ __align__(128) unsigned char br_smem[];
@@ -449,7 +454,7 @@ __global__ void __launch_bounds__(32 * BR_WARPS) band_rows_kernel(
         if (lane == 0 && ahead < nfull) fetch(ahead, st_ahead);
         const float my_mass = lane < rows ? __ldg(mass + c * rows + lane) : 0.f;
         if (!__all_sync(0xffffffffu, mbar_wait(&bar[st], parity))) {
-            atomicOr(&g_band_timeout, 1u);
+            atomicOr(timeout, 1);
             // the copies still in flight land in this block's memory: give them their time
             for (int k = 1; k < BR_STAGES; ++k) {
                 const int s2 = (st + k) % BR_STAGES;
@@ -475,13 +480,14 @@ __global__ void __launch_bounds__(32 * BR_WARPS) band_rows_kernel(
 }
 
 template <int W>
-cudaError_t launch_band_rows(const double* A, long long ncell, int n_in, const int* d_start, const float* mass,
+cudaError_t launch_band_rows(const double* A, long long ncell, int n_in, int* d_start, const float* mass,
                              float* features, double* total, cudaStream_t s)
 {
     // stages of about 3 KB (an even number of rows, which keeps them 16-byte aligned)
     const int rows = std::min(32, std::max(2, 2 * (3072 / (16 * n_in))));
     const size_t smem = 128 + (size_t)BR_WARPS * BR_STAGES * rows * n_in * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(band_rows_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(band_rows_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)BR_SMEM_MAX);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
@@ -489,7 +495,8 @@ cudaError_t launch_band_rows(const double* A, long long ncell, int n_in, const i
         return e;
     const long long want = (ncell + (long long)rows * BR_WARPS - 1) / ((long long)rows * BR_WARPS);
     const int blocks = (int)std::max<long long>(1, std::min<long long>(want, (long long)sms * std::max(1, per_sm)));
-    band_rows_kernel<W><<<blocks, 32 * BR_WARPS, smem, s>>>(A, ncell, n_in, rows, d_start, mass, 1e-30f, features, total);
+    band_rows_kernel<W><<<blocks, 32 * BR_WARPS, smem, s>>>(A, ncell, n_in, rows, d_start, d_start + NB + 1, mass, 1e-30f, features,
+                                                     total);
     return cudaGetLastError();
 }
 
@@ -1074,15 +1081,12 @@ __global__ void zero_temperature_kernel(float* t, long long n)
 }
 
 // band compression on either kernel; start: the host's copy of d_start
-cudaError_t launch_band_features(const double* A, long long ncell, int n_in, const std::vector<int>& start,
-                                 const int* d_start, const float* mass, float* features, double* total, cudaStream_t s)
+cudaError_t launch_band_features(const double* A, long long ncell, int n_in, const std::vector<int>& start, int* d_start,
+                                 const float* mass, float* features, double* total, cudaStream_t s)
 {
     int w = 0;
     for (int b = 0; b < NB; ++b) w = std::max(w, start[b + 1] - start[b]);
     if ((reinterpret_cast<uintptr_t>(A) & 15) == 0 && w <= BR_MAXW && n_in <= BR_MAXW * NB) {
-        const unsigned zero = 0;
-        cudaError_t e = cudaMemcpyToSymbolAsync(g_band_timeout, &zero, sizeof zero, 0, cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) return e;
         if (w <= 4) return launch_band_rows<4>(A, ncell, n_in, d_start, mass, features, total, s);
         if (w <= 8) return launch_band_rows<8>(A, ncell, n_in, d_start, mass, features, total, s);
         return launch_band_rows<16>(A, ncell, n_in, d_start, mass, features, total, s);
@@ -1091,14 +1095,10 @@ cudaError_t launch_band_features(const double* A, long long ncell, int n_in, con
     return cudaGetLastError();
 }
 
-// after the stream has synchronised: an error when a launch gave up waiting for a copy
-int band_check_timeout()
+// after the stream has synchronised: an error when the call gave up waiting for a copy
+int band_check_timeout(int v)
 {
-    unsigned v = 0;
-    const cudaError_t e = cudaMemcpyFromSymbol(&v, g_band_timeout, sizeof v);
-    if (e != cudaSuccess) return set_error(SKIRT_ERR_CUDA, "band features: %s", cudaGetErrorString(e));
-    if (v) return set_error(SKIRT_ERR_CUDA, "band compression: a row copy did not complete in time");
-    return SKIRT_OK;
+    return v ? set_error(SKIRT_ERR_CUDA, "band compression: a row copy did not complete in time") : SKIRT_OK;
 }
 
 int grid_blocks(long long n, int block)
@@ -1148,6 +1148,7 @@ std::vector<int> band_starts(const double* lam, int n)
             if (idx[j] >= b) { s = j; break; }
         start[b] = b == NB ? n : s;
     }
+    start.push_back(0);
     return start;
 }
 
@@ -1210,7 +1211,7 @@ int launch_exact_emission(const double* absorbed, int n_in, const double* w_dev,
     if (nrows > 0) {
         // full batches once there are enough rows for them to fill the warps the
         // device holds (152 SMs x 24); below that as many warps as rows allow, each
-        // with fewer rows in series (2000 rows: 115 us by tens, one by one below)
+        // with fewer rows in series (2000 rows: 115 us by tens, 28 us one by one)
         const long long warps = 152LL * 24;
         const int batch = (int)std::min<long long>(EX_BATCH, (nrows + warps - 1) / warps);
         long long blocks = (nrows + EX_WARPS * batch - 1) / (EX_WARPS * batch);
@@ -1258,13 +1259,15 @@ extern "C" int skirt_band_features(const double* absorbed, long long ncell, int 
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<int> start = band_starts(lambda_in, n_in);
     int* d_start = nullptr;
-    ECK(cudaMallocAsync((void**)&d_start, sizeof(int) * (NB + 1), s));
-    ECK(cudaMemcpyAsync(d_start, start.data(), sizeof(int) * (NB + 1), cudaMemcpyHostToDevice, s));
-    const cudaError_t e = launch_band_features(absorbed, ncell, n_in, start, d_start, mass, features, total, s);
+    int timeout = 0;
+    ECK(cudaMallocAsync((void**)&d_start, sizeof(int) * BAND_INTS, s));
+    ECK(cudaMemcpyAsync(d_start, start.data(), sizeof(int) * BAND_INTS, cudaMemcpyHostToDevice, s));
+    cudaError_t e = launch_band_features(absorbed, ncell, n_in, start, d_start, mass, features, total, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&timeout, d_start + NB + 1, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaFreeAsync(d_start, s);
     if (e != cudaSuccess) return set_error(SKIRT_ERR_CUDA, "band features: %s", cudaGetErrorString(e));
     ECK(cudaStreamSynchronize(s));
-    return band_check_timeout();
+    return band_check_timeout(timeout);
 }
 
 extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int n_in, const double* lambda_in,
@@ -1288,7 +1291,7 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
     ECK(cudaMemcpyAsync(d_w, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice, s));
     cudaEvent_t ev[4];
     for (auto& e : ev) ECK(cudaEventCreate(&e));
-    int rc = SKIRT_OK;
+    int rc = SKIRT_OK, timeout = 0;
     unsigned long long nfb = 0;
     if (mode == SKIRT_EMIT_EXACT) {
         ECK(cudaEventRecord(ev[0], s));
@@ -1306,7 +1309,7 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
         } drain{s};
         auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
         const size_t o_tot = 0, o_cnt = o_tot + al(sizeof(double) * (size_t)ncell), o_start = o_cnt + al(8),
-                     o_feat = o_start + al(sizeof(int) * (NB + 1)),
+                     o_feat = o_start + al(sizeof(int) * BAND_INTS),
                      o_rows = o_feat + al(sizeof(float) * NB * (size_t)ncell),
                      o_flag = o_rows + al(sizeof(unsigned) * (size_t)ncell), ws_total = o_flag + al((size_t)ncell);
         unsigned char* ws = nullptr;
@@ -1323,7 +1326,7 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
         unsigned char* d_flag = ws + o_flag;
         ECK(cudaMemsetAsync(d_cnt, 0, sizeof(unsigned long long), s));
         std::vector<int> start = band_starts(lambda_in, n_in);
-        ECK(cudaMemcpyAsync(d_start, start.data(), sizeof(int) * (NB + 1), cudaMemcpyHostToDevice, s));
+        ECK(cudaMemcpyAsync(d_start, start.data(), sizeof(int) * BAND_INTS, cudaMemcpyHostToDevice, s));
         if (temperature) zero_temperature_kernel<<<grid_blocks(3 * ncell, 256), 256, 0, s>>>(temperature, 3 * ncell);
         ECK(cudaEventRecord(ev[0], s));
         ECK(launch_band_features(absorbed, ncell, n_in, start, d_start, mass, d_feat, d_tot, s));
@@ -1334,6 +1337,7 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
             ECK(cudaGetLastError());
             ECK(cudaEventRecord(ev[2], s));
             ECK(cudaMemcpyAsync(&nfb, d_cnt, sizeof nfb, cudaMemcpyDeviceToHost, s));
+            ECK(cudaMemcpyAsync(&timeout, d_start + NB + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
             ECK(cudaStreamSynchronize(s));
             rc = launch_exact_emission(absorbed, n_in, d_w, mass, d_rows, (long long)nfb, emission, temperature, s);
             ECK(cudaEventRecord(ev[3], s));
@@ -1342,7 +1346,7 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
     cudaFreeAsync(d_w, s);
     ECK(cudaStreamSynchronize(s));
     if (rc == SKIRT_OK && mode == SKIRT_EMIT_SURROGATE) rc = mlp_check_timeout();
-    if (rc == SKIRT_OK && mode == SKIRT_EMIT_SURROGATE) rc = band_check_timeout();
+    if (rc == SKIRT_OK && mode == SKIRT_EMIT_SURROGATE) rc = band_check_timeout(timeout);
     if (stats && rc == SKIRT_OK) {
         stats->n_cells = (unsigned long long)ncell;
         stats->n_fallback = nfb;
