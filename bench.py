@@ -389,11 +389,11 @@ def run_selfabs_report(args):
 # the committed ncu capture of the kernel as it stands
 # (profiles/trace_mixed_kernel_disk256_3e6_full.md); None when the kernel has
 # changed since.
-ISSUE_INST_PER_PACKET = 23468.0
+ISSUE_INST_PER_PACKET = 15076.0
 # DRAM bytes (read + write) per packet of the trace kernel from one ncu
 # capture of a 3e6-packet launch of the kernel as it stands (profiles/),
 # scaled by the packets of the launch; None when the kernel has changed since.
-TRAFFIC_PER_PACKET = {"disk": 30254.0, "octree": 102039.0}
+TRAFFIC_PER_PACKET = {"disk": 20677.0, "octree": 100140.0}
 
 
 def trace_rooflines(led, packets, k_ms, ninstr, red_rate, peak, peak_kind, kernel, crossing_bytes, traffic_pp,
@@ -603,7 +603,7 @@ def main():
     k_ms = float(np.mean(kernel_ms))
     key = "octree" if octree else ("disk" if args.workload == "disk" and args.grid == 256 else None)
     roofs = trace_rooflines(led, packets, k_ms, len(prob.instruments), red_rate, peak, peak_kind,
-                            "trace_mixed_kernel<true> (octree)" if octree else "trace_mixed_kernel",
+                            "trace_mixed_kernel (octree)" if octree else "trace_mixed_kernel",
                             12 if octree else 4, TRAFFIC_PER_PACKET.get(key) if key else None,
                             clk["sm_mhz"] if clk else None, sm_count if key == "disk" else None)
 
@@ -676,7 +676,7 @@ def main():
             "roofline_sector": roof_sector,
             "cpu_baseline": cpu,
             "e2e": e2e,
-            "gpu_launches": args.steps * (1 + len(prob.instruments) + (1 if n > 1 else 0)),
+            "gpu_launches": args.steps * (1 + len(prob.instruments) + (1 if n > 1 or args.workload == "disk" else 0)),
             "clocks": clk,
             "plain_fp64": fp64,
             "speedup_vs_plain_fp64": (value / world / fp64["value"]) if fp64 else None,

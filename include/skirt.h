@@ -233,10 +233,13 @@ typedef struct {
  * images and sed may be NULL when ninstr == 0.  ledger (host) may be NULL;
  * ledger_per_lambda (host double[n][4], emitted/absorbed/escaped/residual)
  * may be NULL.
- * With n > 1 the packets deposit into a wavelength-major copy of the
- * absorbed table ([n][ncell], grid scratch of the same size as the table)
- * that one transpose turns into the [ncell][n] result (or adds to it with
- * accumulate); without room for the copy they deposit in place.
+ * With n > 1, and in the mixed form on a Cartesian grid whose cells are
+ * thinnest along y or z (at most 3/4 of their size along x; such cells
+ * are numbered along that axis while packets are traced), the packets deposit
+ * into a wavelength-major copy of the absorbed table ([n][ncell], grid scratch
+ * of the same size as the table) that one transpose turns into the [ncell][n]
+ * result (or adds to it with accumulate); without room for the copy they
+ * deposit in place.
  * Limits: npackets[j] < 2^32; 0 <= ninstr <= 16.
  * Errors: INVALID_ARG, OOM, CUDA; EVENT_CAP / NONFINITE / SOURCE after a
  * completed trace whose ledger flagged the condition (NONFINITE also for an
