@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
         if (s >= 0) v = A.feat ? (A.feat[s * NIN + c] - A.stats[c]) * A.stats[NIN + c] : A.x_std[s * NIN + c];
         X[r * P1 + c] = bf16_bits(v);
     }
-    // the dependents are let go only now, so that they start after the previous
-    // step's results are complete (the gradient sum reads its moments right away)
+    // the dependents are let go only now: they wait for this kernel, and so for the
+    // previous step's results as well
     wait_predecessor();
     launch_dependents();
     // ---- the weights by asynchronous copies of 16 bytes into padded rows, each
@@ -533,16 +533,17 @@ __global__ void __launch_bounds__(32 * TWARPS, 1) train_tile_kernel(const TileAr
 
 // g = sum over the CTAs of their partial gradients (in CTA order); with
 // adam: the Adam step of the FP32 parameters and their BF16 copies for the
-// next step.  The last block instead sums the loss (partials in CTA order) and,
-// at the end of a graph, moves the step counter on by the graph's steps (every
-// other block of the graph has read it by then).
+// next step.  The last block instead sums the loss (partials in CTA order).
+// Nothing of the previous step is read before wait_predecessor: what a kernel
+// wrote is promised only to kernels that wait for it, and the chain of waits
+// leads from a sum through the next tile kernel to the next sum.  The step
+// counter and the schedule do not change within a graph.
 constexpr int RED_T = 128;   // threads per block
 constexpr int RED_C = 64;    // partials per chunk
 __global__ void __launch_bounds__(RED_T) train_reduce_kernel(
     const float* __restrict__ part, const float* __restrict__ part_loss, int ncta, float* __restrict__ G, int adam,
     float* __restrict__ P, float* __restrict__ Mo, float* __restrict__ Vo, const float* __restrict__ sched,
-    long long* t_dev, int ahead, int advance, float b1, float b2, float eps, uint16_t* __restrict__ Wb,
-    float* loss_acc)
+    const long long* t_dev, int ahead, float b1, float b2, float eps, uint16_t* __restrict__ Wb, float* loss_acc)
 {
     launch_dependents();
     if (blockIdx.x == gridDim.x - 1) {
@@ -557,26 +558,24 @@ __global__ void __launch_bounds__(RED_T) train_reduce_kernel(
                 for (int c = 0; c < n; ++c) l += sl[c];
             __syncthreads();
         }
-        if (threadIdx.x == 0) {
-            *loss_acc += l;
-            if (advance) *t_dev += advance;
-        }
+        if (threadIdx.x == 0) *loss_acc += l;
         return;
     }
     const int i = blockIdx.x * RED_T + threadIdx.x;
     const bool mine = i < NPARAM;
     float mi = 0.f, vi = 0.f, p = 0.f, lr = 0.f, c1 = 1.f, c2 = 1.f;
     if (adam && mine) {
-        // the previous step's results, complete before this kernel could start
         const long long st = *t_dev + ahead;
         lr = sched[3 * st];
         c1 = sched[3 * st + 1];
         c2 = sched[3 * st + 2];
+    }
+    wait_predecessor();
+    if (adam && mine) {
         mi = Mo[i];
         vi = Vo[i];
         p = P[i];
     }
-    wait_predecessor();
     float gi = 0.f;
     // a chunk of partials of the block's 128 parameters by asynchronous copies, all
     // in flight at once, then added in order
@@ -613,6 +612,10 @@ __global__ void __launch_bounds__(RED_T) train_reduce_kernel(
         if (w >= 0) Wb[w] = bf16_bits(p);
     }
 }
+
+// Moves the step counter on at the end of a graph: a kernel of its own, launched
+// without the early start, so that every block that reads the counter has ended.
+__global__ void advance_step_kernel(long long* t_dev, int steps) { *t_dev += steps; }
 
 }  // namespace
 
@@ -664,8 +667,11 @@ cudaError_t launch_train_step(const uint16_t* Wb, const float* P, const float* f
     cfg.gridDim = dim3((NPARAM + RED_T - 1) / RED_T + 1);
     cfg.blockDim = dim3(RED_T);
     cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, train_reduce_kernel, (const float*)part, (const float*)part_loss, ncta, G, adam, Pw,
-                              Mo, Vo, sched, t_dev, ahead, advance, b1, b2, eps, Wb_out, loss_acc);
+    e = cudaLaunchKernelEx(&cfg, train_reduce_kernel, (const float*)part, (const float*)part_loss, ncta, G, adam, Pw, Mo,
+                           Vo, sched, (const long long*)t_dev, ahead, b1, b2, eps, Wb_out, loss_acc);
+    if (e != cudaSuccess || advance == 0) return e;
+    advance_step_kernel<<<1, 1, 0, s>>>(t_dev, advance);
+    return cudaGetLastError();
 }
 
 }  // namespace skirt
