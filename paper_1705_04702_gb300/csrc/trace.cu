@@ -139,6 +139,7 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
     double tcur = 0;
     double tau = 0.0;                  // optical depth along this traversal
     double par = 0.0;                  // deposit: L (1 - albedo) e^{-tau}; search: interaction optical depth
+    double taken = 0.0;                // deposit: what the cells have taken, the ledger's absorbed power
     double s_found = 0, last_dusty_end = 0;
     bool found = false;
     unsigned nsteps = 0;
@@ -255,8 +256,10 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
         } else if (mode == M_DEPOSIT) {
             if (bits(dtau) > 0) {
                 const double dep = take(dtau, par);
-                if (bits(dep) > 0)
+                if (bits(dep) > 0) {
                     atomicAdd(A.absorbed + ((size_t)cur_m * A.abs_cs + (size_t)lam * A.abs_ls), dep);
+                    taken += dep;
+                }
             }
         } else if (bits(krl) > 0) {
             if (bits(tau_n) >= bits(par)) {
@@ -371,7 +374,7 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
                 I(I_C_DEP) += (int)nsteps;
                 const double om = -expm1(-tau);  // what the path takes
                 D(D_P_ESC) += L * exp(-tau);
-                D(D_P_ABS) += D(D_LABS) * om;
+                D(D_P_ABS) += taken;
                 if (!(tau > 0.0)) {
                     if (!(tau == 0.0)) atomicOr(A.err, (unsigned)ERRBIT_NONFINITE);
                     L = 0.0;
@@ -601,6 +604,7 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
                 I(I_EV) += 1;
                 par = L * (1.0 - D(D_ALB));
                 D(D_LABS) = par;
+                taken = 0.0;
                 need = M_DEPOSIT;
                 i0 = k0 != 0.0 ? 1.0 / k0 : 0.0;
                 i1 = k1 != 0.0 ? 1.0 / k1 : 0.0;
