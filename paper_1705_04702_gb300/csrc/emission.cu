@@ -519,11 +519,20 @@ int band_blocks(long long ncell)
 //
 //  * The powers are sums in 64-bit integers.  The inputs of a block of 256
 //    columns become fixed-point numbers relative to the largest (59 bits), the
-//    shares carry 58 bits, and a product is three 32-bit multiply-adds into
-//    64-bit sums; what is cut off stays below 2^-57 of the largest product, so
-//    the sums are as exact as FP64 ones and do not depend on their order.  A
-//    block with a negative or non-finite entry, or none above 2^-895, is summed
-//    in FP64 instead.
+//    shares relative to the population's largest in the block (58 bits), and a
+//    product is three 32-bit multiply-adds into 64-bit sums, which do not depend
+//    on their order.  A sum's unit is 2^-56 of the largest entry times the scale
+//    of the shares; its roundings make 3 units (200 columns; 1.5 for 20), and what
+//    is cut off entries below 1/64 of the largest 0.05 units each.  A population
+//    whose sum holds at least 2^55 units (2^54 up to 64 columns) so has it to 0.7 x
+//    2^-53, or 3 x 2^-53 if nearly all entries are that small; 200 FP64 additions in
+//    the lanes' order come to 0.8 x 2^-53 in the mean and 13 x 2^-53 at most.
+//    Where a sum holds fewer (the power lies in few columns, or where the
+//    population's share is small: without the test a share of 5e-4 (1000 micron)
+//    cost 5e-14 of that population's power, one of 5e-7 4e-11) the block is summed
+//    in FP64 instead, and so is one with a negative or non-finite entry, or none
+//    above 2^-895.  A power of two per entry and population instead of the test
+//    took 13% more time for every row.
 //  * Per population (FP64, lane 3r + i holds row r's population i, so the rows
 //    share each FP64 instruction): the target, the clamp to 3 or 2000 K, the
 //    start 1/T_i (cubic Hermite in ln G, on points equally spaced in it: no
@@ -797,10 +806,17 @@ __device__ __forceinline__ double start_invT(int i, double target, int stride, i
 }
 
 // The sums of a block of up to 256 columns of a row, sum_j w_ij A_j of the three
-// populations, in fixed point: value = s 2^(e - 1078), e the biased exponent of
-// the block's largest entry.  False (nothing summed) for a block with a negative or
-// non-finite entry, or none above 2^-895 but one above zero.
+// populations, in fixed point: value = s_i 2^(e - 1078 - x_i), e the biased exponent
+// of the block's largest entry, 2^-x_i the scale of the population's shares in the
+// block.  False (nothing summed) for a block with a negative or non-finite entry,
+// none above 2^-895 but one above zero, or too few units in a sum.
 constexpr int EX_COLS = 256;
+constexpr int SHARE_MAX_EXP = 60;                    // largest x_i
+// x_i of the block whose shares start at wq (one byte each)
+__device__ __forceinline__ int share_scale(const int4* wq, int i)
+{
+    return (int)(((unsigned)__ldg(&wq[1].z) >> (8 * i)) & 0xFFu);
+}
 
 __device__ __forceinline__ void mad_wide(unsigned long long& acc, unsigned a, int b)
 {
@@ -813,7 +829,7 @@ __device__ __forceinline__ void mad_wide(long long& acc, unsigned a, int b)
 }
 
 // wq: the shares' fixed-point pairs, 32 bytes per wavelength: hi, lo of the three
-// populations, 8 bytes of padding (two 16-byte loads)
+// populations, the block's packed x_i, 4 bytes of padding (two 16-byte loads)
 __device__ __forceinline__ bool block_powers(const double* __restrict__ row, int n, const int4* __restrict__ wq,
                                              int lane, unsigned long long& s0, unsigned long long& s1,
                                              unsigned long long& s2, int& e)
@@ -833,8 +849,8 @@ __device__ __forceinline__ bool block_powers(const double* __restrict__ row, int
     // all zero, or too small for a subnormal entry to shift out
     if (mx < 0x08000000u) return mx == 0u && __reduce_or_sync(0xffffffffu, any) == 0u;
     e = (int)(mx >> 20);
-    // products a w: a = v 2^(1081 - e) as hi (27 bits) and lo (32 bits), w 2^58 as
-    // hi (29 bits, unsigned) and lo (28 bits and sign); partial sums of up to 8
+    // products a w: a = v 2^(1081 - e) as hi (27 bits) and lo (32 bits), w 2^(58 + x)
+    // as hi (29 bits, unsigned) and lo (28 bits and sign); partial sums of up to 8
     unsigned long long hh0 = 0, hh1 = 0, hh2 = 0, lh0 = 0, lh1 = 0, lh2 = 0;
     long long hl0 = 0, hl1 = 0, hl2 = 0;
 #pragma unroll
@@ -867,7 +883,8 @@ __device__ __forceinline__ bool block_powers(const double* __restrict__ row, int
     s1 = hh1 + (unsigned long long)((hl1 + (1ll << 28)) >> 29) + ((lh1 + (1ull << 31)) >> 32);
     s2 = hh2 + (unsigned long long)((hl2 + (1ll << 28)) >> 29) + ((lh2 + (1ull << 31)) >> 32);
     warp_sum3(s0, s1, s2);
-    return true;
+    const unsigned least = min((unsigned)(s0 >> 32), min((unsigned)(s1 >> 32), (unsigned)(s2 >> 32)));
+    return least >= (n <= 64 ? 1u << 22 : 1u << 23);
 }
 
 // s 2^(e - 1078)
@@ -939,7 +956,7 @@ __global__ void __launch_bounds__(32 * EX_WARPS, 7) exact_kernel(
                         const unsigned long long sv = my_i == 0 ? s0 : (my_i == 1 ? s1 : s2);
                         if (c > 0) {
                             more = true;
-                            if (my_r == r) rest += fixed_to_double(sv, e);
+                            if (my_r == r) rest += fixed_to_double(sv, e - share_scale(wq + 2 * c, my_i));
                         } else if (my_r == r) {
                             if (tab) { sb = sv; eb = e; } else { sa = sv; ea = e; }
                         }
@@ -952,8 +969,8 @@ __global__ void __launch_bounds__(32 * EX_WARPS, 7) exact_kernel(
                 }
             }
         }
-        double P = fixed_to_double(sa, ea);
-        if (A2) P += fixed_to_double(sb, eb);
+        double P = fixed_to_double(sa, ea - share_scale(reinterpret_cast<const int4*>(w), my_i));
+        if (A2) P += fixed_to_double(sb, eb - share_scale(reinterpret_cast<const int4*>(w2), my_i));
         if (more) P += rest;
         // binary exponent of the row's largest population power (0 if none is positive)
         const int xe = P > 0.0 ? (__double2hiint(P) >> 20) + 1 : 0;
@@ -1153,27 +1170,48 @@ std::vector<int> band_starts(const double* lam, int n)
 }
 
 // shares w_i(lambda_j) = (lambda_j/0.55)^delta_i / sum_k (lambda_j/0.55)^delta_k:
-// first their fixed-point pairs for block_powers, w 2^58 = hi 2^29 + lo, |lo| <=
-// 2^28, 32 bytes per wavelength, then the shares themselves [3][n]; 8 doubles per
-// wavelength in all, so that a second table behind the first stays aligned
+// first their fixed-point pairs for block_powers, w 2^(58 + x) = hi 2^29 + lo, |lo|
+// <= 2^28, with 2^-x the power of two from the population's largest share among the
+// wavelength's block of EX_COLS on, 32 bytes per wavelength, then the shares
+// themselves [3][n]; 8 doubles per wavelength in all, so that a second table behind
+// the first stays aligned
 constexpr int SHARES = 8;
 void fill_shares(const double* lam, int n, double* out)
 {
     double* w = out + 4 * (size_t)n;
-    for (int j = 0; j < n; ++j) {
-        double r[NPOP], sum = 0.0;
-        for (int i = 0; i < NPOP; ++i) {
-            r[i] = std::pow(lam[j] / 0.55, DELTA[i]);
-            sum += r[i];
+    for (int c = 0; c < n; c += EX_COLS) {
+        const int end = std::min(n, c + EX_COLS);
+        double top[NPOP] = {};
+        for (int j = c; j < end; ++j) {
+            double r[NPOP], sum = 0.0;
+            for (int i = 0; i < NPOP; ++i) {
+                r[i] = std::pow(lam[j] / 0.55, DELTA[i]);
+                sum += r[i];
+            }
+            for (int i = 0; i < NPOP; ++i) {
+                w[(size_t)i * n + j] = r[i] / sum;
+                top[i] = std::max(top[i], w[(size_t)i * n + j]);
+            }
         }
-        int q[8] = {};
+        double scale[NPOP];
+        unsigned packed = 0u;
         for (int i = 0; i < NPOP; ++i) {
-            const double v = r[i] / sum, h = std::floor(v * 536870912.0 + 0.5);
-            w[(size_t)i * n + j] = v;
-            q[2 * i] = (int)h;
-            q[2 * i + 1] = (int)std::floor((v * 536870912.0 - h) * 536870912.0 + 0.5);
+            int x;
+            std::frexp(top[i], &x);
+            x = std::min(std::max(-x, 0), SHARE_MAX_EXP);
+            packed |= (unsigned)x << (8 * i);
+            scale[i] = std::ldexp(536870912.0, x);
         }
-        std::memcpy(out + 4 * (size_t)j, q, sizeof q);
+        for (int j = c; j < end; ++j) {
+            int q[8] = {};
+            for (int i = 0; i < NPOP; ++i) {
+                const double v = w[(size_t)i * n + j] * scale[i], h = std::floor(v + 0.5);
+                q[2 * i] = (int)h;
+                q[2 * i + 1] = (int)std::floor((v - h) * 536870912.0 + 0.5);
+            }
+            q[6] = (int)packed;
+            std::memcpy(out + 4 * (size_t)j, q, sizeof q);
+        }
     }
 }
 
