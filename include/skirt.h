@@ -180,8 +180,8 @@ typedef struct {
     int accumulate;    /* 0: outputs are zeroed first; 1: tallies are added to their contents */
     int block;         /* threads per block: a multiple of 32, up to 256 (mixed form) or 512
                           (FP64 form); 0 = default 256 */
-    int chunk;         /* packets a thread takes per queue refill (persistent), fewer where they would not
-                          leave every thread eight refills; 0 = default */
+    int chunk;         /* packets a thread takes per queue refill (persistent); 0 = default: 4, or
+                          fewer where 4 would not leave every thread eight refills */
     int blocks_per_sm; /* persistent grid = blocks_per_sm x SM count; 0 = from occupancy */
     int use_graph;     /* 1: record the launch sequence in a CUDA graph, cached on the grid
                           and replayed by later calls with identical arguments */

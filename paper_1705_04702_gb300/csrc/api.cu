@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "queue_chunk.cuh"
 #include "skirt_internal.cuh"
 
 using namespace skirt;
@@ -151,7 +152,7 @@ extern "C" int skirt_trace_opts_default(skirt_trace_opts* o)
     o->max_events = 10000;
     o->peel = 1;
     o->block = 256;
-    o->chunk = 4;
+    o->chunk = 0;
     return SKIRT_OK;
 }
 
@@ -613,17 +614,7 @@ extern "C" int skirt_trace(skirt_grid_t g, const skirt_source* src, const skirt_
         if (bps < 1) bps = 1;
     }
     const int pgrid = g->sm_count * bps;
-    // Packets a thread takes per queue refill: what was asked for, but no more than
-    // leaves every thread eight refills.  Fewer starve the launch's end, or, below a
-    // refill per thread, most of the launch: 1e5 packets in the sphere took 1.68 ms by
-    // fours and take 1.00 ms one by one, 3e5 on an octree 12.6 and 7.8 ms; where there
-    // is work for many refills, single packets cost more in queue traffic (2e6 dust
-    // packets 14.9 ms against 13.8 ms by twos).
-    A.chunk = opts->chunk > 0 ? opts->chunk : 4;
-    {
-        const unsigned long long fair = P.total / (8ull * (unsigned long long)pgrid * (unsigned long long)block);
-        if ((unsigned long long)A.chunk > fair) A.chunk = fair > 0 ? (int)fair : 1;
-    }
+    A.chunk = queue_chunk(opts->chunk, P.total, (unsigned long long)pgrid * (unsigned long long)block);
 
     // ---- the device work of one call (recorded into a graph when asked)
     auto enqueue = [&](cudaStream_t s, bool events) -> int {
@@ -789,16 +780,19 @@ extern "C" int skirt_autotune(skirt_grid_t g, const skirt_source* src, const ski
     const bool mixed = o.precision == SKIRT_PREC_MIXED;
     const bool oct = g->oct_levels > 0;
 
-    // the candidates: the requested schedule (defaults resolved), then the sweep
+    // the candidates: the requested schedule (defaults resolved for the full run,
+    // which the default refill depends on), then the sweep
+    unsigned long long ntotal = 0;
+    for (int j = 0; j < wl->n; ++j) ntotal += npk[j];
     std::vector<skirt_tune_point> cand;
     {
         skirt_tune_point p{};
         p.block = o.block > 0 ? o.block : 256;
-        p.chunk = o.chunk > 0 ? o.chunk : 4;
         p.step_min = o.step_min > 0 ? o.step_min : 20;
         int maxbps = 0;
         CK(trace_occupancy(o.precision, p.block, &maxbps, oct));
         p.blocks_per_sm = o.blocks_per_sm > 0 ? o.blocks_per_sm : (maxbps > 0 ? maxbps : 1);
+        p.chunk = queue_chunk(o.chunk, ntotal, (unsigned long long)g->sm_count * p.blocks_per_sm * p.block);
         cand.push_back(p);
     }
     const int blocks[4] = {64, 128, 256, 512};
