@@ -32,6 +32,7 @@
 
 #include "skirt_internal.cuh"
 #include "trace_device.cuh"
+#include "work_count.cuh"
 
 namespace skirt {
 namespace {
@@ -51,7 +52,7 @@ enum {
     D_NUM
 };
 enum {
-    I_C_DEP, I_C_LOC, I_C_PEEL, I_C_SCAT,  // added to the 64-bit counters below 2^32
+    I_C_DEP, I_C_LOC, I_C_PEEL, I_C_SCAT,  // emptied into the 64-bit counters (count_add)
     I_LAM, I_NSCAT, I_PEEL_I, I_PK, I_EV, I_RY, I_RZ, I_LEFT, I_QLO, I_QHI,
     I_B_0, I_B_1, I_B_2, I_B_M,            // start of the deposit traversal: cell (lattice corner) and index (node)
     I_NUM
@@ -347,10 +348,17 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
     // again only where no traversal came of a pass (a peel-off of zero weight).
     auto events = [&]() {
         int need;
+        const auto count = [&](int which, unsigned n) {
+            unsigned c = (unsigned)I(which);
+            const bool full = count_add(c, n);
+            I(which) = (int)c;
+            return full;
+        };
         do {
             need = M_NONE;
+            bool full = false;  // a work counter is to be emptied
             if (stage == ST_PEEL_DONE) {
-                I(I_C_PEEL) += (int)nsteps;
+                full = count(I_C_PEEL, nsteps);
                 const int pk = I(I_PEEL_I), pi = pk & (PEEL_SCATTER - 1);
                 const InstrDev& S = sins[pi];
                 const double w = D(D_PEEL_W);
@@ -371,7 +379,7 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
                 I(I_PEEL_I) = pk + 1;
                 stage = pi + 1 < A.ninstr ? ST_PEEL : (pk & PEEL_SCATTER ? ST_AFTER_SCATTER : ST_START_DEP);
             } else if (stage == ST_DEPOSIT_DONE) {
-                I(I_C_DEP) += (int)nsteps;
+                count(I_C_DEP, nsteps);  // emptied, if need be, behind the search that follows
                 const double om = -expm1(-tau);  // what the path takes
                 D(D_P_ESC) += L * exp(-tau);
                 D(D_P_ABS) += taken;
@@ -407,7 +415,7 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
                     break;
                 }
             } else if (stage == ST_LOCATE_DONE) {
-                I(I_C_LOC) += (int)nsteps;
+                full = count(I_C_LOC, nsteps) || count(I_C_DEP, 0u);
                 const double s = found ? s_found : last_dusty_end;
                 x0 += s * k0;
                 x1 += s * k1;
@@ -445,9 +453,9 @@ __global__ void __launch_bounds__(FP64_MAXB) trace_kernel(const TraceArgs A)
                 }
             }
 
+            if (stage == ST_END_PACKET) full = count(I_C_SCAT, (unsigned)I(I_NSCAT)) || full || count(I_C_DEP, 0u);
+            if (full) flush_counters();
             if (stage == ST_END_PACKET) {
-                I(I_C_SCAT) += I(I_NSCAT);
-                if ((unsigned)(I(I_C_SCAT) | I(I_C_DEP) | I(I_C_LOC) | I(I_C_PEEL)) >> 30) flush_counters();
                 const double pe = D(D_P_ESC), pa = D(D_P_ABS), pr = D(D_P_RES), pp = D(D_P_PEEL);
                 D(D_L_ABS) += pa;
                 D(D_L_ESC) += pe;

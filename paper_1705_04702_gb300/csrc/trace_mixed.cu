@@ -57,6 +57,7 @@
 
 #include "skirt_internal.cuh"
 #include "trace_device.cuh"
+#include "work_count.cuh"
 
 namespace skirt {
 namespace {
@@ -160,7 +161,7 @@ struct Cold {
     double l_emit[MAXB], l_abs[MAXB], l_esc[MAXB], l_res[MAXB];
     unsigned long long q[MAXB];
     unsigned left[MAXB];                                        // packets left of the last queue refill
-    unsigned c_dep[MAXB], c_loc[MAXB], c_peel[MAXB], c_scat[MAXB];  // added to the 64-bit counters below 2^32
+    unsigned c_dep[MAXB], c_loc[MAXB], c_peel[MAXB], c_scat[MAXB];  // emptied into the 64-bit counters
     float L0[MAXB], p_esc[MAXB], p_abs[MAXB], p_res[MAXB], p_peel[MAXB], om[MAXB], peel_w[MAXB], alb[MAXB];
     float xl0[MAXB], xl1[MAXB], xl2[MAXB];  // low words of the double-float position
     int lam[MAXB], nscat[MAXB], peel_i[MAXB];  // peel_i: instrument, + PEEL_SCATTER after a scattering
@@ -208,7 +209,12 @@ __device__ __forceinline__ OctRec oct_load(const OctNode* p)
 // cell of the entry point.
 enum { G_CART = 0, G_CART_BIG = 1, G_OCT = 2 };
 
-template <int G>
+//
+// LONG: the work counters are emptied at every event.  Only a run whose packets may
+// make more than 2^32 crossings each needs it (counts_within_packet): in the other
+// kernels that check, a few instructions per event, cost 2% of the disk and torus
+// runs.
+template <int G, bool LONG>
 __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
 {
     constexpr bool OCT = G == G_OCT, BIG = G == G_CART_BIG;
@@ -601,7 +607,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
         do {
             need = M_NONE;
             if (stage == ST_PEEL_DONE) {
-                C.c_peel[t] += nsteps;
+                if (count_add(C.c_peel[t], nsteps) && LONG) flush_counters();
                 const int pk = C.peel_i[t], pi = pk & (PEEL_SCATTER - 1);
                 const InstrDev& I = sins[pi];
                 const float w = C.peel_w[t];
@@ -630,7 +636,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                 C.peel_i[t] = pk + 1;
                 stage = pi + 1 < A.ninstr ? ST_PEEL : (pk & PEEL_SCATTER ? ST_AFTER_SCATTER : ST_START_DEP);
             } else if (stage == ST_DEPOSIT_DONE) {
-                C.c_dep[t] += nsteps;
+                if (count_add(C.c_dep[t], nsteps) && LONG) flush_counters();
                 // om = 1 - e^{-tau_path}: from expm1 for small tau, from 1 - exp for
                 // large tau, so that both om and 1 - om keep FP32 relative precision
                 const float tf = tau_h + tau_l;
@@ -660,7 +666,7 @@ __global__ void __launch_bounds__(MAXB, 3) trace_mixed_kernel(const TraceArgs A)
                     break;
                 }
             } else if (stage == ST_LOCATE_DONE) {
-                C.c_loc[t] += nsteps;
+                if (count_add(C.c_loc[t], nsteps) && LONG) flush_counters();
                 float l0 = C.xl0[t], l1 = C.xl1[t], l2 = C.xl2[t];
                 const int fm = C.f_m[t];
                 have_pc = fm >= 0;
@@ -946,28 +952,34 @@ size_t trace_mixed_smem_bytes(int ninstr, int block)
     return align16(sizeof(InstrDev) * ninstr) + sizeof(Cold);
 }
 
-static cudaError_t set_smem_limit()
+namespace {
+
+using MixedKernel = void (*)(TraceArgs);
+
+MixedKernel mixed_kernel(int kind, bool long_counts)
 {
-    const int bytes = (int)trace_mixed_smem_bytes(16, MAXB);
-    cudaError_t e = cudaFuncSetAttribute(trace_mixed_kernel<G_CART>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(trace_mixed_kernel<G_CART_BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(trace_mixed_kernel<G_OCT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (kind == G_OCT) return long_counts ? trace_mixed_kernel<G_OCT, true> : trace_mixed_kernel<G_OCT, false>;
+    if (kind == G_CART) return long_counts ? trace_mixed_kernel<G_CART, true> : trace_mixed_kernel<G_CART, false>;
+    return long_counts ? trace_mixed_kernel<G_CART_BIG, true> : trace_mixed_kernel<G_CART_BIG, false>;
 }
+
+cudaError_t set_smem_limit(MixedKernel k)
+{
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trace_mixed_smem_bytes(16, MAXB));
+}
+
+}  // namespace
 
 cudaError_t launch_trace_mixed(const TraceArgs& a, int block, int grid, cudaStream_t s)
 {
     if (block > MAXB || block % 32) return cudaErrorInvalidValue;
-    cudaError_t e = set_smem_limit();
+    const int kind = a.oct_levels > 0 ? G_OCT
+                                      : (a.nx < (1 << 23) && a.ny < (1 << 23) && a.nz < (1 << 23) ? G_CART : G_CART_BIG);
+    const unsigned long long line = (unsigned long long)a.nx + a.ny + a.nz + 8;  // (of an octree: its crossing bound)
+    const MixedKernel k = mixed_kernel(kind, counts_within_packet(a.max_events, a.ninstr, line));
+    cudaError_t e = set_smem_limit(k);
     if (e != cudaSuccess) return e;
-    const size_t smem = trace_mixed_smem_bytes(a.ninstr, block);
-    if (a.oct_levels > 0)
-        trace_mixed_kernel<G_OCT><<<grid, block, smem, s>>>(a);
-    else if (a.nx < (1 << 23) && a.ny < (1 << 23) && a.nz < (1 << 23))
-        trace_mixed_kernel<G_CART><<<grid, block, smem, s>>>(a);
-    else
-        trace_mixed_kernel<G_CART_BIG><<<grid, block, smem, s>>>(a);
+    k<<<grid, block, trace_mixed_smem_bytes(a.ninstr, block), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -977,11 +989,10 @@ cudaError_t trace_mixed_occupancy(int block, int* blocks_per_sm, bool octree)
         *blocks_per_sm = 0;
         return cudaSuccess;
     }
-    cudaError_t e = set_smem_limit();
+    const MixedKernel k = mixed_kernel(octree ? G_OCT : G_CART, false);
+    cudaError_t e = set_smem_limit(k);
     if (e != cudaSuccess) return e;
-    const size_t smem = trace_mixed_smem_bytes(16, block);
-    return octree ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_mixed_kernel<G_OCT>, block, smem)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, trace_mixed_kernel<G_CART>, block, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, trace_mixed_smem_bytes(16, block));
 }
 
 }  // namespace skirt
