@@ -359,9 +359,10 @@ __device__ __forceinline__ double fixed58_to_double(unsigned long long sum, unsi
 constexpr int BR_WARPS = 4;    // warps per block
 constexpr int BR_STAGES = 2;   // stages of a warp's ring
 constexpr int BR_MAXW = 16;
-// The band starts as a call uploads them: NB + 1 starts, then a zero that a kernel
-// sets when a row copy did not arrive in time.
-constexpr int BAND_INTS = NB + 2;
+// The band starts as a call uploads them: NB + 1 starts, then two zeros that a kernel
+// sets when a copy did not arrive in time: of a row (band compression), of a tile's
+// features (inference).
+constexpr int BAND_INTS = NB + 3;
 
 // a stage holds about 3 KB, or two rows of the widest table
 constexpr size_t BR_SMEM_MAX = 128 + (size_t)BR_WARPS * BR_STAGES * 2 * BR_MAXW * NB * sizeof(double);
@@ -1165,7 +1166,7 @@ std::vector<int> band_starts(const double* lam, int n)
             if (idx[j] >= b) { s = j; break; }
         start[b] = b == NB ? n : s;
     }
-    start.push_back(0);
+    start.resize(BAND_INTS, 0);
     return start;
 }
 
@@ -1329,7 +1330,7 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
     ECK(cudaMemcpyAsync(d_w, w.data(), sizeof(double) * w.size(), cudaMemcpyHostToDevice, s));
     cudaEvent_t ev[4];
     for (auto& e : ev) ECK(cudaEventCreate(&e));
-    int rc = SKIRT_OK, timeout = 0;
+    int rc = SKIRT_OK, timeout[2] = {0, 0};
     unsigned long long nfb = 0;
     if (mode == SKIRT_EMIT_EXACT) {
         ECK(cudaEventRecord(ev[0], s));
@@ -1369,13 +1370,13 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
         ECK(cudaEventRecord(ev[0], s));
         ECK(launch_band_features(absorbed, ncell, n_in, start, d_start, mass, d_feat, d_tot, s));
         ECK(cudaEventRecord(ev[1], s));
-        rc = mlp_forward_internal(net, d_feat, d_tot, ncell, emission, d_flag, s);
+        rc = mlp_forward_internal(net, d_feat, d_tot, ncell, emission, d_flag, d_start + NB + 2, s);
         if (rc == SKIRT_OK) {
             compact_flags_kernel<<<grid_blocks(ncell, 256), 256, 0, s>>>(d_flag, ncell, d_rows, d_cnt);
             ECK(cudaGetLastError());
             ECK(cudaEventRecord(ev[2], s));
             ECK(cudaMemcpyAsync(&nfb, d_cnt, sizeof nfb, cudaMemcpyDeviceToHost, s));
-            ECK(cudaMemcpyAsync(&timeout, d_start + NB + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+            ECK(cudaMemcpyAsync(timeout, d_start + NB + 1, sizeof timeout, cudaMemcpyDeviceToHost, s));
             ECK(cudaStreamSynchronize(s));
             rc = launch_exact_emission(absorbed, n_in, d_w, mass, d_rows, (long long)nfb, emission, temperature, s);
             ECK(cudaEventRecord(ev[3], s));
@@ -1383,8 +1384,8 @@ extern "C" int skirt_dust_emission(const double* absorbed, long long ncell, int 
     }
     cudaFreeAsync(d_w, s);
     ECK(cudaStreamSynchronize(s));
-    if (rc == SKIRT_OK && mode == SKIRT_EMIT_SURROGATE) rc = mlp_check_timeout();
-    if (rc == SKIRT_OK && mode == SKIRT_EMIT_SURROGATE) rc = band_check_timeout(timeout);
+    if (rc == SKIRT_OK) rc = mlp_check_timeout(timeout[1]);
+    if (rc == SKIRT_OK) rc = band_check_timeout(timeout[0]);
     if (stats && rc == SKIRT_OK) {
         stats->n_cells = (unsigned long long)ncell;
         stats->n_fallback = nfb;

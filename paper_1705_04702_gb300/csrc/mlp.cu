@@ -81,9 +81,6 @@ static_assert(SM_TOTAL <= 227 * 1024, "shared memory of one block");
 static_assert((KP1 * 2) % 16 == 0 && (KP2 * 2) % 16 == 0 && SM_ST % 16 == 0 && SM_A % 16 == 0 && SM_BAR % 8 == 0,
               "padded rows and parts keep 16-byte alignment");
 
-// a wait for a bulk copy that runs out sets it, and the kernel stops
-__device__ unsigned g_mlp_timeout;
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -193,7 +190,7 @@ __device__ __forceinline__ void zero_rows(double* emission, long long r, int cou
 __global__ void __launch_bounds__(32 * INF_WARPS, 1) mlp_infer_kernel(
     const uint16_t* __restrict__ Wg, const float* __restrict__ Bg, const float* __restrict__ stats,
     const float* __restrict__ features, const double* __restrict__ total, long long n,
-    double* __restrict__ emission, unsigned char* __restrict__ flags, float inv_share_max)
+    double* __restrict__ emission, unsigned char* __restrict__ flags, float inv_share_max, int* timeout)
 {
     extern __shared__ __align__(128) unsigned char sm[];
     // stage the weights (bf16, contiguous W1 W2 W3) and biases / statistics
@@ -249,7 +246,8 @@ __global__ void __launch_bounds__(32 * INF_WARPS, 1) mlp_infer_kernel(
         const int rows = n - base < INF_TILE ? (int)(n - base) : INF_TILE;
         const double tot = lane < rows ? __ldcs(total + base + lane) : 0.0;  // of row `lane`
         if (!__all_sync(0xffffffffu, mbar_wait(bar, parity))) {
-            atomicOr(&g_mlp_timeout, 1u);
+            atomicOr(timeout, 1);
+            mbar_wait(bar, parity);  // the copy lands in this block's memory: give it its time
             break;
         }
         // ---- lane = row: the row's features in 8 groups of four, in an order rotated
@@ -623,8 +621,11 @@ int mlp_workspace(skirt_mlp_s* net, size_t bytes, void** p)
     return SKIRT_OK;
 }
 
+// timeout: a zero in device memory that belongs to the call (concurrent calls must
+// not clear or see each other's); a wait for a bulk copy that runs out sets it, and
+// mlp_check_timeout reports what the call read back from it
 int mlp_forward_internal(skirt_mlp_s* net, const float* features, const double* total, long long n, double* emission,
-                         unsigned char* flags, cudaStream_t s)
+                         unsigned char* flags, int* timeout, cudaStream_t s)
 {
     if ((reinterpret_cast<uintptr_t>(features) & 15) != 0)
         return set_error(SKIRT_ERR_INVALID_ARG, "features must be 16-byte aligned");
@@ -632,8 +633,6 @@ int mlp_forward_internal(skirt_mlp_s* net, const float* features, const double* 
         int r = repack(net, s);
         if (r) return r;
     }
-    const unsigned zero = 0;
-    MCK(cudaMemcpyToSymbolAsync(g_mlp_timeout, &zero, sizeof zero, 0, cudaMemcpyHostToDevice, s));
     MCK(cudaFuncSetAttribute(mlp_infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL));
     int sms = 0, dev = 0, per_sm = 0;
     MCK(cudaGetDevice(&dev));
@@ -645,17 +644,14 @@ int mlp_forward_internal(skirt_mlp_s* net, const float* features, const double* 
     if (grid < 1) grid = 1;
     const float inv_share_max = net->share_max > 0.f ? 1.f / net->share_max : 3.0e38f;
     mlp_infer_kernel<<<(int)grid, 32 * INF_WARPS, SM_TOTAL, s>>>(net->Wb, net->Bb, net->stats, features, total, n,
-                                                                  emission, flags, inv_share_max);
+                                                                  emission, flags, inv_share_max, timeout);
     MCK(cudaGetLastError());
     return SKIRT_OK;
 }
 
-int mlp_check_timeout()
+int mlp_check_timeout(int v)
 {
-    unsigned v = 0;
-    MCK(cudaMemcpyFromSymbol(&v, g_mlp_timeout, sizeof v));
-    if (v) return set_error(SKIRT_ERR_CUDA, "surrogate inference: a feature copy did not complete in time");
-    return SKIRT_OK;
+    return v ? set_error(SKIRT_ERR_CUDA, "surrogate inference: a feature copy did not complete in time") : SKIRT_OK;
 }
 
 }  // namespace skirt
@@ -1039,8 +1035,16 @@ extern "C" int skirt_mlp_forward(skirt_mlp_t net, const float* features, const d
     if (!net || !features || !total || !emission || n < 0) return set_error(SKIRT_ERR_INVALID_ARG, "mlp forward args");
     if (n == 0) return SKIRT_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    int r = mlp_forward_internal(net, features, total, n, emission, flags, s);
+    int* d_timeout = nullptr;
+    int timeout = 0;
+    MCK(cudaMallocAsync((void**)&d_timeout, sizeof(int), s));
+    cudaError_t e = cudaMemsetAsync(d_timeout, 0, sizeof(int), s);
+    const int r = e == cudaSuccess ? mlp_forward_internal(net, features, total, n, emission, flags, d_timeout, s) : SKIRT_OK;
+    if (e == cudaSuccess && r == SKIRT_OK)
+        e = cudaMemcpyAsync(&timeout, d_timeout, sizeof(int), cudaMemcpyDeviceToHost, s);
+    cudaFreeAsync(d_timeout, s);
     if (r) return r;
+    MCK(e);
     MCK(cudaStreamSynchronize(s));
-    return mlp_check_timeout();
+    return mlp_check_timeout(timeout);
 }

@@ -270,10 +270,10 @@ struct skirt_mlp_s;
 namespace skirt {
 // mlp.cu: tensor-core inference of the emission surrogate (stream-ordered, no sync)
 int mlp_forward_internal(skirt_mlp_s* net, const float* features, const double* total, long long n,
-                         double* emission, unsigned char* flags, cudaStream_t s);
-// after the stream has synchronised: INVALID (CUDA) when an inference launch
-// gave up waiting for a feature copy
-int mlp_check_timeout();
+                         double* emission, unsigned char* flags, int* timeout, cudaStream_t s);
+// after the stream has synchronised, with what `timeout` then holds: an error
+// when the call gave up waiting for a feature copy
+int mlp_check_timeout(int v);
 // the network's working tables for skirt_dust_emission (at least `bytes`,
 // 256-byte aligned); the caller holds mlp_workspace_mutex(net) while it uses them
 std::mutex& mlp_workspace_mutex(skirt_mlp_s* net);
