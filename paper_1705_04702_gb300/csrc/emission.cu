@@ -561,6 +561,8 @@ int band_blocks(long long ncell)
 constexpr int NS = NPOP * NOUT;
 constexpr int EX_SLOTS = (NS + 31) / 32;
 constexpr int EX_WARPS = 4;   // warps per block
+constexpr int EX_BLOCKS = 7;  // blocks per SM (the registers' bound)
+constexpr int EX_SPREAD = 24; // warps per SM that short row lists are spread over
 constexpr int EX_BATCH = 10;  // most rows per warp batch: lanes 3r + i, r < 10
 constexpr float Z_CUT = 70.f * (float)DF_Z_PER_X;
 
@@ -914,7 +916,7 @@ __device__ __noinline__ void block_powers_fp64(const double* __restrict__ row, i
 // shares as fill_shares lays them out (16-byte aligned).  A
 // second absorbed table A2 [ncell][n2] with its shares w2 (may be NULL) adds its
 // power to each population's.
-__global__ void __launch_bounds__(32 * EX_WARPS, 7) exact_kernel(
+__global__ void __launch_bounds__(32 * EX_WARPS, EX_BLOCKS) exact_kernel(
     const double* __restrict__ A, int n_in, const double* __restrict__ w, const double* __restrict__ A2, int n2,
     const double* __restrict__ w2, const float* __restrict__ mass, const unsigned* __restrict__ rows, long long nrows,
     double* __restrict__ emission, float* __restrict__ temperature, int stride, int batch)
@@ -1248,13 +1250,18 @@ int launch_exact_emission(const double* absorbed, int n_in, const double* w_dev,
         if (v >= 1 && v <= 64 && (v & (v - 1)) == 0) stride = v;
     }
     if (nrows > 0) {
-        // full batches once there are enough rows for them to fill the warps the
-        // device holds (152 SMs x 24); below that as many warps as rows allow, each
-        // with fewer rows in series (2000 rows: 115 us by tens, 28 us one by one)
-        const long long warps = 152LL * 24;
+        // full batches once there are enough rows for them to fill 24 warps per SM;
+        // below that as many warps as rows allow, each with fewer rows in series (2000
+        // rows: 115 us by tens, 28 us one by one).  24 of the 28 warps an SM holds: 4256
+        // rows take 37 us on 2128 warps and 41 on 4256, 12,000 55 by fours and 59 by
+        // threes.
+        int dev = 0, sms = 0;
+        ECK(cudaGetDevice(&dev));
+        ECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const long long warps = (long long)sms * EX_SPREAD;
         const int batch = (int)std::min<long long>(EX_BATCH, (nrows + warps - 1) / warps);
         long long blocks = (nrows + EX_WARPS * batch - 1) / (EX_WARPS * batch);
-        if (blocks > 152LL * 32) blocks = 152LL * 32;
+        if (blocks > sms * 32LL) blocks = sms * 32LL;
         exact_kernel<<<(int)blocks, 32 * EX_WARPS, 0, s>>>(absorbed, n_in, w_dev, absorbed2, n2, w2_dev, mass, rows,
                                                            nrows, emission, temperature, stride, batch);
     }
