@@ -249,7 +249,15 @@ extern "C" int skirt_grid_create(skirt_grid_t* out, int nx, int ny, int nz, cons
     // of the density and of the absorbed table.  The 256^3 disk (z cells an eighth
     // of the x cells: four crossings in five along z): 158 ms instead of 171 for
     // 1e7 packets, L1 hits 36% instead of 17%, DRAM traffic 42 GB instead of 61 per
-    // 2e6 packets; cubic cells gain nothing, which sets the line.
+    // 2e6 packets.  Where the line lies: whole calls of 2e6 packets on 256^3 cells,
+    // the transposes included, with this order against x fastest, at thin cells of
+    // 1/8, 1/2, 3/4, 9/10 and 1 of the x cells (1, 3 and 20 wavelengths on the disk):
+    // 7, 5, 4, 3 and 3% faster, 11, 8, 6, 5 and 4%, 25, 11, 5, 2 and 1%; 4 wavelengths,
+    // the least favourable to the transpose, 9, 5, 3, 1.5 and 1%; uniform dust 19, 9, 3,
+    // 0.6 and -0.8% (1 wavelength).  Shorter runs, at 1/8, 1/2 and 3/4: 200,000 packets
+    // 4, 2 and 1% (1 wavelength) and 4, 1 and -2% (4), 400,000 29, 5 and 0% (20).  Where
+    // density and tables fit the L2 (64^3 to 192^3 cells, 1e6 packets, 1 to 10
+    // wavelengths) either order serves: +2.6 to -1.7%.
     const double d[3] = {(bbox[1] - bbox[0]) / nx, (bbox[3] - bbox[2]) / ny, (bbox[5] - bbox[4]) / nz};
     const int f = d[1] < d[2] ? 1 : 2;
     if (d[f] <= 0.75 * d[0]) {
