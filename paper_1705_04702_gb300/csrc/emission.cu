@@ -552,12 +552,12 @@ int band_blocks(long long ncell)
 // diagnostic, or a rare target) continues Newton over the whole warp, and its
 // row is evaluated and written again.
 //
-// What bounds it is instruction issue (80%): 2480 warp instructions per row, of
-// which the powers take 660, the output 340 and the terms most of the rest, at
-// 72 registers and 28 warps per SM.  1e6 rows of 200 wavelengths take 2.7 ms
+// What bounds it is instruction issue (78%): 2530 warp instructions per row, of
+// which the powers take some 670, the output 340 and the terms most of the rest, at
+// 72 registers and 28 warps per SM.  1e6 rows of 200 wavelengths take 2.8 ms
 // (5.3 with FP64 power sums, a start table searched in ln G and Taylor-series
 // exponentials: FP64 pipe 62% busy, 4270 instructions per row), 2.1e6 rows of
-// 200 + 100 wavelengths 6.5 ms (12.5).
+// 200 + 100 wavelengths 6.6 ms (12.5).
 constexpr int NS = NPOP * NOUT;
 constexpr int EX_SLOTS = (NS + 31) / 32;
 constexpr int EX_WARPS = 4;   // warps per block

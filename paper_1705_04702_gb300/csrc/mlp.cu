@@ -296,9 +296,9 @@ __global__ void __launch_bounds__(32 * INF_WARPS, 1) mlp_infer_kernel(
         }
         __syncwarp();  // every lane is done with the feature tile
         if (lane == 0 && base + stride < n) fetch(base + stride);
-        // a 16-row tile none of whose rows absorbs power (empty space): its emission
-        // rows are zeros (the epilogue scales every row by its FP32 total), so its
-        // products are skipped
+        // a tile none of whose 32 rows absorbs power (empty space): its emission rows
+        // are zeros (the epilogue scales every row by its FP32 total), so its products
+        // are skipped; so is the last layer of a half of the tile
         const float ftot = (float)tot;
         const unsigned live = __ballot_sync(0xffffffffu, ftot != 0.f);
         if (live == 0u) {

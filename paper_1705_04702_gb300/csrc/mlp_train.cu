@@ -26,7 +26,7 @@
 // step, and the loss.
 //
 // A step is a chain of latencies on less than half of the SMs (a batch of 2048
-// rows has 64 tiles): 16.6 us, of which the weights' copy takes 1.0, the layers
+// rows has 64 tiles): 16.8 us, of which the weights' copy takes 1.0, the layers
 // and the softmax 4.6, the way back 2.1, the weight gradients and their stores
 // about 2.5, the hand-over to the sum 2.2 and the sum 1.5 (35 us with 8 warps
 // that staged the weights and divided 64-bit row numbers in every thread, and

@@ -12,7 +12,7 @@
 // exit face, through the precomputed face neighbour and a descent by the
 // lattice cell of the entry point).
 //
-// What bounds it is the FP64 pipe (85% active in a long run): a warp instruction
+// What bounds it is the FP64 pipe (83% active): a warp instruction
 // holds it for some 20 cycles of the SM, whatever its active lanes.  So the lanes
 // of a warp step together, peel-offs in some rounds and deposits and searches in
 // others (a deposit crossing costs three times a peel-off's FP64 instructions),
@@ -22,9 +22,9 @@
 // saved start of the deposit traversal it repeats, and the deposits of a path take
 // e^{-tau} once per round of crossings and carry what each cell leaves of it in
 // between.  A peel-off crossing is 5 or 6 FP64 instructions, a deposit crossing
-// 17 in thin cells.  3e5 packets of 3 wavelengths on a 97^3 disk take 39 ms (132
-// with one state machine per lane, every crossing 12 FP64 instructions and two
-// exponentials more per deposit, at 5 of 32 lanes).
+// 18 in thin cells.  3e5 packets of 3 wavelengths on a 97^3 disk take 37 ms, 36 to
+// 39 by their seed (132 with one state machine per lane, every crossing 12 FP64
+// instructions and two exponentials more per deposit, at 5 of 32 lanes).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -39,7 +39,8 @@ namespace {
 
 // Lanes of one kind stepping below which a warp handles its idle lanes' events, and
 // crossings between warp votes (and between evaluations of e^{-tau}).  The case
-// named above with 8 / 24: 39 ms; 16 / 16: 48, 8 / 16: 43, 8 / 32: 43, 12 / 16: 46.
+// named above with 8 / 24: 39 ms; 8 / 16: 43, 16 / 16: 48, 8 / 32: 43, 12 / 16: 46
+// (deposits as they were before take(); with it 8 / 24: 39.1, 8 / 16: 43.2).
 constexpr int FP64_STEP_MIN = 8;
 constexpr int FP64_ROUND = 24;
 constexpr int FP64_MAXB = 512;     // threads per block (upper bound)
